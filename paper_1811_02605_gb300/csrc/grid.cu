@@ -329,6 +329,9 @@ mhd_status_t create_grid(const mhd_grid_desc_t* desc, int i0, int i1, bool as_sl
     g->slab_nr_global = slab ? dg.nr : 0;
     ok = ok && dalloc(&g->partials, (size_t)kMaxBlocks * kPartialsPerBlock + 16, owned) &&
          dalloc(&g->sc, 1, owned) && dalloc(&g->ss, 1, owned);
+    unsigned char* pbuf = nullptr;
+    ok = ok && dalloc(&pbuf, persist_buf_bytes(), owned);
+    g->persist_buf = pbuf;
     if (!ok) {
         for (void* m : owned) cudaFree(m);
         if (g->side) cudaStreamDestroy(g->side);

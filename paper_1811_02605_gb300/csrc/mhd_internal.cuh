@@ -266,6 +266,7 @@ struct mhd_grid_s {
     double* partials;       // [kMaxBlocks * kPartialsPerBlock]
     void* adj_mem;          // adjoint workspace, allocated by the first adjoint call
     void* res_mem;          // implicit-resistivity workspace, allocated by the first such step
+    void* persist_buf;      // slots of the persistent PCG kernel's exchanges (persist.cu)
     void* pc2_mem;          // PC2 workspace (1 / dt of the phi-line ILU(0)), allocated by the first PC2 solve
     mhd::PcgScalars* sc;    // device
     mhd::StepScalars* ss;   // device
@@ -279,9 +280,10 @@ struct mhd_grid_s {
     int slab32;             // FP32 CG kernels: r-slab length of the tiled pair (> 0), split kernels (-1),
                             // p update folded into the stencil (-2), recompute pair (-3, -4 with the
                             // r update walking backwards), bulk-staged pair with units of L planes
-                            // (-100 - L); 0: not tuned
+                            // (-100 - L), whole inner solve in one persistent launch (-9); 0: not tuned
     int slab64;             // same for the FP64 fused p-update + stencil kernel; -2: the split kernels
-                            // with each component's p update overlapping the previous component's stencil
+                            // with each component's p update overlapping the previous component's
+                            // stencil; -3: whole solve in one persistent launch
     int pc2_fused32;        // FP32 PC2 iteration: p update folded into the stencil (1) or split (-1); 0: unset
     double visc_lambda_unit; // Gershgorin bound on the spectral radius of D^-1 K (nu = 1)
     std::string last_error;
@@ -365,6 +367,11 @@ void enqueue_tiled64_a(mhd_grid_s* g, cudaStream_t st, int slab, int prof_id);
 // FP32 CG iteration as a bulk-copy-staged plane-marching pair (bulk.cu); slab: planes per work unit
 bool bulk32_ok(const mhd_grid_s* g);
 void enqueue_bulk32(mhd_grid_s* g, cudaStream_t st, int nc, int slab);
+
+// all iterations of a point-Jacobi solve in one cooperative launch (persist.cu)
+size_t persist_buf_bytes();
+int persist_mode(const mhd_grid_s* g, bool fp32, int nc);
+mhd_status_t persist_iterate(mhd_grid_s* g, bool fp32, int nc);
 
 // PCG (pcg.cu). alpha is read from device memory (alpha_dev) so a step never syncs on it.
 void build_tables(mhd_grid_s* g, const double* alpha_dev, bool fp32);

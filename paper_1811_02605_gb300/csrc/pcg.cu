@@ -8,7 +8,8 @@
 // That matters on this part: FP64 runs at 2 FMA/clk/SM, so the FP64 iteration is bound by its
 // FP64 instruction count, not by HBM.
 //
-// One iteration is three kernels: the p update (which also adds the previous iteration's alpha p
+// Systems whose vectors fit the chip's shared memory are solved by one persistent launch (persist.cu).
+// Otherwise one iteration is three kernels: the p update (which also adds the previous iteration's alpha p
 // to x: the x update is deferred by one kernel, so the update kernel need not read p or x), the
 // stencil with <p, q>, and the r update with the dot products and the stop test. In the FP32
 // inner solves the first two can run as one kernel with p double-buffered (chosen per grid by
@@ -1600,7 +1601,7 @@ __global__ void k_inner_end(PcgScalars* sc, const double* saved) {
 }  // namespace
 
 namespace {
-__global__ void k_tune_reset(PcgScalars* sc) {
+__global__ void k_tune_reset(PcgScalars* sc, int max_iter = 1 << 30) {
     sc->done = 0;
     sc->alpha = 0.0;
     sc->beta = 0.0;
@@ -1608,7 +1609,8 @@ __global__ void k_tune_reset(PcgScalars* sc) {
     sc->tol = 0.0;
     sc->bb = 1.0;
     sc->iter = 0;
-    sc->max_iter = 1 << 30;
+    sc->max_iter = max_iter;
+    sc->total_iter = 0;
     sc->par = 0;
     sc->ax = 0.0;
     sc->count = 0u;
@@ -1624,12 +1626,36 @@ int forced_slab() {
     return f ? (int)std::strtol(f, nullptr, 10) : 0;
 }
 
+// milliseconds per iteration of the persistent kernel over 8 iterations, one untimed launch before
+// (huge when it cannot run); the vectors hold the trial values
+float time_persist(mhd_grid_s* g, bool fp32, int nc, cudaEvent_t e0, cudaEvent_t e1) {
+    if (!persist_mode(g, fp32, nc)) return 1e30f;
+    for (int warm = 1; warm >= 0; warm--) {
+        k_tune_reset<<<1, 1, 0, g->stream>>>(g->sc, 8);
+        if (!warm) cudaEventRecord(e0, g->stream);
+        if (persist_iterate(g, fp32, nc) != MHD_OK) return 1e30f;
+        if (!warm) cudaEventRecord(e1, g->stream);
+    }
+    float ms = 0.f;
+    if (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) return 1e30f;
+    return ms / 8.f;
+}
+
 mhd_status_t tune_slab32(mhd_grid_s* g, int nc) {
     if (g->slab32 != 0) return MHD_OK;
     if (const int f = forced_slab()) {
         if (f <= -2 && f >= -8) g->slab32 = f;
+        else if (f == -9) g->slab32 = persist_mode(g, true, 3) ? f : -1;
         else if (f <= -100) g->slab32 = (bulk32_ok(g) && f < -100) ? f : -1;
         else g->slab32 = (f > 0 && tiled32_ok(g) && tiled32_blocks(g, f) <= kMaxBlocks) ? f : -1;
+        return MHD_OK;
+    }
+    // vectors that fit the CTAs' shared memory (736 thousand cells with np a multiple of 4): the persistent
+    // kernel, by rule. us per iteration, it against the best of the others: 32x32x64 10.0 / 17.4,
+    // 48x48x96 11.5 / 20.4, 64x64x128 14.5 / 26.3. Above that it is one of the timed candidates
+    // (96x96x192: 35.4 / 44.4; 128x128x256: 108 / 85.7).
+    if (persist_mode(g, true, nc) == 1) {
+        g->slab32 = -9;
         return MHD_OK;
     }
     cudaEvent_t e0, e1;
@@ -1688,11 +1714,14 @@ mhd_status_t tune_slab32(mhd_grid_s* g, int nc) {
             best = slab;
         }
     }
+    cudaMemsetAsync(g->r32, 0x3F, sizeof(float) * n3, g->stream);
+    cudaMemsetAsync(g->p32, 0x3F, sizeof(float) * 2 * n3, g->stream);
+    if (3.f * time_persist(g, true, nc, e0, e1) < best_ms) best = -9;
     g->prof = prof;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (best == 0) return set_error(g, MHD_ERR_CUDA, "FP32 CG kernels: no launchable variant");
-    g->slab32 = best;  // -1 split, -2 folded, -3/-4 recompute pair, <= -100 bulk-staged pair, > 0 tiled slab
+    g->slab32 = best;  // -1 split, -2 folded, -3/-4 recompute pair, -9 persistent, <= -100 bulk-staged pair, > 0 tiled slab
     return check_cuda(g, "tune slab");
 }
 }  // namespace
@@ -1703,7 +1732,16 @@ namespace {
 mhd_status_t tune_slab64(mhd_grid_s* g) {
     if (g->slab64 != 0) return MHD_OK;
     if (const int f = forced_slab()) {
-        g->slab64 = (f > 0 && tiled32_ok(g) && tiled32_blocks(g, f) <= kMaxBlocks) ? f : (f == -64 ? -2 : -1);
+        if (f == -65) g->slab64 = persist_mode(g, false, 3) ? -3 : -1;
+        else g->slab64 = (f > 0 && tiled32_ok(g) && tiled32_blocks(g, f) <= kMaxBlocks) ? f : (f == -64 ? -2 : -1);
+        return MHD_OK;
+    }
+    // vectors that fit the CTAs' shared memory (368 thousand cells): the persistent kernel, by rule. us per
+    // iteration, it against the split kernels: 32x32x64 13.5 / 20.0, 48x48x96 23.5 / 32.7,
+    // 61x47x118 30.7 / 43.1. Above that it is one of the timed candidates (64x64x128: 42.7 / 54.3;
+    // 96x96x192: 137.7 / 140.8; 160x160x320: 615 / 560).
+    if (persist_mode(g, false, 3) == 1) {
+        g->slab64 = -3;
         return MHD_OK;
     }
     cudaEvent_t e0, e1;
@@ -1733,6 +1771,9 @@ mhd_status_t tune_slab64(mhd_grid_s* g) {
             best = slab;
         }
     }
+    cudaMemsetAsync(g->r64, 0x3F, sizeof(double) * n3, g->stream);
+    cudaMemsetAsync(g->p64, 0x3F, sizeof(double) * 2 * n3, g->stream);
+    if (2.f * time_persist(g, false, 3, e0, e1) < best_ms) best = -3;
     g->prof = prof;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -1756,11 +1797,11 @@ mhd_status_t solver_reserve(mhd_grid_s* g, int features) {
     cudaGraphExec_t ge = nullptr;
     if (features & MHD_RESERVE_PC1) {
         if (g->slab64 == 0 && (st = tune_slab64(g)) != MHD_OK) return st;
-        if ((st = iteration_graph(g, 0, 3, &ge)) != MHD_OK) return st;
+        if (g->slab64 != -3 && (st = iteration_graph(g, 0, 3, &ge)) != MHD_OK) return st;
     }
     if (features & MHD_RESERVE_MIXED) {
         if (g->slab32 == 0 && (st = tune_slab32(g, 3)) != MHD_OK) return st;
-        if ((st = iteration_graph(g, 1, 3, &ge)) != MHD_OK) return st;
+        if (g->slab32 != -9 && (st = iteration_graph(g, 1, 3, &ge)) != MHD_OK) return st;
     }
     if (features & MHD_RESERVE_CG) {
         if ((st = iteration_graph(g, 2, 3, &ge)) != MHD_OK) return st;
@@ -1802,7 +1843,8 @@ mhd_status_t solve(mhd_grid_s* g, const double* alpha_dev, int nc, const double*
             if ((st = pc2_factor(g)) != MHD_OK) return st;
             pc2_init64(g, nc);
         }
-        st = run_iterations(g, pc2 ? 3 : (prm->pcg_variant == 1 ? 2 : 0), nc);
+        if (!pc2 && prm->pcg_variant == 0 && g->slab64 == -3) st = persist_iterate(g, false, nc);
+        else st = run_iterations(g, pc2 ? 3 : (prm->pcg_variant == 1 ? 2 : 0), nc);
         if (st != MHD_OK) return st;
         k_finish64<<<blocks2, kThreads, 0, g->stream>>>(d, nc, g->x64, g->p64, x, g->t64.s, g->sc);
         if ((st = check_cuda(g, "pcg finish")) != MHD_OK) return st;
@@ -1814,6 +1856,7 @@ mhd_status_t solve(mhd_grid_s* g, const double* alpha_dev, int nc, const double*
         if (h.done == 1) return MHD_OK;
         if (h.done == 3) return set_error(g, MHD_ERR_NONFINITE, "pcg: non-finite value in a reduction");
         if (h.done == 4) return set_error(g, MHD_ERR_NOCONV, "pcg: breakdown (operator not positive definite)");
+        if (h.done == 6) return set_error(g, MHD_ERR_TIMEOUT, "pcg: a bounded wait of the persistent kernel gave up");
         return set_error(g, MHD_ERR_NOCONV, "pcg: no convergence within max_iter");
     }
     // mixed precision: x starts as x0 in FP64 (in place in the caller's x)
@@ -1842,11 +1885,16 @@ mhd_status_t solve(mhd_grid_s* g, const double* alpha_dev, int nc, const double*
         outer_done = g->h_sc->outer_done;
         if (outer_done || o == prm->max_outer) break;
         k_inner_begin<<<1, 1, 0, g->stream>>>(g->sc, saved);
-        st = run_iterations(g, pc2 ? 4 : 1, nc);
+        if (!pc2 && g->slab32 == -9) {
+            st = persist_iterate(g, true, nc);
+            if (st == MHD_OK) st = read_scalars(g);
+        } else {
+            st = run_iterations(g, pc2 ? 4 : 1, nc);
+        }
         if (st != MHD_OK) return st;
         k_inner_end<<<1, 1, 0, g->stream>>>(g->sc, saved);
         if (g->h_sc->done == 6)
-            return set_error(g, MHD_ERR_TIMEOUT, "pcg (mixed): a bounded wait for a bulk copy gave up");
+            return set_error(g, MHD_ERR_TIMEOUT, "pcg (mixed): a bounded device-side wait gave up");
         if (g->h_sc->done == 3) break;
         k_correct<<<blocks2, kThreads, 0, g->stream>>>(d, nc, x, g->x32, g->p32, g->t64.s, g->sc);
         if ((st = check_cuda(g, "correction")) != MHD_OK) return st;
