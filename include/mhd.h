@@ -127,7 +127,7 @@ enum { MHD_PREC_FP64 = 0, MHD_PREC_MIXED = 1 };
  * the second kernel walking the grid backwards, -5 recompute pair at 6 CTAs per SM, -6 / -7 / -8
  * single-reduction pair (-7: its residual kernel unrolled over the components, both kernels at 3
  * CTAs per SM; -8: unrolled residual kernel, update kernel at 4), -9 whole inner solve in one
- * persistent launch, -64 the FP64 iteration with its components overlapped, -65 the whole FP64 solve
+ * persistent launch, -10 the single-reduction iteration as one marching kernel, -64 the FP64 iteration with its components overlapped, -65 the whole FP64 solve
  * in one persistent launch, n > 0 tiles of n planes). */
 typedef struct {
     double nu, eta, cfl, dt_fixed, dt_max, alpha_si_fixed;
@@ -339,7 +339,8 @@ enum {
     MHD_KERNEL_CGU32 = 17,   /* FP32 single-reduction pair: p, A p, r and x updates */
     MHD_KERNEL_PERSIST64 = 18, /* FP64 point-Jacobi PCG: all iterations of a solve in one launch */
     MHD_KERNEL_PERSIST32 = 19, /* FP32 inner PCG: all iterations of an inner solve in one launch */
-    MHD_KERNEL_COUNT = 20
+    MHD_KERNEL_MARCH32 = 20,   /* FP32 single-reduction iteration as one plane-marching kernel */
+    MHD_KERNEL_COUNT = 21
 };
 mhd_status_t mhd_profile_enable(mhd_grid_t grid, int enable);
 /* Total milliseconds and launch count of one kernel id since profiling was enabled.
@@ -348,8 +349,8 @@ mhd_status_t mhd_profile_read(mhd_grid_t grid, int kernel, double* total_ms, lon
 /* The kernel forms the grid's autotuner chose, in the codes of MHD_FORCE_SLAB: *fp64_form for the
  * FP64 iteration (-1 split, -2 components overlapped, -3 whole solve in one persistent launch, n > 0
  * tiles of n planes) and *fp32_form for the FP32 inner iteration (-1 split, -2 folded, -3/-4/-5
- * recompute pair, -6/-7/-8 single-reduction pair, -9 whole inner solve in one persistent launch,
- * <= -100 bulk-staged pair, n > 0 tiles); 0 where that precision has not been tuned yet.
+ * recompute pair, -6/-7/-8 single-reduction pair, -9 whole inner solve in one persistent launch, -10
+ * single-reduction iteration as one marching kernel, <= -100 bulk-staged pair, n > 0 tiles); 0 where that precision has not been tuned yet.
  * Either pointer may be NULL. */
 mhd_status_t mhd_grid_kernel_forms(mhd_grid_t grid, int* fp64_form, int* fp32_form);
 

@@ -29,7 +29,7 @@
 namespace mhd {
 // kernels of pcg.cu launched from here (host stubs resolve across translation units)
 __global__ void k_tables(Dims d, Geo G, const double* __restrict__ alpha_p, OpTab<double> t, OpTab<float> t32,
-                         OpTab64u tu, int want32);
+                         OpTab64u tu, int want32, float4* row32);
 __global__ void k_init64(Dims d, int nc, const double* __restrict__ b, const double* __restrict__ x0,
                          double* __restrict__ xs, double* __restrict__ r, double* __restrict__ p, OpTab<double> t,
                          OpTab64u tu, PcgScalars* sc, double* __restrict__ partials);
@@ -430,7 +430,7 @@ void enqueue_batch(Plan& P, cudaStream_t st, bool finish, int max_iter_override)
     for (int s = 0; s < P.n; s++) {
         mhd_grid_s* g = P.grids[s];
         const int nij = g->d.nr * g->d.nt;
-        k_tables<<<(nij + 255) / 256, 256, 0, st>>>(g->d, g->geo, P.d_alpha + s, g->t64, g->t32, g->tu, 0);
+        k_tables<<<(nij + 255) / 256, 256, 0, st>>>(g->d, g->geo, P.d_alpha + s, g->t64, g->t32, g->tu, 0, nullptr);
     }
     // per-system scalar set-up (scalar pointers kept in the spare tail of d_part's neighbour)
     PcgScalars** scs = reinterpret_cast<PcgScalars**>(P.d_sys + P.n);

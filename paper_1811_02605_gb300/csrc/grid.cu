@@ -316,7 +316,7 @@ mhd_status_t create_grid(const mhd_grid_desc_t* desc, int i0, int i1, bool as_sl
     ok = ok && dalloc(&g->x64, n3, owned) && dalloc(&g->r64, n3, owned) && dalloc(&g->p64, 2 * n3, owned) &&
          dalloc(&g->q64, n3, owned);
     ok = ok && dalloc(&g->x32, n3, owned) && dalloc(&g->r32, n3, owned) && dalloc(&g->p32, 2 * n3, owned) &&
-         dalloc(&g->q32, n3, owned);
+         dalloc(&g->q32, n3, owned) && dalloc(&g->row32, 8 * (size_t)nr * nt, owned);
     ok = ok && dalloc(&g->b0, n3, owned) && dalloc(&g->b1, n3, owned) && dalloc(&g->dlt, n3, owned);
     ok = ok && dalloc(&g->er, (size_t)nr * (nt + 1) * d.np, owned) &&
          dalloc(&g->et, (size_t)(nr + 1) * nt * d.np, owned) &&

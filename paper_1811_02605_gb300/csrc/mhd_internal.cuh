@@ -42,6 +42,30 @@ struct PcgScalars {
     double wp;       // FP32 single-reduction pair: <r~, A~ p~_old> summed by the update kernel
 };
 
+// FP32 single-reduction iteration, end of its reduction over the new residual: the stop test, then beta and
+// alpha of the next update. gam = <r~, r~>, del = <r~, A~ r~>, rr = sum dg r~^2; sc->wp = <r~, A~ p~_old> and
+// sc->pq, the previous denominator, give <p~, A~ p~> without another reduction.
+__device__ __forceinline__ void single_reduction_finish(PcgScalars* sc, double gam, double del, double rr) {
+    const double beta = (sc->iter == 0) ? sc->beta : gam / sc->rho;
+    const double wp = sc->wp;   // from the update kernel or the residual replacement
+    sc->rho_prev = sc->rho;
+    sc->rho = gam;
+    sc->rr = rr;
+    if (!isfinite(gam) || !isfinite(del) || !isfinite(rr)) sc->done = 3;
+    else if (sqrt(rr) <= sc->tol * sqrt(sc->bb)) sc->done = 1;
+    else if (sc->iter >= sc->max_iter) sc->done = 2;
+    else {
+        const double den = (beta == 0.0) ? del : del + beta * (2.0 * wp + beta * sc->pq);
+        if (!isfinite(den)) sc->done = 3;
+        else if (!(den > 0.0)) sc->done = 4;
+        else {
+            sc->beta = beta;
+            sc->pq = den;
+            sc->alpha = gam / den;
+        }
+    }
+}
+
 // Device-resident scalars of one step.
 struct StepScalars {
     double dt, cf, cw, alpha_si, alpha_nu;
@@ -251,6 +275,8 @@ struct mhd_grid_s {
     double *x64, *r64, *p64, *q64;
     // FP32 PCG workspace
     float *x32, *r32, *p32, *q32;
+    float* row32;           // [8*nr*nt] per (i, j): ar low, ar high, at low, at high, ap, the diagonal over a power of
+                            // two, unused, and that power's exponent (the marching kernel's rows)
     // step workspace
     double *b0, *b1, *dlt;
     double *er, *et, *ep;   // edge arrays (E or J)
@@ -280,7 +306,8 @@ struct mhd_grid_s {
     int slab32;             // FP32 CG kernels: r-slab length of the tiled pair (> 0), split kernels (-1),
                             // p update folded into the stencil (-2), recompute pair (-3, -4 with the
                             // r update walking backwards), bulk-staged pair with units of L planes
-                            // (-100 - L), whole inner solve in one persistent launch (-9); 0: not tuned
+                            // (-100 - L), whole inner solve in one persistent launch (-9), single-reduction
+                            // iteration as one marching kernel (-10); 0: not tuned
     int slab64;             // same for the FP64 fused p-update + stencil kernel; -2: the split kernels
                             // with each component's p update overlapping the previous component's
                             // stencil; -3: whole solve in one persistent launch
@@ -367,6 +394,10 @@ void enqueue_tiled64_a(mhd_grid_s* g, cudaStream_t st, int slab, int prof_id);
 // FP32 CG iteration as a bulk-copy-staged plane-marching pair (bulk.cu); slab: planes per work unit
 bool bulk32_ok(const mhd_grid_s* g);
 void enqueue_bulk32(mhd_grid_s* g, cudaStream_t st, int nc, int slab);
+
+// FP32 single-reduction iteration as one plane-marching kernel (march.cu)
+bool march32_ok(const mhd_grid_s* g);
+void enqueue_march32(mhd_grid_s* g, cudaStream_t st, int nc);
 
 // all iterations of a point-Jacobi solve in one cooperative launch (persist.cu)
 size_t persist_buf_bytes();

@@ -97,7 +97,7 @@ __device__ __forceinline__ double diag_at(const Geo& G, int nt, double a, int i,
 }
 
 __global__ void k_tables(Dims d, Geo G, const double* __restrict__ alpha_p, OpTab<double> t,
-                         OpTab<float> t32, OpTab64u tu, int want32) {
+                         OpTab<float> t32, OpTab64u tu, int want32, float4* row32) {
     const int nr = d.nr, nt = d.nt;
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= nr * nt) return;
@@ -125,6 +125,13 @@ __global__ void k_tables(Dims d, Geo G, const double* __restrict__ alpha_p, OpTa
         t32.ap[idx] = (float)ap;
         if (i == nr - 1) t32.ar[nr * nt + j] = 0.f;
         if (j == nt - 1) t32.at[i * (nt + 1) + nt] = 0.f;
+        // the marching kernel's rows: the coefficients and the diagonal over a power of two that keeps its
+        // products with r~^2 within r~^2's own range
+        const double ah = (i < nr - 1) ? a * G.wr[(i + 1) * nt + j] * (1.0 / sqrt(diag_at(G, nt, a, i + 1, j))) * s : 0.0;
+        const double th = (j < nt - 1) ? a * G.wt[i * (nt + 1) + j + 1] * (1.0 / sqrt(diag_at(G, nt, a, i, j + 1))) * s : 0.0;
+        const int e = ilogb(diag_at(G, nt, a, nr - 1, nt / 2));
+        row32[2 * idx] = make_float4((float)ar, (float)ah, (float)at, (float)th);
+        row32[2 * idx + 1] = make_float4((float)ap, (float)ldexp(dc, -e), 0.f, __int_as_float(e));
     }
 }
 
@@ -689,29 +696,6 @@ __device__ __forceinline__ void cgr_component(const Dims& d, const Cell& c, cons
 
 // UNR: the component loop unrolled (every component's loads can be in flight at once, at fewer
 // CTAs per SM: MINB)
-// last CTA of the residual kernel: the stop test, then beta and alpha for the next update
-__device__ __forceinline__ void cgr_finish(PcgScalars* sc, const double* out) {
-    const double gam = out[0], del = out[1], rr = out[2];
-    const double beta = (sc->iter == 0) ? sc->beta : gam / sc->rho;
-    const double wp = sc->wp;   // <r~, A~ p~_old>, from the update kernel or the replacement
-    sc->rho_prev = sc->rho;
-    sc->rho = gam;
-    sc->rr = rr;
-    if (!finite(gam) || !finite(del) || !finite(rr)) sc->done = 3;
-    else if (sqrt(rr) <= sc->tol * sqrt(sc->bb)) sc->done = 1;
-    else if (sc->iter >= sc->max_iter) sc->done = 2;
-    else {
-        const double den = (beta == 0.0) ? del : del + beta * (2.0 * wp + beta * sc->pq);
-        if (!finite(den)) sc->done = 3;
-        else if (!(den > 0.0)) sc->done = 4;
-        else {
-            sc->beta = beta;
-            sc->pq = den;
-            sc->alpha = gam / den;
-        }
-    }
-}
-
 template <int V, int NC, int MINB, bool UNR>
 __global__ void __launch_bounds__(kThreads, MINB) k_cgr32(Dims d, const float* __restrict__ ra,
                                                           const float* __restrict__ rb, OpTab<float> t,
@@ -754,7 +738,8 @@ __global__ void __launch_bounds__(kThreads, MINB) k_cgr32(Dims d, const float* _
         a_rr = fma(dg[c.ij], (double)cell, a_rr);
     }
     double val[3] = {a_g.get(), a_d.get(), a_rr}, out[3];
-    if (reduce_last<3>(val, partials, &sc->count, out) && threadIdx.x == 0) cgr_finish(sc, out);
+    if (reduce_last<3>(val, partials, &sc->count, out) && threadIdx.x == 0)
+        single_reduction_finish(sc, out[0], out[1], out[2]);
 }
 
 // U (k_cgu32): p~ = r~ + beta p~_old at the cell and its neighbours, q~ = A~ p~ at the cell,
@@ -1223,7 +1208,7 @@ __global__ void __launch_bounds__(kThreads) k_apply64(Dims d, int nc, const doub
 void build_tables(mhd_grid_s* g, const double* alpha_dev, bool fp32) {
     const int n = g->d.nr * g->d.nt;
     k_tables<<<(n + 255) / 256, 256, 0, g->stream>>>(g->d, g->geo, alpha_dev, g->t64, g->t32, g->tu,
-                                                      fp32 ? 1 : 0);
+                                                      fp32 ? 1 : 0, reinterpret_cast<float4*>(g->row32));
 }
 
 void apply_operator(mhd_grid_s* g, const double* alpha_dev, int nc, const double* p, double* q) {
@@ -1487,6 +1472,8 @@ void enqueue_iteration(mhd_grid_s* g, cudaStream_t st, int prec, int nc) {
     } else if (g->slab32 <= -100) {
         // plane-marching pair with bulk-copy staging, when the autotuner measured it fastest
         enqueue_bulk32(g, st, nc, -100 - g->slab32);
+    } else if (g->slab32 == -10) {
+        enqueue_march32(g, st, nc);
     } else if (g->slab32 <= -6 && g->slab32 >= -8) {
         // single-reduction pair (residual kernel, then the update), when measured fastest
         if (use_v4(g)) enqueue_cgpair32_nc<4>(g, st, nc);
@@ -1546,8 +1533,23 @@ mhd_status_t read_scalars(mhd_grid_s* g) {
     return MHD_OK;
 }
 
+// the residual kernel of the single-reduction pair, ahead of the marching iterations of an inner solve: the
+// scalars of the first update (the marching kernel forms those of the next one itself)
+template <int NC>
+void enqueue_first_residual(mhd_grid_s* g) {
+    const int s = prof_begin(g, g->stream, MHD_KERNEL_CGR32);
+    k_cgr32<4, NC, 3, true><<<grid_blocks(g, g->d.N / 4, resident_per_sm<k_cgr32<4, NC, 3, true>>()), kThreads, 0, g->stream>>>(
+        g->d, g->r32, g->q32, g->t32, g->tu.dg, g->sc, g->partials);
+    prof_end(g, g->stream, s);
+}
+
 // run batches of iterations until the device flags completion
 mhd_status_t run_iterations(mhd_grid_s* g, int prec, int nc) {
+    if (prec == 1 && g->slab32 == -10) {
+        if (nc == 3) enqueue_first_residual<3>(g);
+        else if (nc == 2) enqueue_first_residual<2>(g);
+        else enqueue_first_residual<1>(g);
+    }
     cudaGraphExec_t ge = nullptr;
     if (!g->prof) {
         mhd_status_t st = iteration_graph(g, prec, nc, &ge);
@@ -1626,6 +1628,11 @@ int forced_slab() {
     return f ? (int)std::strtol(f, nullptr, 10) : 0;
 }
 
+// cells up to which the persistent kernel is timed when its vectors do not fit shared memory (us per iteration,
+// it against the best other form: 1.0M cells FP64 77 / 88, FP32 21 / 30; 1.8M 138 / 141, 35 / 37; 4.2M 314 /
+// 301, 108 / 63)
+constexpr long long kPersistTrial = 2500000;
+
 // milliseconds per iteration of the persistent kernel over 8 iterations, one untimed launch before
 // (huge when it cannot run); the vectors hold the trial values
 float time_persist(mhd_grid_s* g, bool fp32, int nc, cudaEvent_t e0, cudaEvent_t e1) {
@@ -1645,6 +1652,7 @@ mhd_status_t tune_slab32(mhd_grid_s* g, int nc) {
     if (g->slab32 != 0) return MHD_OK;
     if (const int f = forced_slab()) {
         if (f <= -2 && f >= -8) g->slab32 = f;
+        else if (f == -10) g->slab32 = march32_ok(g) ? f : -1;
         else if (f == -9) g->slab32 = persist_mode(g, true, 3) ? f : -1;
         else if (f <= -100) g->slab32 = (bulk32_ok(g) && f < -100) ? f : -1;
         else g->slab32 = (f > 0 && tiled32_ok(g) && tiled32_blocks(g, f) <= kMaxBlocks) ? f : -1;
@@ -1652,8 +1660,7 @@ mhd_status_t tune_slab32(mhd_grid_s* g, int nc) {
     }
     // vectors that fit the CTAs' shared memory (736 thousand cells with np a multiple of 4): the persistent
     // kernel, by rule. us per iteration, it against the best of the others: 32x32x64 10.0 / 17.4,
-    // 48x48x96 11.5 / 20.4, 64x64x128 14.5 / 26.3. Above that it is one of the timed candidates
-    // (96x96x192: 35.4 / 44.4; 128x128x256: 108 / 85.7).
+    // 48x48x96 11.5 / 20.4, 64x64x128 14.5 / 26.3. Above that it is one of the timed candidates.
     if (persist_mode(g, true, nc) == 1) {
         g->slab32 = -9;
         return MHD_OK;
@@ -1675,7 +1682,11 @@ mhd_status_t tune_slab32(mhd_grid_s* g, int nc) {
     // -164: the recompute pair as plane-marching kernels staged by bulk copies (units of 32 or 64
     // planes). Four iterations each after one untimed: an even count, so each is timed with its
     // x updates.
-    for (int cand : {-1, -2, -3, -4, -5, -6, -7, -8, -132, -164}) {
+    // Where the marching kernel (-10) can run, only the forms that come near it at some size are timed (us per
+    // iteration at 96x96x192 / 256x256x512: -10 36.9 / 374, -4 42.4 / 600, -7 45.6 / 537, -2 46.5 / 624).
+    const bool march = march32_ok(g);
+    for (int cand : {-10, -7, -4, -2, -1, -3, -5, -6, -8, -132, -164}) {
+        if (cand == -10 ? !march : (march && cand != -7 && cand != -4 && cand != -2)) continue;
         if (cand <= -100 && !bulk32_ok(g)) continue;
         k_tune_reset<<<1, 1, 0, g->stream>>>(g->sc);
         g->slab32 = cand;
@@ -1698,7 +1709,7 @@ mhd_status_t tune_slab32(mhd_grid_s* g, int nc) {
     cudaMemsetAsync(g->r32, 0x3F, sizeof(float) * n3, g->stream);
     cudaMemsetAsync(g->p32, 0x3F, sizeof(float) * 2 * n3, g->stream);
     for (int slab : {8, 16, 32, 64}) {
-        if (!tiled32_ok(g)) break;
+        if (march || !tiled32_ok(g)) break;
         if (slab > 2 * g->d.nr && best > 0) break;
         if (tiled32_blocks(g, slab) > kMaxBlocks) continue;
         k_tune_reset<<<1, 1, 0, g->stream>>>(g->sc);
@@ -1714,14 +1725,17 @@ mhd_status_t tune_slab32(mhd_grid_s* g, int nc) {
             best = slab;
         }
     }
-    cudaMemsetAsync(g->r32, 0x3F, sizeof(float) * n3, g->stream);
-    cudaMemsetAsync(g->p32, 0x3F, sizeof(float) * 2 * n3, g->stream);
-    if (3.f * time_persist(g, true, nc, e0, e1) < best_ms) best = -9;
+    if (g->d.N <= kPersistTrial) {
+        cudaMemsetAsync(g->r32, 0x3F, sizeof(float) * n3, g->stream);
+        cudaMemsetAsync(g->p32, 0x3F, sizeof(float) * 2 * n3, g->stream);
+        if (3.f * time_persist(g, true, nc, e0, e1) < best_ms) best = -9;
+    }
     g->prof = prof;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (best == 0) return set_error(g, MHD_ERR_CUDA, "FP32 CG kernels: no launchable variant");
-    g->slab32 = best;  // -1 split, -2 folded, -3/-4 recompute pair, -9 persistent, <= -100 bulk-staged pair, > 0 tiled slab
+    g->slab32 = best;  // -1 split, -2 folded, -3/-4 recompute pair, -9 persistent, -10 marching,
+                       // <= -100 bulk-staged pair, > 0 tiled slab
     return check_cuda(g, "tune slab");
 }
 }  // namespace
@@ -1738,8 +1752,7 @@ mhd_status_t tune_slab64(mhd_grid_s* g) {
     }
     // vectors that fit the CTAs' shared memory (368 thousand cells): the persistent kernel, by rule. us per
     // iteration, it against the split kernels: 32x32x64 13.5 / 20.0, 48x48x96 23.5 / 32.7,
-    // 61x47x118 30.7 / 43.1. Above that it is one of the timed candidates (64x64x128: 42.7 / 54.3;
-    // 96x96x192: 137.7 / 140.8; 160x160x320: 615 / 560).
+    // 61x47x118 30.7 / 43.1. Above that it is one of the timed candidates.
     if (persist_mode(g, false, 3) == 1) {
         g->slab64 = -3;
         return MHD_OK;
@@ -1771,9 +1784,11 @@ mhd_status_t tune_slab64(mhd_grid_s* g) {
             best = slab;
         }
     }
-    cudaMemsetAsync(g->r64, 0x3F, sizeof(double) * n3, g->stream);
-    cudaMemsetAsync(g->p64, 0x3F, sizeof(double) * 2 * n3, g->stream);
-    if (2.f * time_persist(g, false, 3, e0, e1) < best_ms) best = -3;
+    if (g->d.N <= kPersistTrial) {
+        cudaMemsetAsync(g->r64, 0x3F, sizeof(double) * n3, g->stream);
+        cudaMemsetAsync(g->p64, 0x3F, sizeof(double) * 2 * n3, g->stream);
+        if (2.f * time_persist(g, false, 3, e0, e1) < best_ms) best = -3;
+    }
     g->prof = prof;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -1875,7 +1890,7 @@ mhd_status_t solve(mhd_grid_s* g, const double* alpha_dev, int nc, const double*
         const int ps = prof_begin(g, g->stream, MHD_KERNEL_OUTER_RES);
         const int restart = (o == 0 || prm->mixed_restart) ? 1 : 0;
         k_outer_res<2><<<grid_blocks(g, d.N / 2, resident_per_sm<k_outer_res<2>>()), kThreads, 0, g->stream>>>(
-            d, nc, b, x, g->r32, (!pc2 && g->slab32 <= -6 && g->slab32 >= -8) ? g->q32 : nullptr, g->p32, g->x32, g->t64, g->tu, g->sc,
+            d, nc, b, x, g->r32, (!pc2 && ((g->slab32 <= -6 && g->slab32 >= -8) || g->slab32 == -10)) ? g->q32 : nullptr, g->p32, g->x32, g->t64, g->tu, g->sc,
             g->partials, o == 0 ? 1 : 0, restart, pc2 ? 1 : 0, g->t32);
         if (pc2) pc2_reliable32(g, nc, restart);
         prof_end(g, g->stream, ps);
