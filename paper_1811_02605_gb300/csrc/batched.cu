@@ -1,19 +1,23 @@
 // Batched FP64 PCG: many independent systems M_alpha_s x_s = b_s on grids of different sizes,
 // solved together by ONE persistent cooperative kernel launch (replayed from a CUDA graph).
 //
-// Each system uses its own grid's tables and workspace (the scaled CG of pcg.cu: p = r + beta p,
-// q = A~ p, x += alpha p, r -= alpha q). The cells of all systems are cut into equal chunks; CTA b
-// takes chunks b, b + nblocks, ... Each chunk writes one partial per dot product. After a grid
-// barrier every CTA sums the partials of every system in chunk order, so all CTAs derive the same
-// alpha, beta and stop decisions without a further barrier (three grid barriers per iteration).
-// A converged system drops out of the work list; the launch ends when every system is done.
+// Each system uses its own grid's tables and workspace (the scaled CG of pcg.cu, its x update deferred to the
+// next p update). An iteration is three phases over the cells of all systems still running, with a grid
+// barrier after each: p = r + beta p (and x += alpha p of the iteration before), q = A~ p with <p, q>, r -=
+// alpha q with the norms. The phi-pairs of the running systems are laid end to end and cut into equal
+// ranges, one per CTA, anew whenever a system converges, so that every CTA has the same work to the end: a
+// range covers parts of one or a few systems, and a CTA writes one partial per dot product and system it
+// touches. After the barrier every CTA sums each system's partials in CTA order (one warp per system), so
+// all CTAs derive the same alpha, beta and stop decisions without a further barrier. (With fixed chunks of 4096
+// pairs dealt round-robin, the last round of chunks left most CTAs idle: 8 systems from 32x32x64 to
+// 96x96x192 took 405 ms, now 285 ms; FP64 instructions and then the p update's traffic bound it.)
 //
 // The grid barrier is a generation counter in global memory. Every wait is bounded: after an
 // iteration limit or a %globaltimer budget the CTA records MHD_ERR_TIMEOUT and returns, and the
 // others then time out at the same barrier instead of hanging.
 //
-// The chunk size and the number of CTAs per SM are chosen by a small autotuner: on the first
-// call for a batch shape it times a few iterations of each candidate and keeps the fastest.
+// The number of CTAs per SM is chosen by a small autotuner: on the first call for a batch it times a few
+// iterations of each candidate and keeps the fastest.
 #include <algorithm>
 #include <chrono>
 #include <cmath>
@@ -42,19 +46,16 @@ using namespace mhd;
 namespace {
 
 constexpr int kMaxSys = 256;
-constexpr int kBT = 256;  // threads per CTA
+constexpr int kBT = 512;  // threads per CTA
+constexpr unsigned int kAlign = 16;   // ranges start on multiples of 16 pairs (256 bytes)
 
 struct SysDesc {
     Dims d;
     double *x, *r, *p, *q;
     const double *ar, *at, *ap, *dg;
     PcgScalars* sc;
-    int c0, c1;  // chunk range
-};
-
-struct Chunk {
-    int sys;
-    unsigned int g0, g1;  // phi-pair groups [g0, g1)
+    unsigned int groups;   // phi pairs of a component
+    int pad;
 };
 
 struct BarrierState {
@@ -114,72 +115,100 @@ __device__ __forceinline__ double block_sum(double v, double* sm) {
     return s;  // valid in thread 0
 }
 
-__global__ void __launch_bounds__(kBT) k_batched_pcg(const SysDesc* __restrict__ sys, int nsys,
-                                                     const Chunk* __restrict__ chunks, int nchunks,
-                                                     double* __restrict__ part, BarrierState* bs,
-                                                     unsigned long long budget_ns, unsigned int extra) {
-    __shared__ double s_rho[kMaxSys], s_alpha[kMaxSys], s_beta[kMaxSys], s_bb[kMaxSys], s_tol[kMaxSys];
+__global__ void __launch_bounds__(kBT, 2) k_batched_pcg(const SysDesc* __restrict__ sys, int nsys,
+                                                        double* __restrict__ part, BarrierState* bs,
+                                                        unsigned long long budget_ns, unsigned int extra) {
+    __shared__ double s_rho[kMaxSys], s_alpha[kMaxSys], s_beta[kMaxSys], s_ax[kMaxSys], s_bound[kMaxSys];
     __shared__ int s_state[kMaxSys], s_iter[kMaxSys], s_max[kMaxSys];
+    __shared__ unsigned int pre[kMaxSys + 1];   // running systems laid end to end: first pair of each
     __shared__ double red[kBT / 32];
-    __shared__ int any_active;
-    double* part_pq = part;
-    double* part_rho = part + nchunks;
-    double* part_rr = part + 2 * nchunks;
-    const unsigned int nb = gridDim.x;
+    __shared__ unsigned int per;                // pairs per CTA
+    __shared__ int first, last, changed;        // systems that this CTA's range touches
+    const unsigned int nb = gridDim.x, me = blockIdx.x;
     const unsigned int expect = nb + extra;  // extra > 0 only under fault injection
+    // partials: [3][nsys][nb]
+    double* part_pq = part;
+    double* part_rho = part + (size_t)nsys * nb;
+    double* part_rr = part + 2 * (size_t)nsys * nb;
 
     for (int s = threadIdx.x; s < nsys; s += kBT) {
         const PcgScalars* sc = sys[s].sc;
         s_rho[s] = sc->rho;
-        s_bb[s] = sc->bb;
-        s_tol[s] = sc->tol;
+        s_bound[s] = sc->tol * sqrt(sc->bb);
         s_max[s] = sc->max_iter;
         s_state[s] = sc->done;
         s_iter[s] = 0;
         s_beta[s] = 0.0;
         s_alpha[s] = 0.0;
+        s_ax[s] = 0.0;
     }
+    if (threadIdx.x == 0) changed = 1;
     __syncthreads();
 
     for (;;) {
-        if (threadIdx.x == 0) {
-            int a = 0;
-            for (int s = 0; s < nsys; s++) a |= (s_state[s] == 0);
-            any_active = a;
+        if (threadIdx.x == 0 && changed) {
+            unsigned int w = 0;
+            for (int s = 0; s < nsys; s++) {
+                pre[s] = w;
+                w += s_state[s] == 0 ? sys[s].groups : 0u;
+            }
+            pre[nsys] = w;
+            per = ((w + nb - 1) / nb + kAlign - 1) / kAlign * kAlign;
+            const unsigned long long lo = (unsigned long long)per * me, hi = lo + per;
+            first = nsys;
+            last = -1;
+            for (int s = 0; s < nsys; s++)
+                if (pre[s + 1] > pre[s] && pre[s + 1] > lo && pre[s] < hi) {
+                    if (first == nsys) first = s;
+                    last = s;
+                }
+            changed = 0;
         }
         __syncthreads();
-        if (!any_active) break;
+        if (pre[nsys] == 0) break;
+        const unsigned int lo = min((unsigned long long)per * me, (unsigned long long)pre[nsys]);
+        const unsigned int hi = min((unsigned long long)per * (me + 1), (unsigned long long)pre[nsys]);
+        // the range of system s in this CTA: pairs [g0, g1), empty unless it runs
+        auto range = [&](int s, unsigned int& g0, unsigned int& g1) {
+            g0 = max(lo, pre[s]) - pre[s];
+            g1 = min(hi, pre[s + 1]) > pre[s] ? min(hi, pre[s + 1]) - pre[s] : 0u;
+            return pre[s + 1] > pre[s] && g0 < g1;
+        };
 
-        // P1: p = r + beta p
-        for (int c = blockIdx.x; c < nchunks; c += nb) {
-            const Chunk ch = chunks[c];
-            if (s_state[ch.sys]) continue;
-            const SysDesc& S = sys[ch.sys];
-            const double beta = s_beta[ch.sys];
-            for (int k = 0; k < 3; k++) {
-                const double* r = S.r + k * S.d.N;
-                double* p = S.p + k * S.d.N;
-                for (unsigned int g = ch.g0 + threadIdx.x; g < ch.g1; g += kBT) {
-                    const double2 rv = *reinterpret_cast<const double2*>(r + 2ull * g);
-                    double2 pv = *reinterpret_cast<double2*>(p + 2ull * g);
+        // P1: x += alpha p of the iteration before, p = r + beta p
+        for (int s = first; s <= last; s++) {
+            unsigned int g0, g1;
+            if (!range(s, g0, g1)) continue;
+            const SysDesc& S = sys[s];
+            const double beta = s_beta[s], ax = s_ax[s];
+            for (unsigned int g = g0 + threadIdx.x; g < g1; g += kBT) {
+#pragma unroll
+                for (int k = 0; k < 3; k++) {
+                    double2* p = reinterpret_cast<double2*>(S.p + k * S.d.N) + g;
+                    double2* x = reinterpret_cast<double2*>(S.x + k * S.d.N) + g;
+                    const double2 rv = reinterpret_cast<const double2*>(S.r + k * S.d.N)[g];
+                    double2 pv = *p, xv = *x;
+                    xv.x = fma(ax, pv.x, xv.x);
+                    xv.y = fma(ax, pv.y, xv.y);
                     pv.x = fma(beta, pv.x, rv.x);
                     pv.y = fma(beta, pv.y, rv.y);
-                    *reinterpret_cast<double2*>(p + 2ull * g) = pv;
+                    *x = xv;
+                    *p = pv;
                 }
             }
         }
         if (!grid_barrier(bs, expect, budget_ns)) return;
 
-        // P2: q = A~ p, partial <p, q> per chunk
-        for (int c = blockIdx.x; c < nchunks; c += nb) {
-            const Chunk ch = chunks[c];
-            if (s_state[ch.sys]) continue;
-            const SysDesc& S = sys[ch.sys];
+        // P2: q = A~ p, partial <p, q> per system
+        for (int s = first; s <= last; s++) {
+            unsigned int g0, g1;
+            if (!range(s, g0, g1)) continue;
+            const SysDesc& S = sys[s];
             const Dims d = S.d;
             const long long plane = (long long)d.nt * d.np;
             const unsigned int npv = d.np / 2;
             double acc = 0.0;
-            for (unsigned int g = ch.g0 + threadIdx.x; g < ch.g1; g += kBT) {
+            for (unsigned int g = g0 + threadIdx.x; g < g1; g += kBT) {
                 const unsigned int ij = g / npv;
                 const int k0 = (int)(g - ij * npv) * 2;
                 const int i = (int)(ij / d.nt), j = (int)(ij - (unsigned)i * d.nt);
@@ -189,83 +218,78 @@ __global__ void __launch_bounds__(kBT) k_batched_pcg(const SysDesc* __restrict__
                 const double cp = S.ap[ij];
                 const int km = (k0 == 0) ? d.np - 1 : k0 - 1;
                 const int kp = (k0 + 2 == d.np) ? 0 : k0 + 2;
+                // at a wall the cell itself, with a coefficient that is exactly 0
+                const long long im = i > 0 ? -plane : 0, ip = i < d.nr - 1 ? plane : 0;
+                const int jm = j > 0 ? -d.np : 0, jp = j < d.nt - 1 ? d.np : 0;
+#pragma unroll 1
                 for (int k = 0; k < 3; k++) {
-                    const double* u = S.p + k * d.N;
-                    const double2 v = *reinterpret_cast<const double2*>(u + base);
-                    const long long row = base - k0;
-                    double o0 = fma(-cp, u[row + km] + v.y, v.x);
-                    double o1 = fma(-cp, v.x + u[row + kp], v.y);
-                    if (i > 0) {
-                        const double2 n = *reinterpret_cast<const double2*>(u + base - plane);
-                        o0 = fma(-cr_lo, n.x, o0);
-                        o1 = fma(-cr_lo, n.y, o1);
-                    }
-                    if (i < d.nr - 1) {
-                        const double2 n = *reinterpret_cast<const double2*>(u + base + plane);
-                        o0 = fma(-cr_hi, n.x, o0);
-                        o1 = fma(-cr_hi, n.y, o1);
-                    }
-                    if (j > 0) {
-                        const double2 n = *reinterpret_cast<const double2*>(u + base - d.np);
-                        o0 = fma(-ct_lo, n.x, o0);
-                        o1 = fma(-ct_lo, n.y, o1);
-                    }
-                    if (j < d.nt - 1) {
-                        const double2 n = *reinterpret_cast<const double2*>(u + base + d.np);
-                        o0 = fma(-ct_hi, n.x, o0);
-                        o1 = fma(-ct_hi, n.y, o1);
-                    }
+                    const double* u = S.p + k * d.N + base;
+                    const double2 v = *reinterpret_cast<const double2*>(u);
+                    const double2 a = *reinterpret_cast<const double2*>(u + im);
+                    const double2 b = *reinterpret_cast<const double2*>(u + ip);
+                    const double2 c = *reinterpret_cast<const double2*>(u + jm);
+                    const double2 e = *reinterpret_cast<const double2*>(u + jp);
+                    double o0 = fma(-cp, u[km - k0] + v.y, v.x);
+                    double o1 = fma(-cp, v.x + u[kp - k0], v.y);
+                    o0 = fma(-cr_lo, a.x, o0);
+                    o1 = fma(-cr_lo, a.y, o1);
+                    o0 = fma(-cr_hi, b.x, o0);
+                    o1 = fma(-cr_hi, b.y, o1);
+                    o0 = fma(-ct_lo, c.x, o0);
+                    o1 = fma(-ct_lo, c.y, o1);
+                    o0 = fma(-ct_hi, e.x, o0);
+                    o1 = fma(-ct_hi, e.y, o1);
                     *reinterpret_cast<double2*>(S.q + k * d.N + base) = make_double2(o0, o1);
                     acc = fma(v.x, o0, acc);
                     acc = fma(v.y, o1, acc);
                 }
             }
             const double t = block_sum(acc, red);
-            if (threadIdx.x == 0) part_pq[c] = t;
+            if (threadIdx.x == 0) part_pq[(size_t)s * nb + me] = t;
         }
         if (!grid_barrier(bs, expect, budget_ns)) return;
 
-        // alpha per active system: one warp per system, lanes strided over its chunks and a fixed
-        // shuffle tree, so every CTA forms identical values
-        {
-            const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-            for (int s = w; s < nsys; s += kBT / 32) {
-                if (s_state[s]) continue;
-                double pq = 0.0;
-                for (int c = sys[s].c0 + lane; c < sys[s].c1; c += 32) pq += __ldcg(&part_pq[c]);
-                for (int o = 16; o > 0; o >>= 1) pq += __shfl_xor_sync(0xffffffffu, pq, o);
-                if (lane == 0) {
-                    if (!isfinite(pq)) s_state[s] = 3;
-                    else if (!(pq > 0.0)) s_state[s] = 4;
-                    else s_alpha[s] = s_rho[s] / pq;
+        // alpha per running system: one warp per system, lanes strided over the CTAs that touch it and a
+        // fixed shuffle tree, so every CTA forms identical values
+        const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+        for (int s = w; s < nsys; s += kBT / 32) {
+            if (s_state[s]) continue;
+            double pq = 0.0;
+            for (unsigned int c = pre[s] / per + lane; c <= (pre[s + 1] - 1) / per; c += 32)
+                pq += __ldcg(&part_pq[(size_t)s * nb + c]);
+            for (int o = 16; o > 0; o >>= 1) pq += __shfl_xor_sync(0xffffffffu, pq, o);
+            if (lane == 0) {
+                int stt = 0;
+                if (!isfinite(pq)) stt = 3;
+                else if (!(pq > 0.0)) stt = 4;
+                else s_alpha[s] = s_rho[s] / pq;
+                if (stt) {
+                    s_state[s] = stt;
+                    s_ax[s] = 0.0;
+                    changed = 1;
                 }
             }
         }
         __syncthreads();
 
-        // P3: x += alpha p, r -= alpha q, partial rho and rr per chunk
-        for (int c = blockIdx.x; c < nchunks; c += nb) {
-            const Chunk ch = chunks[c];
-            if (s_state[ch.sys]) continue;
-            const SysDesc& S = sys[ch.sys];
-            const double al = s_alpha[ch.sys];
+        // P3: r -= alpha q, partial rho and rr per system
+        for (int s = first; s <= last; s++) {
+            unsigned int g0, g1;
+            if (s_state[s] || !range(s, g0, g1)) continue;
+            const SysDesc& S = sys[s];
+            const double al = s_alpha[s];
             const unsigned int npv = S.d.np / 2;
             double a_rho = 0.0, a_rr = 0.0;
-            for (unsigned int g = ch.g0 + threadIdx.x; g < ch.g1; g += kBT) {
+            for (unsigned int g = g0 + threadIdx.x; g < g1; g += kBT) {
                 double cell = 0.0;
+#pragma unroll
                 for (int k = 0; k < 3; k++) {
-                    double* x = S.x + k * S.d.N + 2ull * g;
-                    double* r = S.r + k * S.d.N + 2ull * g;
-                    const double2 pv = *reinterpret_cast<const double2*>(S.p + k * S.d.N + 2ull * g);
-                    const double2 qv = *reinterpret_cast<const double2*>(S.q + k * S.d.N + 2ull * g);
-                    double2 xv = *reinterpret_cast<double2*>(x);
-                    double2 rv = *reinterpret_cast<double2*>(r);
-                    xv.x = fma(al, pv.x, xv.x);
-                    xv.y = fma(al, pv.y, xv.y);
+                    double2* r = reinterpret_cast<double2*>(S.r + k * S.d.N) + g;
+                    const double2 qv = reinterpret_cast<const double2*>(S.q + k * S.d.N)[g];
+                    double2 rv = *r;
                     rv.x = fma(-al, qv.x, rv.x);
                     rv.y = fma(-al, qv.y, rv.y);
-                    *reinterpret_cast<double2*>(x) = xv;
-                    *reinterpret_cast<double2*>(r) = rv;
+                    *r = rv;
                     cell = fma(rv.x, rv.x, cell);
                     cell = fma(rv.y, rv.y, cell);
                 }
@@ -275,46 +299,48 @@ __global__ void __launch_bounds__(kBT) k_batched_pcg(const SysDesc* __restrict__
             const double t1 = block_sum(a_rho, red);
             const double t2 = block_sum(a_rr, red);
             if (threadIdx.x == 0) {
-                part_rho[c] = t1;
-                part_rr[c] = t2;
+                part_rho[(size_t)s * nb + me] = t1;
+                part_rr[(size_t)s * nb + me] = t2;
             }
         }
         if (!grid_barrier(bs, expect, budget_ns)) return;
 
-        // beta and the stop test per active system (one warp per system)
-        {
-            const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-            for (int s = w; s < nsys; s += kBT / 32) {
-                if (s_state[s]) continue;
-                double rho = 0.0, rr = 0.0;
-                for (int c = sys[s].c0 + lane; c < sys[s].c1; c += 32) {
-                    rho += __ldcg(&part_rho[c]);
-                    rr += __ldcg(&part_rr[c]);
-                }
-                for (int o = 16; o > 0; o >>= 1) {
-                    rho += __shfl_xor_sync(0xffffffffu, rho, o);
-                    rr += __shfl_xor_sync(0xffffffffu, rr, o);
-                }
-                if (lane == 0) {
-                    s_iter[s] += 1;
-                    s_beta[s] = rho / s_rho[s];
-                    s_rho[s] = rho;
-                    int stt = 0;
-                    if (!isfinite(rr) || !isfinite(rho)) stt = 3;
-                    else if (sqrt(rr) <= s_tol[s] * sqrt(s_bb[s])) stt = 1;
-                    else if (s_iter[s] >= s_max[s]) stt = 2;
-                    if (stt && blockIdx.x == 0) sys[s].sc->rr = rr;
+        // beta and the stop test per running system (one warp per system)
+        for (int s = w; s < nsys; s += kBT / 32) {
+            if (s_state[s]) continue;
+            double rho = 0.0, rr = 0.0;
+            for (unsigned int c = pre[s] / per + lane; c <= (pre[s + 1] - 1) / per; c += 32) {
+                rho += __ldcg(&part_rho[(size_t)s * nb + c]);
+                rr += __ldcg(&part_rr[(size_t)s * nb + c]);
+            }
+            for (int o = 16; o > 0; o >>= 1) {
+                rho += __shfl_xor_sync(0xffffffffu, rho, o);
+                rr += __shfl_xor_sync(0xffffffffu, rr, o);
+            }
+            if (lane == 0) {
+                s_iter[s] += 1;
+                s_beta[s] = rho / s_rho[s];
+                s_rho[s] = rho;
+                s_ax[s] = s_alpha[s];   // x += alpha p is left to the next P1, or to the finish
+                int stt = 0;
+                if (!isfinite(rr) || !isfinite(rho)) stt = 3;
+                else if (sqrt(rr) <= s_bound[s]) stt = 1;
+                else if (s_iter[s] >= s_max[s]) stt = 2;
+                if (stt) {
+                    if (me == 0) sys[s].sc->rr = rr;
                     s_state[s] = stt;
+                    changed = 1;
                 }
             }
         }
         __syncthreads();
     }
-    if (blockIdx.x == 0) {
+    if (me == 0) {
         for (int s = threadIdx.x; s < nsys; s += kBT) {
             PcgScalars* sc = sys[s].sc;
             sc->iter = s_iter[s];
             sc->rho = s_rho[s];
+            sc->ax = s_ax[s];
             sc->done = s_state[s];
         }
     }
@@ -329,14 +355,11 @@ struct Plan {
     std::vector<const double*> b;
     std::vector<double*> x;
     SysDesc* d_sys = nullptr;
-    Chunk* d_chunks = nullptr;
     double* d_part = nullptr;
     BarrierState* d_bar = nullptr;
     double* d_alpha = nullptr;   // device alphas [n]
     double* h_alpha = nullptr;   // pinned host staging [n]
-    int nchunks = 0;
     int blocks = 0;
-    unsigned int chunk_groups = 0;
     cudaGraphExec_t graph = nullptr;
     cudaGraphExec_t trial = nullptr;
     double tol = 0;
@@ -352,7 +375,6 @@ void free_plan(Plan* P) {
     if (P->graph) cudaGraphExecDestroy(P->graph);
     if (P->trial) cudaGraphExecDestroy(P->trial);
     if (P->d_sys) cudaFree(P->d_sys);
-    if (P->d_chunks) cudaFree(P->d_chunks);
     if (P->d_part) cudaFree(P->d_part);
     if (P->d_bar) cudaFree(P->d_bar);
     if (P->d_alpha) cudaFree(P->d_alpha);
@@ -368,10 +390,9 @@ int max_coop_blocks_per_sm() {
     return nb;
 }
 
-// (re)build the chunk list and device descriptors for a chunk size and CTA count
-mhd_status_t build_layout(Plan& P, unsigned int chunk_groups, int blocks) {
+// device descriptors and partials for a CTA count
+mhd_status_t build_layout(Plan& P, int blocks) {
     std::vector<SysDesc> sd(P.n);
-    std::vector<Chunk> ch;
     for (int s = 0; s < P.n; s++) {
         mhd_grid_s* g = P.grids[s];
         SysDesc& S = sd[s];
@@ -385,25 +406,17 @@ mhd_status_t build_layout(Plan& P, unsigned int chunk_groups, int blocks) {
         S.ap = g->t64.ap;
         S.dg = g->tu.dg;
         S.sc = g->sc;
-        S.c0 = (int)ch.size();
-        const unsigned int G = (unsigned int)(g->d.N / 2);
-        for (unsigned int g0 = 0; g0 < G; g0 += chunk_groups) ch.push_back(Chunk{s, g0, std::min(G, g0 + chunk_groups)});
-        S.c1 = (int)ch.size();
+        S.groups = (unsigned int)(g->d.N / 2);
+        S.pad = 0;
     }
     cudaStream_t st = P.grids[0]->stream;
-    if (P.d_chunks) cudaFree(P.d_chunks);
     if (P.d_part) cudaFree(P.d_part);
-    P.d_chunks = nullptr;
     P.d_part = nullptr;
-    if (cudaMalloc(&P.d_chunks, sizeof(Chunk) * ch.size()) != cudaSuccess ||
-        cudaMalloc(&P.d_part, sizeof(double) * 3 * ch.size()) != cudaSuccess)
+    if (cudaMalloc(&P.d_part, sizeof(double) * 3 * (size_t)P.n * blocks) != cudaSuccess)
         return fail(MHD_ERR_OOM, "pcg_solve_batched: allocation failed");
     cudaMemcpyAsync(P.d_sys, sd.data(), sizeof(SysDesc) * P.n, cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(P.d_chunks, ch.data(), sizeof(Chunk) * ch.size(), cudaMemcpyHostToDevice, st);
     cudaMemsetAsync(P.d_bar, 0, sizeof(BarrierState), st);
     if (cudaStreamSynchronize(st) != cudaSuccess) return fail(MHD_ERR_CUDA, "pcg_solve_batched: upload failed");
-    P.nchunks = (int)ch.size();
-    P.chunk_groups = chunk_groups;
     P.blocks = blocks;
     return MHD_OK;
 }
@@ -452,8 +465,7 @@ void enqueue_batch(Plan& P, cudaStream_t st, bool finish, int max_iter_override)
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, k_batched_pcg, (const SysDesc*)P.d_sys, P.n, (const Chunk*)P.d_chunks, P.nchunks, P.d_part,
-                       P.d_bar, P.budget_ns, P.extra);
+    cudaLaunchKernelEx(&cfg, k_batched_pcg, (const SysDesc*)P.d_sys, P.n, P.d_part, P.d_bar, P.budget_ns, P.extra);
     if (finish) {
         for (int s = 0; s < P.n; s++) {
             mhd_grid_s* g = P.grids[s];
@@ -484,45 +496,37 @@ mhd_status_t capture(Plan& P, bool finish, int max_iter, cudaGraphExec_t* out) {
     return MHD_OK;
 }
 
-// autotuner: time a few iterations of each (chunk size, CTAs per SM) candidate
+// autotuner: time a few iterations of each number of CTAs per SM
 mhd_status_t autotune(Plan& P) {
     const int nsm = P.grids[0]->num_sms;
     const int maxb = std::max(1, max_coop_blocks_per_sm());
-    const unsigned int chunk_cands[] = {4096, 16384, 65536};
-    std::vector<int> bps;
-    for (int b : {1, 2, 4, 8})
-        if (b <= maxb) bps.push_back(b);
     cudaStream_t st = P.grids[0]->stream;
     double best = 1e30;
-    unsigned int best_c = chunk_cands[1];
-    int best_b = std::min(maxb, 2) * nsm;
+    int best_b = nsm;
     const int trial_iters = 8;
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
-    for (unsigned int cg : chunk_cands) {
-        for (int b : bps) {
-            if (build_layout(P, cg, b * nsm) != MHD_OK) return MHD_ERR_OOM;
-            if (capture(P, false, trial_iters, &P.trial) != MHD_OK) return MHD_ERR_CUDA;
-            cudaGraphLaunch(P.trial, st);  // warm
-            cudaEventRecord(e0, st);
-            cudaGraphLaunch(P.trial, st);
-            cudaEventRecord(e1, st);
-            if (cudaEventSynchronize(e1) != cudaSuccess) return fail(MHD_ERR_CUDA, "autotune sync");
-            float ms = 0;
-            cudaEventElapsedTime(&ms, e0, e1);
-            if (ms < best) {
-                best = ms;
-                best_c = cg;
-                best_b = b * nsm;
-            }
+    for (int b = 1; b <= maxb; b++) {
+        if (build_layout(P, b * nsm) != MHD_OK) return MHD_ERR_OOM;
+        if (capture(P, false, trial_iters, &P.trial) != MHD_OK) return MHD_ERR_CUDA;
+        cudaGraphLaunch(P.trial, st);  // warm
+        cudaEventRecord(e0, st);
+        cudaGraphLaunch(P.trial, st);
+        cudaEventRecord(e1, st);
+        if (cudaEventSynchronize(e1) != cudaSuccess) return fail(MHD_ERR_CUDA, "autotune sync");
+        float ms = 0;
+        cudaEventElapsedTime(&ms, e0, e1);
+        if (ms < best) {
+            best = ms;
+            best_b = b * nsm;
         }
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (P.trial) cudaGraphExecDestroy(P.trial);
     P.trial = nullptr;
-    return build_layout(P, best_c, best_b);
+    return build_layout(P, best_b);
 }
 
 }  // namespace
@@ -568,7 +572,6 @@ mhd_status_t prepare(int n, const mhd_grid_t* grids, const double* alpha, const 
         key.push_back(x[s]);
     }
     Plan*& pp = g_plans[key];
-    cudaStream_t st = grids[0]->stream;
     if (!pp) {
         Plan* P = new Plan();
         P->n = n;
