@@ -660,7 +660,7 @@ extern "C" mhd_status_t mhd_adjoint_step(mhd_grid_t g, const mhd_params_t* p, co
     cudaMemcpyAsync(w.b1r, s0->br, sizeof(double) * nbr, cudaMemcpyDeviceToDevice, st);
     cudaMemcpyAsync(w.b1t, s0->bt, sizeof(double) * nbt, cudaMemcpyDeviceToDevice, st);
     cudaMemcpyAsync(w.b1p, s0->bp, sizeof(double) * nbp, cudaMemcpyDeviceToDevice, st);
-    induction(g, s0->vr, s0->vt, s0->vp, g->dlt, 0.5, eta, nullptr, dt, w.b1r, w.b1t, w.b1p);
+    induction(g, s0->vr, s0->vt, s0->vp, g->dlt, 0.5, eta, nullptr, dt, w.b1r, w.b1t, w.b1p, true);
     if (res) {
         stt = res_solve(g, &g->ss->dt, p->eta, w.b1r, w.b1t, w.b1p, p, nullptr, nullptr);
         if (stt == MHD_ERR_CUDA || stt == MHD_ERR_OOM) return stt;

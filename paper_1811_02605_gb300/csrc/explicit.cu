@@ -1,5 +1,5 @@
 // Explicit parts of the zero-beta step (Eq. 1; Sec. 2.2 explicit predictor-corrector
-// upwinding), all FP64, one thread per output element:
+// upwinding), all FP64, one warp per row of output elements:
 //   - step coefficients: dt from the flow CFL, C_w, the semi-implicit coefficient (Sec. 2.1)
 //   - J = curl_h B on edges (Stokes on the dual faces around each edge)
 //   - momentum force b = rho V dt (-(v.grad)v + J x B / rho)
@@ -14,6 +14,7 @@
 //   - Ghost tangential B beyond r0 and r1 equals the first interior value, at mirrored radii.
 //   - Advection: Dirichlet mirror ghost (-u) at r0, zero gradient at r1, no flux from the pole.
 //   - Tangential E is 0 on r0 (line-tied); on r1 it is the mean of the two interior cells.
+#include <algorithm>
 #include <cmath>
 
 #include "mhd_internal.cuh"
@@ -24,19 +25,75 @@ namespace mhd {
 namespace {
 
 
-// cell-centred B: mean of opposite faces; in the polar rings B_theta is the mean of the non-polar
-// face and the pole value (bh: first-harmonic sums of the B_theta face rings, bt_harmonics)
-__device__ __forceinline__ void bcentre(const Dims& d, const Geo& G, const double* __restrict__ bh,
-                                        const double* __restrict__ br, const double* __restrict__ bt,
-                                        const double* __restrict__ bp, int i, int j, int k, double (&o)[3]) {
-    o[0] = 0.5 * (br[ix(d, i, j, k)] + br[ix(d, i + 1, j, k)]);
-    if (j == 0) o[1] = polar_btc(G, d.np, bh + 2 * i, k, bt[ixt(d, i, 1, k)]);
-    else if (j == d.nt - 1) o[1] = polar_btc(G, d.np, bh + 2 * (d.nr + i), k, bt[ixt(d, i, d.nt - 1, k)]);
-    else o[1] = 0.5 * (bt[ixt(d, i, j, k)] + bt[ixt(d, i, j + 1, k)]);
-    o[2] = 0.5 * (bp[ix(d, i, j, k)] + bp[ix(d, i, j, kp1(d, k))]);
+// FP64 runs at 2 multiply-adds per clock and SM on this part (64 cycles a warp instruction and scheduler), so
+// these kernels are bound by their count of FP64 instructions; integer work, loads and address arithmetic are
+// free beside it. Hence: one warp per row (i, j) of np elements, so that whatever depends on the row alone is
+// formed once a row; the means are kept as plain sums (B_c doubled, J_c and the edge E by powers of two, which
+// scale exactly) and the factor goes into a row constant; signs and maxima are integer tests; the upwind
+// difference is |u_d| / h (u - u_upwind), one form for both signs. Coefficients, force, induction with
+// resistivity and diagnostics of a 256x256x512 grid: 21.3 -> 13.9 ms, at about 200 FP64 instructions a cell and 82 to 89% of the pipe.
+__device__ __forceinline__ unsigned int first_row() {
+    return blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
+}
+__device__ __forceinline__ unsigned int row_stride() { return gridDim.x * (kThreads / 32); }
+
+__device__ __forceinline__ double warp_sum(double s) {
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+}
+// x > 0 (true also for a NaN with a clear sign, which makes every use of the result a NaN)
+__device__ __forceinline__ bool positive(double x) { return __double_as_longlong(x) > 0; }
+// m = max(m, |x|) on the bits of non-negative doubles; a NaN is ignored, as by fmax
+__device__ __forceinline__ void max_abs(long long& m, double x) {
+    const long long b = __double_as_longlong(x) & 0x7fffffffffffffffll;
+    if (b > m && b <= 0x7ff0000000000000ll) m = b;
 }
 
-// velocity u = v + f * dlt (dlt may be null)
+// a row (i, j) of cells: the addresses of the faces around it, and the polar rule
+struct FaceRow {
+    const double *r0, *r1, *t0, *t1, *p0;
+    const double* h;   // polar rings: the two harmonic sums of the B_theta ring beside it
+    const double* pcs;
+    double pole_f;
+    int np;
+    __device__ __forceinline__ FaceRow(const Dims& d, const Geo& G, const double* __restrict__ bh, const double* br,
+                                       const double* bt, const double* bp, int i, int j)
+        : r0(br + ix(d, i, j, 0)), r1(br + ix(d, i + 1, j, 0)), t0(bt + ixt(d, i, j, 0)), t1(bt + ixt(d, i, j + 1, 0)),
+          p0(bp + ix(d, i, j, 0)), h(j == 0 ? bh + 2 * i : (j == d.nt - 1 ? bh + 2 * (d.nr + i) : nullptr)), pcs(G.pcs),
+          pole_f(G.pole_f), np(d.np) {
+        if (j == 0) t0 = t1;        // the non-polar face on either side
+        else if (j == d.nt - 1) t1 = t0;
+    }
+    // twice the cell-centred B: sums of opposite faces; in the polar rings B_theta is the non-polar face and the
+    // pole value (first phi harmonic of the ring, see polar_btc)
+    __device__ __forceinline__ void twice(int k, int kp, double (&o)[3]) const {
+        o[0] = r0[k] + r1[k];
+        o[1] = h ? t0[k] + (h[0] * pcs[k] + h[1] * pcs[np + k]) * pole_f : t0[k] + t1[k];
+        o[2] = p0[k] + p0[kp];
+    }
+};
+
+// four times J at the cells of a row, from the edge arrays (polar phi edges left out)
+struct EdgeRow {
+    const double *r0, *r1, *t0, *t1, *p00, *p01, *p10, *p11;
+    __device__ __forceinline__ EdgeRow(const Dims& d, const double* jr, const double* jt, const double* jp, int i, int j)
+        : r0(jr + ixt(d, i, j, 0)), r1(jr + ixt(d, i, j + 1, 0)), t0(jt + ix(d, i, j, 0)), t1(jt + ix(d, i + 1, j, 0)) {
+        const int lo = j == 0 ? 1 : j, hi = j == d.nt - 1 ? d.nt - 1 : j + 1;
+        p00 = jp + ixt(d, i, lo, 0);
+        p01 = jp + ixt(d, i, hi, 0);
+        p10 = jp + ixt(d, i + 1, lo, 0);
+        p11 = jp + ixt(d, i + 1, hi, 0);
+    }
+    __device__ __forceinline__ void four(int k, int kp, double (&o)[3]) const {
+        o[0] = (r0[k] + r0[kp]) + (r1[k] + r1[kp]);
+        o[1] = (t0[k] + t0[kp]) + (t1[k] + t1[kp]);
+        o[2] = (p00[k] + p01[k]) + (p10[k] + p11[k]);
+    }
+};
+
+// velocity u = v + f * dlt; DLT false: u = v (a test of the pointer at run time would leave the multiply-adds in
+// place, switched off but taking their turn of the FP64 pipe: force 69 FP64 instructions a cell instead of 54)
+template <bool DLT>
 struct Vel {
     const double *vr, *vt, *vp, *dl;
     double f;
@@ -45,7 +102,7 @@ struct Vel {
         u[0] = vr[c];
         u[1] = vt[c];
         u[2] = vp[c];
-        if (dl) {
+        if constexpr (DLT) {
             u[0] += f * dl[c];
             u[1] += f * dl[N + c];
             u[2] += f * dl[2 * N + c];
@@ -58,27 +115,31 @@ struct Vel {
 // ------------------------------------------------------------------------------------------
 // step coefficients
 // ------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreads) k_coeffs(Dims d, Geo G, Vel v, const double* __restrict__ bh,
+// Every term of a row has the same factors, and rounding is monotone, so the row's largest |v|^2 and |B|^2 give
+// the largest products bit for bit.
+__global__ void __launch_bounds__(kThreads) k_coeffs(Dims d, Geo G, Vel<false> v, const double* __restrict__ bh,
                                                      const double* __restrict__ br,
                                                      const double* __restrict__ bt,
                                                      const double* __restrict__ bp, double nu, double cfl,
                                                      double dt_fixed, double dt_max, double asi_fixed,
                                                      StepScalars* ss, double* __restrict__ partials) {
     double mkv = 0.0, mka = 0.0;
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < d.N;
-         c += (long long)gridDim.x * blockDim.x) {
-        int k;
-        unsigned int ij;
-        split_np(d, c, k, ij);
-        const int j = (int)(ij % d.nt), i = (int)(ij / d.nt);
-        double u[3], B[3];
-        v.at(c, u);
-        bcentre(d, G, bh, br, bt, bp, i, j, k, B);
+    const unsigned int rows = (unsigned int)(d.nr * d.nt);
+    for (unsigned int ij = first_row(); ij < rows; ij += row_stride()) {
+        const int i = (int)(ij / d.nt), j = (int)(ij - (unsigned int)i * d.nt);
+        const FaceRow F(d, G, bh, br, bt, bp, i, j);
+        long long mv = 0, mb = 0;
+#pragma unroll 4
+        for (int k = threadIdx.x & 31; k < d.np; k += 32) {
+            double u[3], B[3];
+            v.at((long long)ij * d.np + k, u);
+            F.twice(k, kp1(d, k), B);
+            max_abs(mv, u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+            max_abs(mb, B[0] * B[0] + B[1] * B[1] + B[2] * B[2]);
+        }
         const double kt2 = G.kt2[ij];
-        const double vv = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-        const double bb = B[0] * B[0] + B[1] * B[1] + B[2] * B[2];
-        mkv = fmax(mkv, kt2 * vv);
-        mka = fmax(mka, kt2 * bb / G.rho[i]);
+        mkv = fmax(mkv, kt2 * __longlong_as_double(mv));
+        mka = fmax(mka, kt2 * (0.25 * __longlong_as_double(mb)) / G.rho[i]);
     }
     double val[2] = {mkv, mka}, out[2];
     if (reduce_last<2, OpMax>(val, partials, &ss->count, out) && threadIdx.x == 0) {
@@ -111,9 +172,9 @@ __global__ void __launch_bounds__(kThreads) k_coeffs(Dims d, Geo G, Vel v, const
 
 mhd_status_t coeffs(mhd_grid_s* g, const mhd_params_t* p, const double* vr, const double* vt,
                     const double* vp, const double* br, const double* bt, const double* bp) {
-    Vel v{vr, vt, vp, nullptr, 0.0, g->d.N};
+    const Vel<false> v{vr, vt, vp, nullptr, 0.0, g->d.N};
     bt_harmonics(g, bt);
-    const int blocks = grid_blocks(g, g->d.N, 4);
+    const int blocks = grid_blocks(g, 32ll * g->d.nr * g->d.nt, resident_per_sm<k_coeffs>());
     k_coeffs<<<blocks, kThreads, 0, g->stream>>>(g->d, g->geo, v, g->bharm, br, bt, bp, p->nu, p->cfl, p->dt_fixed,
                                                  p->dt_max, p->alpha_si_fixed, g->ss, g->partials);
     return check_cuda(g, "coeffs");
@@ -188,96 +249,112 @@ void bt_harmonics(mhd_grid_s* g, const double* bt, cudaStream_t st) {
 // ------------------------------------------------------------------------------------------
 // current density on edges
 // ------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreads) k_jr(Dims d, const double* __restrict__ cr,
-                                                 const double* __restrict__ bt, const double* __restrict__ bp,
-                                                 const double* __restrict__ ring, double* __restrict__ jr) {
-    const long long n = (long long)d.nr * (d.nt + 1) * d.np;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-        int k;
-        unsigned int q;
-        split_np(d, e, k, q);
-        const int j = (int)(q % (d.nt + 1)), i = (int)(q / (d.nt + 1));
-        const double* c = cr + 4 * (size_t)q;
-        double val;
-        if (j == 0) val = ring[i] * c[3];                   // north cap circulation / cap area
-        else if (j == d.nt) val = -ring[d.nr + i] * c[3];   // south cap
-        else val = c[0] * bp[ix(d, i, j, k)] - c[1] * bp[ix(d, i, j - 1, k)] -
-                   c[2] * (bt[ixt(d, i, j, k)] - bt[ixt(d, i, j, km1(d, k))]);
-        jr[e] = val;
+// J on all edges in one launch, a warp per row; a polar radial row takes its ring's sum of B_phi itself (the cap
+// circulation), and with bh the warps of the first 2 nr rows form the harmonics of the B_theta rings beside the
+// poles. walls_zero: the resistive operator's current, 0 on the tangential edges of r0 and r1.
+__global__ void __launch_bounds__(kThreads) k_current(Dims d, const double* __restrict__ cr,
+                                                      const double* __restrict__ ct, const double* __restrict__ cp,
+                                                      const double* __restrict__ br, const double* __restrict__ bt,
+                                                      const double* __restrict__ bp, double* __restrict__ jr,
+                                                      double* __restrict__ jt, double* __restrict__ jp,
+                                                      const double* __restrict__ pcs, double* __restrict__ bh,
+                                                      int walls_zero) {
+    const unsigned int n_h = bh ? 2u * d.nr : 0u, n_r = (unsigned int)(d.nr * (d.nt + 1)),
+                       n_t = (unsigned int)((d.nr + 1) * d.nt), n_p = (unsigned int)((d.nr + 1) * (d.nt + 1));
+    const int np = d.np, lane = threadIdx.x & 31;
+    for (unsigned int w = first_row(); w < n_h + n_r + n_t + n_p; w += row_stride()) {
+        if (w < n_h) {
+            const int i = (int)(w % d.nr), south = (int)(w / d.nr);
+            const double* row = bt + ixt(d, i, south ? d.nt - 1 : 1, 0);
+            double c = 0.0, s = 0.0;
+            for (int k = lane; k < np; k += 32) {
+                c = fma(row[k], pcs[k], c);
+                s = fma(row[k], pcs[np + k], s);
+            }
+            c = warp_sum(c);
+            s = warp_sum(s);
+            if (lane == 0) {
+                bh[2 * w] = c;
+                bh[2 * w + 1] = s;
+            }
+        } else if (w < n_h + n_r) {
+            const unsigned int q = w - n_h;
+            const int i = (int)(q / (d.nt + 1)), j = (int)(q - (unsigned int)i * (d.nt + 1));
+            const double* c = cr + 4 * (size_t)q;
+            double* out = jr + (long long)q * np;
+            if (j == 0 || j == d.nt) {
+                const double* row = bp + ix(d, i, j == 0 ? 0 : d.nt - 1, 0);
+                double s = 0.0;
+                for (int k = lane; k < np; k += 32) s += row[k];
+                s = warp_sum(s) * (j == 0 ? c[3] : -c[3]);   // cap circulation / cap area
+                for (int k = lane; k < np; k += 32) out[k] = s;
+            } else {
+                const double c0 = c[0], c1 = c[1], c2 = c[2];
+                const double *b = bp + ix(d, i, j, 0), *a = b - np, *t = bt + ixt(d, i, j, 0);
+#pragma unroll 4
+                for (int k = lane; k < np; k += 32) out[k] = c0 * b[k] - c1 * a[k] - c2 * (t[k] - t[km1(d, k)]);
+            }
+        } else if (w < n_h + n_r + n_t) {
+            const unsigned int q = w - n_h - n_r;
+            const int i = (int)(q / d.nt), j = (int)(q - (unsigned int)i * d.nt);
+            const bool wall = walls_zero && (i == 0 || i == d.nr);
+            // ghost B_phi beyond r0 / r1 = the first interior value (at the mirrored radius in the table)
+            const double *lo = bp + ix(d, i > 0 ? i - 1 : 0, j, 0), *hi = bp + ix(d, i < d.nr ? i : d.nr - 1, j, 0);
+            const double* b = br + ix(d, i, j, 0);
+            const double* c = ct + 3 * (size_t)q;
+            const double c0 = c[0], c1 = c[1], c2 = c[2];
+            double* out = jt + (long long)q * np;
+#pragma unroll 4
+            for (int k = lane; k < np; k += 32)
+                out[k] = wall ? 0.0 : c0 * lo[k] + c1 * (b[k] - b[km1(d, k)]) - c2 * hi[k];
+        } else {
+            const unsigned int q = w - n_h - n_r - n_t;
+            const int i = (int)(q / (d.nt + 1)), j = (int)(q - (unsigned int)i * (d.nt + 1));
+            double* out = jp + (long long)q * np;
+            if (j == 0 || j == d.nt || (walls_zero && (i == 0 || i == d.nr))) {
+                for (int k = lane; k < np; k += 32) out[k] = 0.0;
+            } else {
+                const double *lo = bt + ixt(d, i > 0 ? i - 1 : 0, j, 0), *hi = bt + ixt(d, i < d.nr ? i : d.nr - 1, j, 0);
+                const double *b = br + ix(d, i, j, 0), *a = b - np;
+                const double* c = cp + 3 * (size_t)q;
+                const double c0 = c[0], c1 = c[1], c2 = c[2];
+#pragma unroll 4
+                for (int k = lane; k < np; k += 32) out[k] = c0 * (a[k] - b[k]) + c1 * hi[k] - c2 * lo[k];
+            }
+        }
     }
 }
 
-// walls_zero: the resistive operator's current, 0 on the tangential edges of r0 and r1
-__global__ void __launch_bounds__(kThreads) k_jt(Dims d, const double* __restrict__ ct,
-                                                 const double* __restrict__ br, const double* __restrict__ bp,
-                                                 double* __restrict__ jt, int walls_zero) {
-    const long long n = (long long)(d.nr + 1) * d.nt * d.np;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-        int k;
-        unsigned int q;
-        split_np(d, e, k, q);
-        const int j = (int)(q % d.nt), i = (int)(q / d.nt);
-        if (walls_zero && (i == 0 || i == d.nr)) {
-            jt[e] = 0.0;
-            continue;
-        }
-        // ghost B_phi beyond r0 / r1 = the first interior value (at the mirrored radius in the table)
-        const int ilo = (i > 0) ? i - 1 : 0, ihi = (i < d.nr) ? i : d.nr - 1;
-        const double* c = ct + 3 * (size_t)q;
-        jt[e] = c[0] * bp[ix(d, ilo, j, k)] + c[1] * (br[ix(d, i, j, k)] - br[ix(d, i, j, km1(d, k))]) -
-                c[2] * bp[ix(d, ihi, j, k)];
-    }
+namespace {
+
+// CTAs of a kernel that hands rows to warps: as many as are resident at once
+template <auto K>
+int row_blocks(const mhd_grid_s* g, long long rows) {
+    return grid_blocks(g, 32 * rows, resident_per_sm<K>());
 }
 
-__global__ void __launch_bounds__(kThreads) k_jp(Dims d, const double* __restrict__ cp,
-                                                 const double* __restrict__ br, const double* __restrict__ bt,
-                                                 double* __restrict__ jp, int walls_zero) {
-    const long long n = (long long)(d.nr + 1) * (d.nt + 1) * d.np;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-        int k;
-        unsigned int q;
-        split_np(d, e, k, q);
-        const int j = (int)(q % (d.nt + 1)), i = (int)(q / (d.nt + 1));
-        if (j == 0 || j == d.nt || (walls_zero && (i == 0 || i == d.nr))) {
-            jp[e] = 0.0;
-            continue;
-        }
-        const int ilo = (i > 0) ? i - 1 : 0, ihi = (i < d.nr) ? i : d.nr - 1;
-        const double* c = cp + 3 * (size_t)q;
-        jp[e] = c[0] * (br[ix(d, i, j - 1, k)] - br[ix(d, i, j, k)]) + c[1] * bt[ixt(d, ihi, j, k)] -
-                c[2] * bt[ixt(d, ilo, j, k)];
-    }
+void current_and_harmonics(mhd_grid_s* g, const double* br, const double* bt, const double* bp, double* bh,
+                           bool walls_zero, cudaStream_t st) {
+    const Dims d = g->d;
+    const long long rows = (bh ? 2ll * d.nr : 0ll) + (long long)d.nr * (d.nt + 1) + (long long)(d.nr + 1) * d.nt +
+                           (long long)(d.nr + 1) * (d.nt + 1);
+    k_current<<<row_blocks<k_current>(g, rows), kThreads, 0, st>>>(d, g->ex.jr, g->ex.jt, g->ex.jp, br, bt, bp, g->er, g->et,
+                                                                   g->ep, g->geo.pcs, bh, walls_zero ? 1 : 0);
 }
+
+}  // namespace
 
 void current_edges(mhd_grid_s* g, const double* br, const double* bt, const double* bp, bool walls_zero,
                    cudaStream_t st) {
-    const Dims d = g->d;
-    if (!st) st = g->stream;
-    k_ring<<<2 * d.nr, kThreads, 0, st>>>(d, bp, g->ring);
-    const long long n = (long long)(d.nr + 1) * (d.nt + 1) * d.np;
-    const int blocks = grid_blocks(g, n, 8);
-    k_jr<<<blocks, kThreads, 0, st>>>(d, g->ex.jr, bt, bp, g->ring, g->er);
-    k_jt<<<blocks, kThreads, 0, st>>>(d, g->ex.jt, br, bp, g->et, walls_zero ? 1 : 0);
-    k_jp<<<blocks, kThreads, 0, st>>>(d, g->ex.jp, br, bt, g->ep, walls_zero ? 1 : 0);
-}
-
-// J at a cell centre from the edge arrays (polar phi edges left out)
-__device__ __forceinline__ void jcentre(const Dims& d, const double* __restrict__ jr, const double* __restrict__ jt,
-                                        const double* __restrict__ jp, int i, int j, int k, double (&o)[3]) {
-    const int kp = kp1(d, k);
-    o[0] = 0.25 * (jr[ixt(d, i, j, k)] + jr[ixt(d, i, j, kp)] + jr[ixt(d, i, j + 1, k)] + jr[ixt(d, i, j + 1, kp)]);
-    o[1] = 0.25 * (jt[ix(d, i, j, k)] + jt[ix(d, i, j, kp)] + jt[ix(d, i + 1, j, k)] + jt[ix(d, i + 1, j, kp)]);
-    if (j == 0) o[2] = 0.5 * (jp[ixt(d, i, 1, k)] + jp[ixt(d, i + 1, 1, k)]);
-    else if (j == d.nt - 1) o[2] = 0.5 * (jp[ixt(d, i, d.nt - 1, k)] + jp[ixt(d, i + 1, d.nt - 1, k)]);
-    else
-        o[2] = 0.25 * (jp[ixt(d, i, j, k)] + jp[ixt(d, i, j + 1, k)] + jp[ixt(d, i + 1, j, k)] +
-                       jp[ixt(d, i + 1, j + 1, k)]);
+    current_and_harmonics(g, br, bt, bp, nullptr, walls_zero, st ? st : g->stream);
 }
 
 // ------------------------------------------------------------------------------------------
 // momentum force
 // ------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreads) k_force(Dims d, Geo G, ExTab X, Vel v, const double* __restrict__ bh,
+// AVG: the mean with the force in b_avg
+template <bool DLT, bool AVG>
+__global__ void __launch_bounds__(kThreads) k_force(Dims d, Geo G, ExTab X, Vel<DLT> v, const double* __restrict__ bh,
                                                     const double* __restrict__ br,
                                                     const double* __restrict__ bt, const double* __restrict__ bp,
                                                     const double* __restrict__ jr, const double* __restrict__ jt,
@@ -285,254 +362,266 @@ __global__ void __launch_bounds__(kThreads) k_force(Dims d, Geo G, ExTab X, Vel 
                                                     double dt_host, const double* __restrict__ b_avg,
                                                     double* __restrict__ b) {
     const double dt = dt_dev ? *dt_dev : dt_host;
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < d.N;
-         c += (long long)gridDim.x * blockDim.x) {
-        int k;
-        unsigned int ij;
-        split_np(d, c, k, ij);
-        const int j = (int)(ij % d.nt), i = (int)(ij / d.nt);
-        double u[3];
-        v.at(c, u);
-        // per-shell reciprocals: 1/d_lo, 1/d_hi, 1/rc, 1/rho, 1/(rc dth)
+    const unsigned int rows = (unsigned int)(d.nr * d.nt);
+    const long long plane = (long long)d.nt * d.np;
+    for (unsigned int ij = first_row(); ij < rows; ij += row_stride()) {
+        const int i = (int)(ij / d.nt), j = (int)(ij - (unsigned int)i * d.nt);
+        const FaceRow F(d, G, bh, br, bt, bp, i, j);
+        const EdgeRow E(d, jr, jt, jp, i, j);
+        // per-shell reciprocals: 1/d_lo, 1/d_hi, 1/rc, 1/rho, 1/(rc dth); 8 J x B is what the sums give
         const double* sh = X.sh + 5 * (size_t)i;
-        // upwind differences of the three components along r, theta, phi
-        double Dr[3], Dt[3], Dp[3];
-        if (u[0] > 0.0) {
-            if (i > 0) {
-                double n[3];
-                v.at(c - (long long)d.nt * d.np, n);
-                const double ih = sh[0];
-                for (int m = 0; m < 3; m++) Dr[m] = (u[m] - n[m]) * ih;
-            } else {
-                const double ih = sh[0];   // Dirichlet mirror ghost at distance 2 (rc_0 - r0)
-                for (int m = 0; m < 3; m++) Dr[m] = (u[m] - (-u[m])) * ih;
+        const double ir_lo = sh[0], ir_hi = sh[1], irc = sh[2], irho8 = 0.125 * sh[3], iht = sh[4];
+        const double ihp = X.ihp[ij], cot = X.cot[j];
+        const double s = (AVG ? 0.5 : 1.0) * (G.rhoV[ij] * dt);
+        // upwind neighbours: none beyond r1 and the poles (the cell itself: difference 0); the Dirichlet mirror
+        // ghost -u at r0
+        const long long c_row = (long long)ij * d.np;
+        const long long r_lo = i > 0 ? -plane : 0, r_hi = i < d.nr - 1 ? plane : 0;
+        const long long t_lo = j > 0 ? -d.np : 0, t_hi = j < d.nt - 1 ? d.np : 0;
+#pragma unroll 1
+        for (int k = threadIdx.x & 31; k < d.np; k += 32) {
+            const long long c = c_row + k;
+            const int kp = kp1(d, k), km = km1(d, k);
+            double u[3], n[3], adv[3], B[3], J[3];
+            v.at(c, u);
+            const bool ur = positive(u[0]), ut = positive(u[1]), up = positive(u[2]);
+            F.twice(k, kp, B);
+            E.four(k, kp, J);
+            {
+                v.at(c + (ur ? r_lo : r_hi), n);
+                if (i == 0 && ur)
+                    for (int m = 0; m < 3; m++) n[m] = -n[m];
+                const double a = fabs(u[0]) * (ur ? ir_lo : ir_hi);
+#pragma unroll
+                for (int m = 0; m < 3; m++) adv[m] = a * (u[m] - n[m]);
             }
-        } else {
-            if (i < d.nr - 1) {
-                double n[3];
-                v.at(c + (long long)d.nt * d.np, n);
-                const double ih = sh[1];
-                for (int m = 0; m < 3; m++) Dr[m] = (n[m] - u[m]) * ih;
-            } else {
-                for (int m = 0; m < 3; m++) Dr[m] = 0.0;
+            {
+                v.at(c + (ut ? t_lo : t_hi), n);
+                const double a = fabs(u[1]) * iht;
+#pragma unroll
+                for (int m = 0; m < 3; m++) adv[m] = fma(a, u[m] - n[m], adv[m]);
             }
+            {
+                v.at(c_row + (up ? km : kp), n);
+                const double a = fabs(u[2]) * ihp;
+#pragma unroll
+                for (int m = 0; m < 3; m++) adv[m] = fma(a, u[m] - n[m], adv[m]);
+            }
+            // spherical curvature terms
+            const double a1 = u[1] * irc, a2 = u[2] * irc, c2 = u[2] * cot;
+            adv[0] = fma(-u[1], a1, fma(-u[2], a2, adv[0]));
+            adv[1] = fma(u[0], a1, fma(-c2, a2, adv[1]));
+            adv[2] = fma(u[0], a2, fma(c2, a1, adv[2]));
+            double f0 = s * fma(J[1] * B[2] - J[2] * B[1], irho8, -adv[0]);
+            double f1 = s * fma(J[2] * B[0] - J[0] * B[2], irho8, -adv[1]);
+            double f2 = s * fma(J[0] * B[1] - J[1] * B[0], irho8, -adv[2]);
+            if constexpr (AVG) {
+                f0 = fma(0.5, b_avg[c], f0);
+                f1 = fma(0.5, b_avg[d.N + c], f1);
+                f2 = fma(0.5, b_avg[2 * d.N + c], f2);
+            }
+            b[c] = f0;
+            b[d.N + c] = f1;
+            b[2 * d.N + c] = f2;
         }
-        const double iht = sh[4];
-        if (u[1] > 0.0) {
-            if (j > 0) {
-                double n[3];
-                v.at(c - d.np, n);
-                for (int m = 0; m < 3; m++) Dt[m] = (u[m] - n[m]) * iht;
-            } else {
-                for (int m = 0; m < 3; m++) Dt[m] = 0.0;
-            }
-        } else {
-            if (j < d.nt - 1) {
-                double n[3];
-                v.at(c + d.np, n);
-                for (int m = 0; m < 3; m++) Dt[m] = (n[m] - u[m]) * iht;
-            } else {
-                for (int m = 0; m < 3; m++) Dt[m] = 0.0;
-            }
-        }
-        const double ihp = X.ihp[ij];
-        {
-            double n[3];
-            if (u[2] > 0.0) {
-                v.at(c - k + km1(d, k), n);
-                for (int m = 0; m < 3; m++) Dp[m] = (u[m] - n[m]) * ihp;
-            } else {
-                v.at(c - k + kp1(d, k), n);
-                for (int m = 0; m < 3; m++) Dp[m] = (n[m] - u[m]) * ihp;
-            }
-        }
-        double adv[3];
-        for (int m = 0; m < 3; m++) adv[m] = u[0] * Dr[m] + u[1] * Dt[m] + u[2] * Dp[m];
-        const double cot = X.cot[j];
-        const double irc = sh[2];
-        adv[0] += -(u[1] * u[1] + u[2] * u[2]) * irc;
-        adv[1] += (u[0] * u[1] - u[2] * u[2] * cot) * irc;
-        adv[2] += (u[0] * u[2] + u[1] * u[2] * cot) * irc;
-        double B[3], J[3];
-        bcentre(d, G, bh, br, bt, bp, i, j, k, B);
-        jcentre(d, jr, jt, jp, i, j, k, J);
-        const double irho = sh[3];
-        const double jxb0 = J[1] * B[2] - J[2] * B[1];
-        const double jxb1 = J[2] * B[0] - J[0] * B[2];
-        const double jxb2 = J[0] * B[1] - J[1] * B[0];
-        const double s = G.rhoV[ij] * dt;
-        double f0 = s * (-adv[0] + jxb0 * irho);
-        double f1 = s * (-adv[1] + jxb1 * irho);
-        double f2 = s * (-adv[2] + jxb2 * irho);
-        if (b_avg) {
-            f0 = 0.5 * (b_avg[c] + f0);
-            f1 = 0.5 * (b_avg[d.N + c] + f1);
-            f2 = 0.5 * (b_avg[2 * d.N + c] + f2);
-        }
-        b[c] = f0;
-        b[d.N + c] = f1;
-        b[2 * d.N + c] = f2;
     }
 }
+
+namespace {
+template <bool DLT, bool AVG>
+void force_launch(mhd_grid_s* g, const Vel<DLT>& v, const double* br, const double* bt, const double* bp,
+                  const double* dt_dev, double dt_host, const double* b_avg, double* b) {
+    k_force<DLT, AVG><<<row_blocks<k_force<DLT, AVG>>(g, (long long)g->d.nr * g->d.nt), kThreads, 0, g->stream>>>(
+        g->d, g->geo, g->ex, v, g->bharm, br, bt, bp, g->er, g->et, g->ep, dt_dev, dt_host, b_avg, b);
+}
+}  // namespace
 
 void force(mhd_grid_s* g, const double* vr, const double* vt, const double* vp, const double* dlt, double dfac,
            const double* br, const double* bt, const double* bp, const double* dt_dev, double dt_host,
            const double* b_avg, double* b) {
-    current_edges(g, br, bt, bp);
-    bt_harmonics(g, bt);
-    Vel v{vr, vt, vp, dlt, dfac, g->d.N};
-    const int blocks = grid_blocks(g, g->d.N, 8);
-    k_force<<<blocks, kThreads, 0, g->stream>>>(g->d, g->geo, g->ex, v, g->bharm, br, bt, bp, g->er, g->et, g->ep,
-                                                dt_dev, dt_host, b_avg, b);
+    current_and_harmonics(g, br, bt, bp, g->bharm, false, g->stream);
+    const Vel<false> v{vr, vt, vp, nullptr, 0.0, g->d.N};
+    const Vel<true> w{vr, vt, vp, dlt, dfac, g->d.N};
+    if (dlt && b_avg) force_launch<true, true>(g, w, br, bt, bp, dt_dev, dt_host, b_avg, b);
+    else if (dlt) force_launch<true, false>(g, w, br, bt, bp, dt_dev, dt_host, b_avg, b);
+    else if (b_avg) force_launch<false, true>(g, v, br, bt, bp, dt_dev, dt_host, b_avg, b);
+    else force_launch<false, false>(g, v, br, bt, bp, dt_dev, dt_host, b_avg, b);
 }
 
 // ------------------------------------------------------------------------------------------
 // electric field and constrained transport
 // ------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreads) k_ecentre(Dims d, Geo G, Vel v, const double* __restrict__ bh,
+// twice E at the cell centres; ETA: with the resistive part
+template <bool DLT, bool ETA>
+__global__ void __launch_bounds__(kThreads) k_ecentre(Dims d, Geo G, Vel<DLT> v, const double* __restrict__ bh,
                                                       const double* __restrict__ br,
                                                       const double* __restrict__ bt, const double* __restrict__ bp,
                                                       const double* __restrict__ jr, const double* __restrict__ jt,
                                                       const double* __restrict__ jp, double eta,
                                                       double* __restrict__ ec) {
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < d.N;
-         c += (long long)gridDim.x * blockDim.x) {
-        int k;
-        unsigned int ij;
-        split_np(d, c, k, ij);
-        const int j = (int)(ij % d.nt), i = (int)(ij / d.nt);
-        double u[3], B[3];
-        v.at(c, u);
-        bcentre(d, G, bh, br, bt, bp, i, j, k, B);
-        double e0 = -(u[1] * B[2] - u[2] * B[1]);
-        double e1 = -(u[2] * B[0] - u[0] * B[2]);
-        double e2 = -(u[0] * B[1] - u[1] * B[0]);
-        if (eta != 0.0) {
-            double J[3];
-            jcentre(d, jr, jt, jp, i, j, k, J);
-            e0 += eta * J[0];
-            e1 += eta * J[1];
-            e2 += eta * J[2];
-        }
-        ec[c] = e0;
-        ec[d.N + c] = e1;
-        ec[2 * d.N + c] = e2;
-    }
-}
-
-__global__ void __launch_bounds__(kThreads) k_eedges(Dims d, const double* __restrict__ ec,
-                                                     const double* __restrict__ ring, double* __restrict__ er,
-                                                     double* __restrict__ et, double* __restrict__ ep) {
-    const double* Er = ec;
-    const double* Et = ec + d.N;
-    const double* Ep = ec + 2 * d.N;
-    const long long n_r = (long long)d.nr * (d.nt + 1) * d.np;
-    const long long n_t = (long long)(d.nr + 1) * d.nt * d.np;
-    const long long n_p = (long long)(d.nr + 1) * (d.nt + 1) * d.np;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n_r + n_t + n_p;
-         e += (long long)gridDim.x * blockDim.x) {
-        if (e < n_r) {
-            int k;
-            unsigned int q;
-            split_np(d, e, k, q);
-            const int j = (int)(q % (d.nt + 1)), i = (int)(q / (d.nt + 1));
-            double val;
-            if (j == 0) val = ring[i] / d.np;
-            else if (j == d.nt) val = ring[d.nr + i] / d.np;
-            else {
-                const int km = km1(d, k);
-                val = 0.25 * (Er[ix(d, i, j - 1, km)] + Er[ix(d, i, j - 1, k)] + Er[ix(d, i, j, km)] + Er[ix(d, i, j, k)]);
+    const unsigned int rows = (unsigned int)(d.nr * d.nt);
+    const double eta_h = 0.5 * eta;   // of four times J
+    for (unsigned int ij = first_row(); ij < rows; ij += row_stride()) {
+        const int i = (int)(ij / d.nt), j = (int)(ij - (unsigned int)i * d.nt);
+        const FaceRow F(d, G, bh, br, bt, bp, i, j);
+        const EdgeRow E(d, jr, jt, jp, i, j);
+#pragma unroll 2
+        for (int k = threadIdx.x & 31; k < d.np; k += 32) {
+            const long long c = (long long)ij * d.np + k;
+            const int kp = kp1(d, k);
+            double u[3], B[3];
+            v.at(c, u);
+            F.twice(k, kp, B);
+            double e0 = u[2] * B[1] - u[1] * B[2];
+            double e1 = u[0] * B[2] - u[2] * B[0];
+            double e2 = u[1] * B[0] - u[0] * B[1];
+            if constexpr (ETA) {
+                double J[3];
+                E.four(k, kp, J);
+                e0 = fma(eta_h, J[0], e0);
+                e1 = fma(eta_h, J[1], e1);
+                e2 = fma(eta_h, J[2], e2);
             }
-            er[e] = val;
-        } else if (e < n_r + n_t) {
-            const long long f = e - n_r;
-            int k;
-            unsigned int q;
-            split_np(d, f, k, q);
-            const int j = (int)(q % d.nt), i = (int)(q / d.nt);
-            const int km = km1(d, k);
-            double val;
-            if (i == 0) val = 0.0;
-            else if (i == d.nr) val = 0.5 * (Et[ix(d, d.nr - 1, j, km)] + Et[ix(d, d.nr - 1, j, k)]);
-            else
-                val = 0.25 * (Et[ix(d, i - 1, j, km)] + Et[ix(d, i - 1, j, k)] + Et[ix(d, i, j, km)] + Et[ix(d, i, j, k)]);
-            et[f] = val;
-        } else {
-            const long long f = e - n_r - n_t;
-            int k;
-            unsigned int q;
-            split_np(d, f, k, q);
-            const int j = (int)(q % (d.nt + 1)), i = (int)(q / (d.nt + 1));
-            double val;
-            if (j == 0 || j == d.nt || i == 0) val = 0.0;
-            else if (i == d.nr) val = 0.5 * (Ep[ix(d, d.nr - 1, j - 1, k)] + Ep[ix(d, d.nr - 1, j, k)]);
-            else
-                val = 0.25 * (Ep[ix(d, i - 1, j - 1, k)] + Ep[ix(d, i - 1, j, k)] + Ep[ix(d, i, j - 1, k)] +
-                              Ep[ix(d, i, j, k)]);
-            ep[f] = val;
+            ec[c] = e0;
+            ec[d.N + c] = e1;
+            ec[2 * d.N + c] = e2;
         }
     }
 }
 
+// eight times E on the edges, from twice E at the centres (kEdgeScale undoes it)
+constexpr double kEdgeScale = 0.125;
+__global__ void __launch_bounds__(kThreads) k_eedges(Dims d, const double* __restrict__ ec, double* __restrict__ er,
+                                                     double* __restrict__ et, double* __restrict__ ep) {
+    const unsigned int n_r = (unsigned int)(d.nr * (d.nt + 1)), n_t = (unsigned int)((d.nr + 1) * d.nt),
+                       n_p = (unsigned int)((d.nr + 1) * (d.nt + 1));
+    const int np = d.np, lane = threadIdx.x & 31;
+    for (unsigned int w = first_row(); w < n_r + n_t + n_p; w += row_stride()) {
+        if (w < n_r) {
+            const int i = (int)(w / (d.nt + 1)), j = (int)(w - (unsigned int)i * (d.nt + 1));
+            double* out = er + (long long)w * np;
+            if (j == 0 || j == d.nt) {
+                // the polar radial edge: the mean of the polar ring
+                const double* row = ec + ix(d, i, j == 0 ? 0 : d.nt - 1, 0);
+                double s = 0.0;
+                for (int k = lane; k < np; k += 32) s += row[k];
+                s = 4.0 * (warp_sum(s) / np);
+                for (int k = lane; k < np; k += 32) out[k] = s;
+            } else {
+                const double *b = ec + ix(d, i, j, 0), *a = b - np;
+#pragma unroll 4
+                for (int k = lane; k < np; k += 32) {
+                    const int km = km1(d, k);
+                    out[k] = (a[km] + a[k]) + (b[km] + b[k]);
+                }
+            }
+        } else if (w < n_r + n_t) {
+            const unsigned int q = w - n_r;
+            const int i = (int)(q / d.nt), j = (int)(q - (unsigned int)i * d.nt);
+            double* out = et + (long long)q * np;
+            // r0: 0 (line-tied); r1: the mean of the two interior cells
+            const double *a = ec + d.N + ix(d, i > 0 ? i - 1 : 0, j, 0), *b = ec + d.N + ix(d, i < d.nr ? i : d.nr - 1, j, 0);
+#pragma unroll 4
+            for (int k = lane; k < np; k += 32) {
+                const int km = km1(d, k);
+                out[k] = i == 0 ? 0.0 : (a[km] + a[k]) + (b[km] + b[k]);
+            }
+        } else {
+            const unsigned int q = w - n_r - n_t;
+            const int i = (int)(q / (d.nt + 1)), j = (int)(q - (unsigned int)i * (d.nt + 1));
+            double* out = ep + (long long)q * np;
+            if (j == 0 || j == d.nt || i == 0) {
+                for (int k = lane; k < np; k += 32) out[k] = 0.0;
+            } else {
+                const double *a = ec + 2 * d.N + ix(d, i - 1, j, 0), *b = ec + 2 * d.N + ix(d, i < d.nr ? i : d.nr - 1, j, 0);
+#pragma unroll 4
+                for (int k = lane; k < np; k += 32) out[k] = (a[k - np] + a[k]) + (b[k - np] + b[k]);
+            }
+        }
+    }
+}
+
+// B -= scale dt curl_h of the edge arrays
 __global__ void __launch_bounds__(kThreads) k_ct(Dims d, ExTab X, const double* __restrict__ er,
                                                  const double* __restrict__ et, const double* __restrict__ ep,
-                                                 const double* __restrict__ dt_dev, double dt_host,
+                                                 const double* __restrict__ dt_dev, double dt_host, double scale,
                                                  double* __restrict__ br, double* __restrict__ bt,
                                                  double* __restrict__ bp) {
-    const double dt = dt_dev ? *dt_dev : dt_host;
-    const long long n_r = (long long)(d.nr + 1) * d.nt * d.np;
-    const long long n_t = (long long)d.nr * (d.nt + 1) * d.np;
-    const long long n_p = (long long)d.nr * d.nt * d.np;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n_r + n_t + n_p;
-         e += (long long)gridDim.x * blockDim.x) {
-        if (e < n_r) {
-            int k;
-            unsigned int q;
-            split_np(d, e, k, q);
-            const int j = (int)(q % d.nt), i = (int)(q / d.nt);
-            const double* c = X.fr + 3 * (size_t)q;
-            const double circ = c[0] * (et[ix(d, i, j, k)] - et[ix(d, i, j, kp1(d, k))]) +
-                                c[1] * ep[ixt(d, i, j + 1, k)] - c[2] * ep[ixt(d, i, j, k)];
-            br[e] -= dt * circ;
-        } else if (e < n_r + n_t) {
-            const long long f = e - n_r;
-            int k;
-            unsigned int q;
-            split_np(d, f, k, q);
-            const int j = (int)(q % (d.nt + 1)), i = (int)(q / (d.nt + 1));
+    const double dt = scale * (dt_dev ? *dt_dev : dt_host);
+    const unsigned int n_r = (unsigned int)((d.nr + 1) * d.nt), n_t = (unsigned int)(d.nr * (d.nt + 1)),
+                       n_p = (unsigned int)(d.nr * d.nt);
+    const int np = d.np, lane = threadIdx.x & 31;
+    for (unsigned int w = first_row(); w < n_r + n_t + n_p; w += row_stride()) {
+        if (w < n_r) {
+            const int i = (int)(w / d.nt), j = (int)(w - (unsigned int)i * d.nt);
+            const double* c = X.fr + 3 * (size_t)w;
+            const double c0 = c[0], c1 = c[1], c2 = c[2];
+            const double *t = et + ix(d, i, j, 0), *p0 = ep + ixt(d, i, j, 0), *p1 = p0 + np;
+            double* out = br + (long long)w * np;
+#pragma unroll 4
+            for (int k = lane; k < np; k += 32) {
+                const double circ = c0 * (t[k] - t[kp1(d, k)]) + c1 * p1[k] - c2 * p0[k];
+                out[k] -= dt * circ;
+            }
+        } else if (w < n_r + n_t) {
+            const unsigned int q = w - n_r;
+            const int i = (int)(q / (d.nt + 1)), j = (int)(q - (unsigned int)i * (d.nt + 1));
             if (j == 0 || j == d.nt) continue;
             const double* c = X.ft + 3 * (size_t)q;
-            const double circ = c[0] * ep[ixt(d, i, j, k)] + c[1] * (er[ixt(d, i, j, kp1(d, k))] - er[ixt(d, i, j, k)]) -
-                                c[2] * ep[ixt(d, i + 1, j, k)];
-            bt[f] -= dt * circ;
+            const double c0 = c[0], c1 = c[1], c2 = c[2];
+            const double *r = er + ixt(d, i, j, 0), *p0 = ep + ixt(d, i, j, 0), *p1 = ep + ixt(d, i + 1, j, 0);
+            double* out = bt + (long long)q * np;
+#pragma unroll 4
+            for (int k = lane; k < np; k += 32) {
+                const double circ = c0 * p0[k] + c1 * (r[kp1(d, k)] - r[k]) - c2 * p1[k];
+                out[k] -= dt * circ;
+            }
         } else {
-            const long long f = e - n_r - n_t;
-            int k;
-            unsigned int q;
-            split_np(d, f, k, q);
-            const int j = (int)(q % d.nt), i = (int)(q / d.nt);
+            const unsigned int q = w - n_r - n_t;
+            const int i = (int)(q / d.nt), j = (int)(q - (unsigned int)i * d.nt);
             const double* c = X.fp + 3 * (size_t)q;
-            const double circ = c[0] * (er[ixt(d, i, j, k)] - er[ixt(d, i, j + 1, k)]) + c[1] * et[ix(d, i + 1, j, k)] -
-                                c[2] * et[ix(d, i, j, k)];
-            bp[f] -= dt * circ;
+            const double c0 = c[0], c1 = c[1], c2 = c[2];
+            const double *r0 = er + ixt(d, i, j, 0), *r1 = r0 + np, *t0 = et + ix(d, i, j, 0), *t1 = et + ix(d, i + 1, j, 0);
+            double* out = bp + (long long)q * np;
+#pragma unroll 4
+            for (int k = lane; k < np; k += 32) {
+                const double circ = c0 * (r0[k] - r1[k]) + c1 * t1[k] - c2 * t0[k];
+                out[k] -= dt * circ;
+            }
         }
     }
 }
 
-void induction(mhd_grid_s* g, const double* vr, const double* vt, const double* vp, const double* dlt, double dfac,
-               double eta, const double* dt_dev, double dt_host, double* br, double* bt, double* bp) {
+namespace {
+template <bool DLT, bool ETA>
+void ecentre_launch(mhd_grid_s* g, const Vel<DLT>& v, const double* br, const double* bt, const double* bp, double eta) {
+    k_ecentre<DLT, ETA><<<row_blocks<k_ecentre<DLT, ETA>>(g, (long long)g->d.nr * g->d.nt), kThreads, 0, g->stream>>>(
+        g->d, g->geo, v, g->bharm, br, bt, bp, g->er, g->et, g->ep, eta, g->ec);
+}
+void ct_launch(mhd_grid_s* g, const double* dt_dev, double dt_host, double scale, double* br, double* bt, double* bp) {
     const Dims d = g->d;
-    if (eta != 0.0) current_edges(g, br, bt, bp);
-    Vel v{vr, vt, vp, dlt, dfac, d.N};
-    bt_harmonics(g, bt);
-    k_ecentre<<<grid_blocks(g, d.N, 8), kThreads, 0, g->stream>>>(d, g->geo, v, g->bharm, br, bt, bp, g->er, g->et,
-                                                                 g->ep, eta, g->ec);
-    k_ring<<<2 * d.nr, kThreads, 0, g->stream>>>(d, g->ec, g->ring);
-    const long long ne = (long long)d.nr * (d.nt + 1) * d.np + (long long)(d.nr + 1) * d.nt * d.np +
-                         (long long)(d.nr + 1) * (d.nt + 1) * d.np;
-    k_eedges<<<grid_blocks(g, ne, 8), kThreads, 0, g->stream>>>(d, g->ec, g->ring, g->er, g->et, g->ep);
-    k_ct<<<grid_blocks(g, ne, 8), kThreads, 0, g->stream>>>(d, g->ex, g->er, g->et, g->ep, dt_dev, dt_host, br, bt,
-                                                           bp);
+    const long long rows = (long long)(d.nr + 1) * d.nt + (long long)d.nr * (d.nt + 1) + (long long)d.nr * d.nt;
+    k_ct<<<row_blocks<k_ct>(g, rows), kThreads, 0, g->stream>>>(d, g->ex, g->er, g->et, g->ep, dt_dev, dt_host, scale, br, bt,
+                                                                bp);
+}
+}  // namespace
+
+void induction(mhd_grid_s* g, const double* vr, const double* vt, const double* vp, const double* dlt, double dfac,
+               double eta, const double* dt_dev, double dt_host, double* br, double* bt, double* bp, bool current_ready) {
+    const Dims d = g->d;
+    if (!current_ready) {
+        if (eta != 0.0) current_and_harmonics(g, br, bt, bp, g->bharm, false, g->stream);
+        else bt_harmonics(g, bt);
+    }
+    const Vel<false> v{vr, vt, vp, nullptr, 0.0, d.N};
+    const Vel<true> w{vr, vt, vp, dlt, dfac, d.N};
+    if (dlt && eta != 0.0) ecentre_launch<true, true>(g, w, br, bt, bp, eta);
+    else if (dlt) ecentre_launch<true, false>(g, w, br, bt, bp, eta);
+    else if (eta != 0.0) ecentre_launch<false, true>(g, v, br, bt, bp, eta);
+    else ecentre_launch<false, false>(g, v, br, bt, bp, eta);
+    const long long rows = (long long)d.nr * (d.nt + 1) + (long long)(d.nr + 1) * d.nt + (long long)(d.nr + 1) * (d.nt + 1);
+    k_eedges<<<row_blocks<k_eedges>(g, rows), kThreads, 0, g->stream>>>(d, g->ec, g->er, g->et, g->ep);
+    ct_launch(g, dt_dev, dt_host, kEdgeScale, br, bt, bp);
 }
 
 void ring_sums(mhd_grid_s* g, const double* a, cudaStream_t st) {
@@ -540,10 +629,7 @@ void ring_sums(mhd_grid_s* g, const double* a, cudaStream_t st) {
 }
 
 void ct_apply(mhd_grid_s* g, const double* dt_dev, double* br, double* bt, double* bp) {
-    const Dims d = g->d;
-    const long long ne = (long long)d.nr * (d.nt + 1) * d.np + (long long)(d.nr + 1) * d.nt * d.np +
-                         (long long)(d.nr + 1) * (d.nt + 1) * d.np;
-    k_ct<<<grid_blocks(g, ne, 8), kThreads, 0, g->stream>>>(d, g->ex, g->er, g->et, g->ep, dt_dev, 0.0, br, bt, bp);
+    ct_launch(g, dt_dev, 0.0, 1.0, br, bt, bp);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -551,76 +637,65 @@ void ct_apply(mhd_grid_s* g, const double* dt_dev, double* br, double* bt, doubl
 // out[0..3] = magnetic energy, kinetic energy, sum |J_c x B_c| V_c, sum |J_c . B_c| V_c; out[4] =
 // max |div_h B| (net outward flux over the cell volume). B_c and J_c as in the momentum force.
 // ------------------------------------------------------------------------------------------
-__device__ __forceinline__ double cell_volume(const Geo& G, int i, int j) {
-    const double ri = G.r[i], ro = G.r[i + 1];
-    return (ro * ro * ro - ri * ri * ri) / 3.0 * (G.cn[j] - G.cn[j + 1]) * G.dph;
-}
-
-__global__ void __launch_bounds__(kThreads) k_diag_sums(Dims d, Geo G, Vel v, const double* __restrict__ bh,
-                                                        const double* __restrict__ br, const double* __restrict__ bt,
-                                                        const double* __restrict__ bp, const double* __restrict__ jr,
-                                                        const double* __restrict__ jt, const double* __restrict__ jp,
-                                                        unsigned int* count, double* __restrict__ partials,
-                                                        double* __restrict__ out) {
-    double em = 0.0, ek = 0.0, jxb = 0.0, jdb = 0.0;
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < d.N;
-         c += (long long)gridDim.x * blockDim.x) {
-        int k;
-        unsigned int ij;
-        split_np(d, c, k, ij);
-        const int j = (int)(ij % d.nt), i = (int)(ij / d.nt);
-        double u[3], B[3], J[3];
-        v.at(c, u);
-        bcentre(d, G, bh, br, bt, bp, i, j, k, B);
-        jcentre(d, jr, jt, jp, i, j, k, J);
-        const double V = cell_volume(G, i, j);
-        const double x0 = J[1] * B[2] - J[2] * B[1], x1 = J[2] * B[0] - J[0] * B[2], x2 = J[0] * B[1] - J[1] * B[0];
-        em += 0.5 * (B[0] * B[0] + B[1] * B[1] + B[2] * B[2]) * V;
-        ek += 0.5 * G.rho[i] * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]) * V;
-        jxb += sqrt(x0 * x0 + x1 * x1 + x2 * x2) * V;
-        jdb += fabs(J[0] * B[0] + J[1] * B[1] + J[2] * B[2]) * V;
+__global__ void __launch_bounds__(kThreads) k_diag(Dims d, Geo G, ExTab X, Vel<false> v, const double* __restrict__ bh,
+                                                   const double* __restrict__ br, const double* __restrict__ bt,
+                                                   const double* __restrict__ bp, const double* __restrict__ jr,
+                                                   const double* __restrict__ jt, const double* __restrict__ jp,
+                                                   unsigned int* count, unsigned int* count_max,
+                                                   double* __restrict__ partials, double* __restrict__ out) {
+    double em = 0.0, ek = 0.0, jxb = 0.0, jdb = 0.0, dmax = 0.0;
+    const unsigned int rows = (unsigned int)(d.nr * d.nt);
+    for (unsigned int ij = first_row(); ij < rows; ij += row_stride()) {
+        const int i = (int)(ij / d.nt), j = (int)(ij - (unsigned int)i * d.nt);
+        const FaceRow F(d, G, bh, br, bt, bp, i, j);
+        const EdgeRow E(d, jr, jt, jp, i, j);
+        const double *t0 = bt + ixt(d, i, j, 0), *t1 = t0 + d.np;
+        // face areas and volume of the row's cells
+        const double ri = G.r[i], ro = G.r[i + 1];
+        const double ring = 0.5 * (ro * ro - ri * ri), band = (G.cn[j] - G.cn[j + 1]) * G.dph;
+        const double ari = ri * ri * band, aro = ro * ro * band;
+        const double atj = G.sn[j] * ring * G.dph, atj1 = G.sn[j + 1] * ring * G.dph;
+        const double ap = ring * G.dth, V = G.rhoV[ij] * X.sh[5 * (size_t)i + 3];
+        double sb = 0.0, su = 0.0, sx = 0.0, sd = 0.0;
+        long long mf = 0;
+#pragma unroll 1
+        for (int k = threadIdx.x & 31; k < d.np; k += 32) {
+            const int kp = kp1(d, k);
+            double u[3], B[3], J[3];
+            v.at((long long)ij * d.np + k, u);
+            F.twice(k, kp, B);
+            E.four(k, kp, J);
+            const double x0 = J[1] * B[2] - J[2] * B[1], x1 = J[2] * B[0] - J[0] * B[2], x2 = J[0] * B[1] - J[1] * B[0];
+            sb = fma(B[0], B[0], fma(B[1], B[1], fma(B[2], B[2], sb)));
+            su = fma(u[0], u[0], fma(u[1], u[1], fma(u[2], u[2], su)));
+            sx += sqrt(x0 * x0 + x1 * x1 + x2 * x2);
+            sd += fabs(J[0] * B[0] + J[1] * B[1] + J[2] * B[2]);
+            max_abs(mf, F.r1[k] * aro - F.r0[k] * ari + t1[k] * atj1 - t0[k] * atj + (F.p0[kp] - F.p0[k]) * ap);
+        }
+        // the sums hold 4 B^2 and 8 times the products of J and B
+        em = fma(0.125 * V, sb, em);
+        ek = fma(0.5 * G.rho[i] * V, su, ek);
+        jxb = fma(0.125 * V, sx, jxb);
+        jdb = fma(0.125 * V, sd, jdb);
+        dmax = fmax(dmax, __longlong_as_double(mf) / V);
     }
     double val[4] = {em, ek, jxb, jdb}, o[4];
     if (reduce_last<4>(val, partials, count, o) && threadIdx.x == 0)
         for (int q = 0; q < 4; q++) out[q] = o[q];
-}
-
-__global__ void __launch_bounds__(kThreads) k_diag_divmax(Dims d, Geo G, const double* __restrict__ br,
-                                                          const double* __restrict__ bt,
-                                                          const double* __restrict__ bp, unsigned int* count,
-                                                          double* __restrict__ partials, double* __restrict__ out) {
-    double m = 0.0;
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < d.N;
-         c += (long long)gridDim.x * blockDim.x) {
-        int k;
-        unsigned int ij;
-        split_np(d, c, k, ij);
-        const int j = (int)(ij % d.nt), i = (int)(ij / d.nt);
-        const double ri = G.r[i], ro = G.r[i + 1];
-        const double ring = 0.5 * (ro * ro - ri * ri);
-        const double band = G.cn[j] - G.cn[j + 1];
-        const double ari = ri * ri * band * G.dph, aro = ro * ro * band * G.dph;
-        const double atj = G.sn[j] * ring * G.dph, atj1 = G.sn[j + 1] * ring * G.dph;
-        const double ap = ring * G.dth;
-        const double flux = br[ix(d, i + 1, j, k)] * aro - br[ix(d, i, j, k)] * ari + bt[ixt(d, i, j + 1, k)] * atj1 -
-                            bt[ixt(d, i, j, k)] * atj + bp[ix(d, i, j, kp1(d, k))] * ap - bp[ix(d, i, j, k)] * ap;
-        m = fmax(m, fabs(flux) / cell_volume(G, i, j));
-    }
-    double val[1] = {m}, o[1];
-    if (reduce_last<1, OpMax>(val, partials, count, o) && threadIdx.x == 0) out[0] = o[0];
+    double vm[1] = {dmax}, om[1];
+    if (reduce_last<1, OpMax>(vm, partials + 4 * (size_t)gridDim.x, count_max, om) && threadIdx.x == 0) out[4] = om[0];
 }
 
 // out (device, 5 doubles): the diagnostics of the fields; enqueued on the grid's stream
 void diagnostics(mhd_grid_s* g, const double* vr, const double* vt, const double* vp, const double* br,
                  const double* bt, const double* bp, double* out) {
     const Dims d = g->d;
-    current_edges(g, br, bt, bp);
-    bt_harmonics(g, bt);
-    Vel v{vr, vt, vp, nullptr, 0.0, d.N};
-    const int blocks = grid_blocks(g, d.N, 8);
-    k_diag_sums<<<blocks, kThreads, 0, g->stream>>>(d, g->geo, v, g->bharm, br, bt, bp, g->er, g->et, g->ep,
-                                                    &g->ss->count, g->partials, out);
-    k_diag_divmax<<<blocks, kThreads, 0, g->stream>>>(d, g->geo, br, bt, bp, &g->ss->count, g->partials, out + 4);
+    current_and_harmonics(g, br, bt, bp, g->bharm, false, g->stream);
+    const Vel<false> v{vr, vt, vp, nullptr, 0.0, d.N};
+    // two reductions: 5 partials a CTA in the array's 4 kMaxBlocks, and a ticket each (the solver's is idle here)
+    const int blocks = std::min(row_blocks<k_diag>(g, (long long)d.nr * d.nt), kMaxBlocks * kPartialsPerBlock / 5);
+    k_diag<<<blocks, kThreads, 0, g->stream>>>(d, g->geo, g->ex, v, g->bharm, br, bt, bp, g->er, g->et, g->ep,
+                                               &g->ss->count, &g->sc->count, g->partials, out);
 }
 
 // ------------------------------------------------------------------------------------------

@@ -365,9 +365,10 @@ void ct_apply(mhd_grid_s* g, const double* dt_dev, double* br, double* bt, doubl
 void force(mhd_grid_s* g, const double* vr, const double* vt, const double* vp,
            const double* dlt, double dfac, const double* br, const double* bt, const double* bp,
            const double* dt_dev, double dt_host, const double* b_avg, double* b);
+// current_ready: force() has just formed J and the harmonics of this B, nothing has changed them since
 void induction(mhd_grid_s* g, const double* vr, const double* vt, const double* vp,
                const double* dlt, double dfac, double eta, const double* dt_dev, double dt_host,
-               double* br, double* bt, double* bp);
+               double* br, double* bt, double* bp, bool current_ready = false);
 void vstar_rhs(mhd_grid_s* g, double* vr, double* vt, double* vp, const double* dlt, double* b);
 void diagnostics(mhd_grid_s* g, const double* vr, const double* vt, const double* vp, const double* br,
                  const double* bt, const double* bp, double* out);

@@ -117,7 +117,7 @@ extern "C" mhd_status_t mhd_step(mhd_grid_t g, const mhd_params_t* p, mhd_fields
     double rr_res = 0.0;
     ps = prof_begin(g, g->stream, MHD_KERNEL_INDUCTION);
     induction(g, f->vr, f->vt, f->vp, g->dlt, 0.5, p->resistivity_implicit ? 0.0 : p->eta, dt_dev, 0.0, f->br,
-              f->bt, f->bp);
+              f->bt, f->bp, true);
     prof_end(g, g->stream, ps);
     if (p->resistivity_implicit) {
         // resistive part implicit on the faces: W (B + dt eta curl_h J(B)) = W B*
