@@ -407,7 +407,7 @@ mhd_status_t persist_iterate(mhd_grid_s* g, bool fp32, int nc);
 
 // PCG (pcg.cu). alpha is read from device memory (alpha_dev) so a step never syncs on it.
 void build_tables(mhd_grid_s* g, const double* alpha_dev, bool fp32);
-void apply_operator(mhd_grid_s* g, const double* alpha_dev, int nc, const double* p, double* q);
+void apply_operator(mhd_grid_s* g, double alpha, int nc, const double* p, double* q);
 mhd_status_t solve(mhd_grid_s* g, const double* alpha_dev, int nc, const double* b, double* x,
                    const double* x0, const mhd_params_t* prm, int* iters, int* outer,
                    double* relres);

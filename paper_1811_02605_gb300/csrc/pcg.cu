@@ -1172,32 +1172,45 @@ __global__ void k_correct(Dims d, int nc, double* __restrict__ x, const float* _
     if (blockIdx.x == 0 && threadIdx.x == 0) sc->outer += 1;
 }
 
-// q = M p (unscaled FP64), for the C-ABI operator call
-__global__ void __launch_bounds__(kThreads) k_apply64(Dims d, int nc, const double* __restrict__ p,
-                                                      double* __restrict__ q, OpTab64u tu) {
+// q = M_alpha p (unscaled FP64), for the C-ABI operator call, in one launch: a CTA takes kApplyRows rows (i, j), its
+// first threads form their coefficients (as k_tables does), and its warps take (row, component) items. Forming all
+// tables first, and alpha on the device before that, made three dependent launches of what is 2.4 us of FP64
+// instructions at 32x32x64, 3 components: 16.4 -> 8.2 us a call.
+constexpr int kApplyRows = 8;
+__global__ void __launch_bounds__(kThreads) k_apply64(Dims d, Geo G, double a, int nc, const double* __restrict__ p,
+                                                      double* __restrict__ q) {
+    __shared__ double co[kApplyRows][6];
     const int nt = d.nt;
-    const unsigned int G = (unsigned int)(d.N / 2);
+    const int row0 = blockIdx.x * kApplyRows, n = min(kApplyRows, d.nr * nt - row0);
     const long long plane = (long long)nt * d.np;
-    for (unsigned int g = blockIdx.x * blockDim.x + threadIdx.x; g < G; g += gridDim.x * blockDim.x) {
-        const Cell c = decompose<2>(d, g);
-        const double dg = tu.dg[c.ij];
-        const double wl = tu.awr[c.i * nt + c.j], wh = tu.awr[(c.i + 1) * nt + c.j];
-        const double tl = tu.awt[c.i * (nt + 1) + c.j], th = tu.awt[c.i * (nt + 1) + c.j + 1];
-        const double wp = tu.awp[c.ij];
-        for (int k = 0; k < nc; k++) {
-            const double* u = p + k * d.N;
-            double xv[2], n[2], mx[2];
-            ldv<double, 2>(u + c.base, xv);
-            const long long row = c.base - c.k0;
-            const int km = (c.k0 == 0) ? d.np - 1 : c.k0 - 1;
-            const int kp = (c.k0 + 2 == d.np) ? 0 : c.k0 + 2;
-            mx[0] = dg * xv[0] - wp * (u[row + km] + xv[1]);
-            mx[1] = dg * xv[1] - wp * (xv[0] + u[row + kp]);
-            if (c.i > 0) { ldv<double, 2>(u + c.base - plane, n); mx[0] -= wl * n[0]; mx[1] -= wl * n[1]; }
-            if (c.i < d.nr - 1) { ldv<double, 2>(u + c.base + plane, n); mx[0] -= wh * n[0]; mx[1] -= wh * n[1]; }
-            if (c.j > 0) { ldv<double, 2>(u + c.base - d.np, n); mx[0] -= tl * n[0]; mx[1] -= tl * n[1]; }
-            if (c.j < nt - 1) { ldv<double, 2>(u + c.base + d.np, n); mx[0] -= th * n[0]; mx[1] -= th * n[1]; }
-            stv<double, 2>(q + k * d.N + c.base, mx);
+    if ((int)threadIdx.x < n) {
+        const int ij = row0 + threadIdx.x, i = ij / nt, j = ij - i * nt;
+        double* c = co[threadIdx.x];
+        c[0] = diag_at(G, nt, a, i, j);
+        c[1] = a * G.wr[i * nt + j];
+        c[2] = a * G.wr[(i + 1) * nt + j];
+        c[3] = a * G.wt[i * (nt + 1) + j];
+        c[4] = a * G.wt[i * (nt + 1) + j + 1];
+        c[5] = a * G.wp[ij];
+    }
+    __syncthreads();
+    for (int item = threadIdx.x >> 5; item < n * nc; item += kThreads / 32) {
+        const int k = item / n, rl = item - k * n, ij = row0 + rl, i = ij / nt, j = ij - i * nt;
+        const double dg = co[rl][0], wl = co[rl][1], wh = co[rl][2], tl = co[rl][3], th = co[rl][4], wp = co[rl][5];
+        const long long row = k * d.N + (long long)ij * d.np;
+        const double* u = p + row;
+        for (int k0 = 2 * (threadIdx.x & 31); k0 < d.np; k0 += 64) {
+            double xv[2], n2[2], mx[2];
+            ldv<double, 2>(u + k0, xv);
+            const int km = (k0 == 0) ? d.np - 1 : k0 - 1;
+            const int kp = (k0 + 2 == d.np) ? 0 : k0 + 2;
+            mx[0] = dg * xv[0] - wp * (u[km] + xv[1]);
+            mx[1] = dg * xv[1] - wp * (xv[0] + u[kp]);
+            if (i > 0) { ldv<double, 2>(u + k0 - plane, n2); mx[0] -= wl * n2[0]; mx[1] -= wl * n2[1]; }
+            if (i < d.nr - 1) { ldv<double, 2>(u + k0 + plane, n2); mx[0] -= wh * n2[0]; mx[1] -= wh * n2[1]; }
+            if (j > 0) { ldv<double, 2>(u + k0 - d.np, n2); mx[0] -= tl * n2[0]; mx[1] -= tl * n2[1]; }
+            if (j < nt - 1) { ldv<double, 2>(u + k0 + d.np, n2); mx[0] -= th * n2[0]; mx[1] -= th * n2[1]; }
+            stv<double, 2>(q + row + k0, mx);
         }
     }
 }
@@ -1211,10 +1224,9 @@ void build_tables(mhd_grid_s* g, const double* alpha_dev, bool fp32) {
                                                       fp32 ? 1 : 0, reinterpret_cast<float4*>(g->row32));
 }
 
-void apply_operator(mhd_grid_s* g, const double* alpha_dev, int nc, const double* p, double* q) {
-    build_tables(g, alpha_dev, false);
-    const int blocks = grid_blocks(g, g->d.N / 2, 8);
-    k_apply64<<<blocks, kThreads, 0, g->stream>>>(g->d, nc, p, q, g->tu);
+void apply_operator(mhd_grid_s* g, double alpha, int nc, const double* p, double* q) {
+    const int rows = g->d.nr * g->d.nt;
+    k_apply64<<<(rows + kApplyRows - 1) / kApplyRows, kThreads, 0, g->stream>>>(g->d, g->geo, alpha, nc, p, q);
 }
 
 namespace {

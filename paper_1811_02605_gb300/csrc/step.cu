@@ -181,8 +181,7 @@ extern "C" mhd_status_t mhd_apply_operator(mhd_grid_t g, double alpha, int ncomp
     if (ncomp < 1 || ncomp > 3 || !p || !q || p == q)
         return set_error(g, MHD_ERR_ARG, "mhd_apply_operator: need 1 <= ncomp <= 3, distinct non-null p, q");
     if (!(alpha >= 0.0)) return set_error(g, MHD_ERR_ARG, "mhd_apply_operator: alpha must be >= 0");
-    k_set_alpha<<<1, 1, 0, g->stream>>>(g->ss, alpha);
-    apply_operator(g, &g->ss->alpha_user, ncomp, p, q);
+    apply_operator(g, alpha, ncomp, p, q);
     return check_cuda(g, "mhd_apply_operator");
 }
 
