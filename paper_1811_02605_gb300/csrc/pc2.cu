@@ -11,8 +11,8 @@
 // with PC2 on M, in exact arithmetic. On a line of A~: m = 1 and w = the scaled phi coefficient.
 //
 // z = P^-1 r is a forward and a backward substitution along each line, both first-order linear
-// recurrences u_k = a_k u_{k-1} + b_k, which one warp per line evaluates as an affine scan: each
-// lane composes the maps of its segment of ceil(np/32) elements, a five-step shuffle scan composes
+// recurrences u_k = a_k u_{k-1} + b_k, which the lanes of a line evaluate as an affine scan: each
+// lane composes the maps of its segment, a shuffle scan composes
 // the segments, and each lane replays its segment from the value entering it. The multipliers
 // (a_k = w / dt_k) do not depend on the component, so their segment products and the scan's
 // per-step multipliers are formed once per line and reused by the three components; per
@@ -24,7 +24,9 @@
 // products, are formed in FP32 and summed over lines in FP64),
 // with the FP64 outer residual of the reliable-update scheme followed by one preconditioner pass
 // that recomputes z and <r, z> for the replaced residual.
+#include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "mhd_internal.cuh"
 #include "reduce.cuh"
@@ -37,13 +39,18 @@ constexpr unsigned kFull = 0xffffffffu;
 
 enum { kIter = 0, kInit = 1, kReliable = 2 };
 
+// launch shape of the line kernel: lanes and elements per lane of a line (0: the generic kernel), warps per CTA,
+// dynamic shared memory, CTAs
+struct LineShape {
+    int lanes, seg, warps, blocks;
+    size_t smem;
+};
+
 struct Pc2Work {
     double* idt;      // [N] 1 / dt of the scaled lines (FP64)
     float* idt32;     // [N] the same in FP32
     float* z32;       // [3N] z~ of the FP32 iteration (the p double buffer keeps both halves for p~)
-    int warps[2];     // warps per CTA of the line kernel, [0] FP64, [1] FP32
-    size_t smem[2];   // its dynamic shared memory
-    int line_blocks[2];
+    LineShape shape[2];   // of the line kernel, [0] FP64, [1] FP32
 };
 
 // 1 / dt along every phi line of A~ (one thread per line); a non-positive pivot flags a breakdown
@@ -77,22 +84,57 @@ __host__ __device__ inline int padded_len(int np) {
     return np + (np + S - 1) / S;
 }
 
+// end of a line kernel: <r~, z~> and ||r||^2 over the grid; the last CTA does the scalar recurrence of its mode
+template <typename T, int MODE>
+__device__ __forceinline__ void line_finish(double a_rz, double a_rr, PcgScalars* sc, double* __restrict__ partials,
+                                            int restart) {
+    double val[2] = {a_rz, a_rr}, out[2];
+    if (reduce_last<2>(val, partials, &sc->count, out) && threadIdx.x == 0) {
+        const double rz = out[0], rr = out[1];
+        if (MODE == kReliable) {
+            const bool keep = !restart && sc->rho_prev > 0.0 && rz <= 4.0 * sc->rho;
+            sc->beta = keep ? rz / sc->rho_prev : 0.0;
+            sc->rho = rz;
+            sc->rr = rr;
+            if (!isfinite(rz) || !isfinite(rr)) {
+                sc->done = 3;
+                sc->outer_done = 3;
+            } else if (!(rz > 0.0)) {
+                sc->done = 4;
+            }
+            return;
+        }
+        if (MODE == kInit) {
+            sc->beta = 0.0;
+        } else {
+            sc->iter += 1;
+            sc->total_iter += 1;
+            sc->beta = rz / sc->rho;
+            sc->rho_prev = sc->rho;
+            sc->ax = sc->alpha;   // x~ += alpha p~ is left to the next p update
+        }
+        sc->rho = rz;
+        sc->rr = rr;
+        if (!isfinite(rz) || !isfinite(rr)) sc->done = 3;
+        else if (sc->bb == 0.0 || sqrt(rr) <= sc->tol * sqrt(sc->bb)) sc->done = 1;
+        else if (sc->iter >= sc->max_iter) sc->done = 2;
+        else if (!(rz > 0.0)) sc->done = 4;
+    }
+}
+
 // One warp per phi line of the scaled system.
-//   kIter:     x~ += alpha p~ (FP64), r~ -= alpha q~; z~ = P~^-1 r~; <r~, z~> and
+//   kIter:     r~ -= alpha q~; z~ = P~^-1 r~; <r~, z~> and
 //              ||r||^2 = sum dg r~^2; last CTA: beta = rho_new / rho, stop test, iteration count.
-//              FP32 defers the x update: alpha is handed on in sc->ax, and the p update of the
-//              next iteration (or the correction kernel when the inner solve stops here) adds
-//              alpha p~ to x~.
+//              alpha is handed on in sc->ax, and the p update of the next iteration (or the kernel
+//              that takes x~ over when the solve stops here) adds alpha p~ to x~.
 //   kInit:     z~ = P~^-1 r~, p~ = z~; last CTA: rho, beta = 0, stop test (after the FP64 set-up).
 //   kReliable: z~ = P~^-1 r~ for the replaced residual; last CTA: rho = <r~, z~>, and the
 //              recurrence continues (beta = rho / rho_prev) while rho stays within 4x of the
 //              recursive one, else restarts (beta = 0); the stop flags are the outer kernel's.
-// SEG > 0: np = 32 SEG exactly, so the segment length is a compile-time constant: the segment
-// loops unroll (their shared-memory loads issue together) and the bounds tests vanish (the first
-// and last elements of the line are lane 0's first and lane 31's last). SEG = 0: any np.
-template <typename T, int NC, int MODE, int SEG>
-__global__ void __launch_bounds__(kThreads) k_pc2_line(Dims d, OpTab<T> t, const double* __restrict__ dgv,
-                                                       const T* __restrict__ idt, T* __restrict__ x,
+// This is the form for lines longer than the register kernel (k_pc2_seg) takes: the segments are in shared memory.
+template <typename T, int MODE>
+__global__ void __launch_bounds__(kThreads) k_pc2_line(Dims d, int nc, OpTab<T> t, const double* __restrict__ dgv,
+                                                       const T* __restrict__ idt,
                                                        T* __restrict__ p, T* __restrict__ r,
                                                        const T* __restrict__ q, T* __restrict__ z,
                                                        PcgScalars* sc, double* __restrict__ partials, int restart) {
@@ -102,7 +144,7 @@ __global__ void __launch_bounds__(kThreads) k_pc2_line(Dims d, OpTab<T> t, const
     const int warps = blockDim.x >> 5;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int np = d.np;
-    const int S = SEG > 0 ? SEG : (np + 31) >> 5;
+    const int S = (np + 31) >> 5;
     const int P = padded_len(np);
     T* ib = smem + (size_t)warp * 3 * P;   // 1 / dt_k
     T* gb = ib + P;                        // w / dt_k
@@ -111,14 +153,10 @@ __global__ void __launch_bounds__(kThreads) k_pc2_line(Dims d, OpTab<T> t, const
     const T zero = T(0);
     const int k0 = lane * S;
     const int s0 = lane * (S + 1);         // element k0 + t of this lane's segment sits at s0 + t
-    constexpr bool exact = SEG > 0;
-    // FP32: x~ += alpha p~ moves to the next p update, which leaves this HBM-bound kernel 52 instead
-    // of 88 B per cell; FP64: the kernel is bound by its FP64 instructions and the x update stays here
-    constexpr bool kDeferX = sizeof(T) == 4;
     // element k0 + t is in the line / is its first / is its last element
-#define IN_LINE(tt) (exact || k0 + (tt) < np)
+#define IN_LINE(tt) (k0 + (tt) < np)
 #define FIRST(tt) ((tt) == 0 && lane == 0)
-#define LAST(tt) (exact ? ((tt) == S - 1 && lane == 31) : (k0 + (tt) == np - 1))
+#define LAST(tt) (k0 + (tt) == np - 1)
     double a_rz = 0.0, a_rr = 0.0;   // per-line partials (in T) are added here in FP64
     const int nl = d.nr * d.nt;
     for (int line = blockIdx.x * warps + warp; line < nl; line += gridDim.x * warps) {
@@ -152,12 +190,11 @@ __global__ void __launch_bounds__(kThreads) k_pc2_line(Dims d, OpTab<T> t, const
         }
         T line_rz = zero, line_rr = zero;
 #pragma unroll 1
-        for (int c = 0; c < NC; c++) {
+        for (int c = 0; c < nc; c++) {
             const long long off = c * d.N + base;
             for (int k = lane; k < np; k += 32) {
                 T rv = r[off + k];
                 if (MODE == kIter) {
-                    if constexpr (!kDeferX) x[off + k] = fma(al, p[off + k], x[off + k]);
                     rv = fma(-al, q[off + k], rv);
                     r[off + k] = rv;
                 }
@@ -242,38 +279,264 @@ __global__ void __launch_bounds__(kThreads) k_pc2_line(Dims d, OpTab<T> t, const
 #undef IN_LINE
 #undef FIRST
 #undef LAST
-    double val[2] = {a_rz, a_rr}, out[2];
-    if (reduce_last<2>(val, partials, &sc->count, out) && threadIdx.x == 0) {
-        const double rz = out[0], rr = out[1];
-        if (MODE == kReliable) {
-            const bool keep = !restart && sc->rho_prev > 0.0 && rz <= 4.0 * sc->rho;
-            sc->beta = keep ? rz / sc->rho_prev : 0.0;
-            sc->rho = rz;
-            sc->rr = rr;
-            if (!isfinite(rz) || !isfinite(rr)) {
-                sc->done = 3;
-                sc->outer_done = 3;
-            } else if (!(rz > 0.0)) {
-                sc->done = 4;
-            }
-            return;
-        }
-        if (MODE == kInit) {
-            sc->beta = 0.0;
+    line_finish<T, MODE>(a_rz, a_rr, sc, partials, restart);
+}
+
+constexpr int kSegMax = 24;   // most elements of a lane in the register kernel
+
+__device__ __forceinline__ void copy_async(void* dst, const void* src, int bytes16) {
+    const unsigned int d = (unsigned int)__cvta_generic_to_shared(dst);
+    if (bytes16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
+}
+
+// V consecutive elements as one access (8 or 16 bytes, aligned to their size)
+template <typename T, int V>
+struct alignas(V * sizeof(T)) Pack {
+    T v[V];
+};
+template <typename T, int V>
+__device__ __forceinline__ Pack<T, V> load(const T* p) {
+    return *reinterpret_cast<const Pack<T, V>*>(p);
+}
+template <typename T, int V>
+__device__ __forceinline__ void store(T* p, const Pack<T, V>& a) {
+    *reinterpret_cast<Pack<T, V>*>(p) = a;
+}
+// f(integral_constant i) for the same i in [LO, HI) in all lanes, by bisection (registers cannot be indexed)
+template <int HI, int LO = 0, typename F>
+__device__ __forceinline__ void one_of(int i, F f) {
+    if constexpr (HI - LO == 1) f(std::integral_constant<int, LO>());
+    else if (i < (LO + HI) / 2) one_of<(LO + HI) / 2, LO>(i, f);
+    else one_of<HI, (LO + HI) / 2>(i, f);
+}
+// distance of two segments in shared memory: an odd number of 16-byte units, so that 16-byte accesses by segment
+// meet no bank conflicts
+template <typename T, int S>
+constexpr int kSegDist = (S * sizeof(T)) % 32 == 0 ? S + 16 / (int)sizeof(T) : S;
+
+// The same line solve with each lane's segment in registers. L lanes hold a line in segments of S elements (the last
+// ones shorter or empty, their missing elements zero), so a warp takes 32 / L consecutive lines, which are contiguous
+// in memory: loads and stores are coalesced, and one exchange through shared memory in either direction brings an
+// element to its lane and back, 16 bytes at a time. 1 / dt and the multipliers stay in registers for the
+// components. What a warp reads next is copied ahead (cp.async) while it solves: the registers allow 12 (FP64) to 20
+// warps per SM, too few to hide the loads' latency otherwise (96x96x192, FP64: 176 us a call without the copies, with
+// them 121).
+// In FP64 the floor is the FP64 instructions, each taking a scheduler's pipe 64 cycles: five
+// per element for the two recurrences (scale, compose and replay forwards, the same backwards), three for r~ and
+// the sums, and per line and lane two for the multipliers and four per scan step. Short scans and long segments are
+// the cheap ones, so L is the least that 16 elements a lane allow. In FP32 the floor is HBM; L is 32, which keeps the
+// FP32 partial sums short. x~ += alpha p~ is left to the next p update, which reads p~ anyway.
+// us per call, 3 components, the shared-memory form / this: FP64 64x64x128 65 / 43, 96x96x192 166 / 114; FP32
+// 256x256x512 334 / 295 (at 6.8 TB/s: 257).
+template <typename T, int S, int MODE>
+__global__ void __launch_bounds__(128, sizeof(T) == 8 ? (S > 16 ? 2 : 3) : (S > 16 ? 4 : 5))
+    k_pc2_seg(Dims d, int nc, int lanes, OpTab<T> t, const double* __restrict__ dgv, const T* __restrict__ idt,
+              T* __restrict__ p, T* __restrict__ r, const T* __restrict__ q, T* __restrict__ z, PcgScalars* sc,
+              double* __restrict__ partials, int restart) {
+    if (sc->done) return;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int L = sizeof(T) == 4 ? 32 : lanes;
+    const int warps = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int np = d.np, nl = d.nr * d.nt, lpw = 32 / L;
+    constexpr int D = kSegDist<T, S>, W = 16 / (int)sizeof(T);
+    T* const sr = reinterpret_cast<T*>(smem_raw) + (size_t)warp * 32 * (3 * S + D);   // r~, q~ and 1 / dt copied ahead
+    T* const sq = sr + 32 * S;
+    T* const si = sq + 32 * S;
+    T* const wb = si + 32 * S;                                                        // r~, then z~, by segments
+    const T al = (MODE == kIter) ? (T)sc->alpha : T(0);
+    const T zero = T(0);
+    const int ln = lane / L, gl = lane - ln * L;
+    T* const seg = wb + lane * D;
+    const int lastl = (np - 1) / S, lastt = (np - 1) - lastl * S;
+    // element e of the warp's lines -> its place by segments (quotient exact for e < 32 kSegMax)
+    const unsigned int m_np = (1u << 20) / np + 1;
+    auto place = [&](unsigned int e) {
+        const unsigned int line = sizeof(T) == 4 ? 0u : (e * m_np) >> 20, k = e - line * np;
+        return line * (L * D) + k + k / S * (D - S);
+    };
+    // f(e, place of e) for the lane's packs of V elements; where a pass of the warp over 32 V elements is a whole
+    // number of segments of one line, the places follow from the first
+    auto packs = [&](auto width, int l0, int E, auto f) {
+        constexpr int V = decltype(width)::value, n = S / V;
+        if constexpr (sizeof(T) == 4 && (32 * V) % S == 0) {
+            const int e0 = V * l0, p0 = (int)place(e0);
+#pragma unroll
+            for (int m = 0; m < n; m++)
+                if (e0 + 32 * V * m < E) f(e0 + 32 * V * m, p0 + m * (32 * V / S) * D);
         } else {
-            sc->iter += 1;
-            sc->total_iter += 1;
-            sc->beta = rz / sc->rho;
-            sc->rho_prev = sc->rho;
-            if (kDeferX) sc->ax = sc->alpha;   // x~ += alpha p~ is left to the next p update
+#pragma unroll 2
+            for (int e = V * l0; e < E; e += 32 * V) f(e, (int)place(e));
         }
-        sc->rho = rz;
-        sc->rr = rr;
-        if (!isfinite(rz) || !isfinite(rr)) sc->done = 3;
-        else if (sc->bb == 0.0 || sqrt(rr) <= sc->tol * sqrt(sc->bb)) sc->done = 1;
-        else if (sc->iter >= sc->max_iter) sc->done = 2;
-        else if (!(rz > 0.0)) sc->done = 4;
+    };
+    const int step = gridDim.x * warps * lpw;
+    // rows of np elements start on 16 bytes, except in FP32 when np is not a multiple of 4 (np is even)
+    const int b16 = (np * (int)sizeof(T)) % 16 == 0, per = (b16 ? 16 : 8) / (int)sizeof(T);
+    auto fetch = [&](int l0, int c) {
+        const int E = min(lpw, nl - l0) * np;
+        const long long base = (long long)l0 * np, off = c * d.N + base;
+        for (int e = per * lane; e < E; e += 32 * per) {
+            copy_async(sr + e, r + off + e, b16);
+            if (MODE == kIter) copy_async(sq + e, q + off + e, b16);
+            if (c == 0) copy_async(si + e, idt + base + e, b16);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    // Elements past a line's end are zeros here and stay so: with g = 0 and 1 / dt = 0 there, whatever is formed from
+    // them is 0 (unless the system holds a NaN or an infinity, which ends the solve).
+    for (int e = lane; e < 32 * D; e += 32) wb[e] = zero;
+    double a_rz = 0.0, a_rr = 0.0;   // per-line partials (in T) are added here in FP64
+    int line0 = (blockIdx.x * warps + warp) * lpw;
+    if (line0 < nl) fetch(line0, 0);
+    for (; line0 < nl; line0 += step) {
+        const int E = min(lpw, nl - line0) * np;
+        const bool valid = line0 + ln < nl;
+        const T w = valid ? t.ap[line0 + ln] : zero;
+        const long long base = (long long)line0 * np;
+        T g[S], id[S], b[S];
+        T A = T(1);
+        // scan multipliers, forwards and backwards (a wrong product in the lane at an end of the line is never used)
+        T As[5], Cs[5];
+        T line_rz = zero, line_rr = zero;
+#pragma unroll 1
+        for (int c = 0; c < nc; c++) {
+            const long long off = c * d.N + base;
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            __syncwarp();
+            // (a value the compiler cannot see through: the places of all elements, formed once for the three
+            // components, would not fit the registers)
+            int l0 = lane;
+            asm volatile("" : "+r"(l0));
+            if (c == 0) {
+                packs(std::integral_constant<int, 2>(), l0, E, [&](int e, int w0) { store<T, 2>(wb + w0, load<T, 2>(si + e)); });
+                __syncwarp();
+#pragma unroll
+                for (int tt = 0; tt < S; tt += W) {
+                    const Pack<T, W> v = load<T, W>(seg + tt);
+#pragma unroll
+                    for (int m = 0; m < W; m++) {
+                        id[tt + m] = valid ? v.v[m] : zero;
+                        g[tt + m] = w * id[tt + m];
+                        A *= g[tt + m];
+                    }
+                }
+                T C = A;
+#pragma unroll
+                for (int st = 0; st < 5; st++) {
+                    const int o = 1 << st;
+                    As[st] = A;
+                    Cs[st] = C;
+                    if (o < L) {
+                        const T Ao = __shfl_up_sync(kFull, A, o, L), Co = __shfl_down_sync(kFull, C, o, L);
+                        if (gl >= o) A *= Ao;
+                        if (gl + o < L) C *= Co;
+                    }
+                }
+                __syncwarp();
+            }
+            T* const rc = r + off;
+            auto update = [&](auto width) {
+                constexpr int V = decltype(width)::value;
+                packs(width, l0, E, [&](int e, int w0) {
+                    Pack<T, V> rv = load<T, V>(sr + e);
+                    if (MODE == kIter) {
+                        const Pack<T, V> qv = load<T, V>(sq + e);
+#pragma unroll
+                        for (int m = 0; m < V; m++) rv.v[m] = fma(-al, qv.v[m], rv.v[m]);
+                        store<T, V>(rc + e, rv);
+                    }
+                    store<T, V>(wb + w0, rv);
+                });
+            };
+            if (b16) update(std::integral_constant<int, W>());
+            else update(std::integral_constant<int, 2>());
+            __syncwarp();
+            if (c + 1 < nc) fetch(line0, c + 1);
+            else if (line0 + step < nl) fetch(line0 + step, 0);
+            // forward: u_0 = r_0 / dt_0; u_k = (r_k + w u_{k-1}) / dt_k; the last also + w u_0 / dt
+            T B = zero;
+#pragma unroll
+            for (int tt = 0; tt < S; tt += W) {
+                const Pack<T, W> v = load<T, W>(seg + tt);
+#pragma unroll
+                for (int m = 0; m < W; m++) b[tt + m] = v.v[m] * id[tt + m];
+            }
+            const T u0 = __shfl_sync(kFull, b[0], 0, L);
+#pragma unroll
+            for (int tt = 0; tt < S; tt++) {
+                B = tt == 0 ? b[0] : fma(g[tt], B, b[tt]);
+            }
+#pragma unroll
+            for (int st = 0; st < 5; st++) {
+                const int o = 1 << st;
+                if (o < L) {
+                    const T Bo = __shfl_up_sync(kFull, B, o, L);
+                    if (gl >= o) B = fma(As[st], Bo, B);
+                }
+            }
+            T u = __shfl_up_sync(kFull, B, 1, L);
+            if (gl == 0) u = zero;
+#pragma unroll
+            for (int tt = 0; tt < S; tt++) {
+                u = fma(g[tt], u, b[tt]);
+                b[tt] = u;
+            }
+            // (nothing follows the last element, so its wrap term is added to it alone)
+            T ul = zero;
+            one_of<S>(lastt, [&](auto at) {
+                constexpr int tt = decltype(at)::value;
+                if (gl == lastl) b[tt] = fma(g[tt], u0, b[tt]);
+                ul = b[tt];
+            });
+            // backward: z_{np-1} = u_{np-1}; z_k = u_k + w z_{k+1} / dt_k; the first also + w z_{np-1} / dt_0
+            const T zl = __shfl_sync(kFull, ul, lastl, L);
+            if (gl == 0) b[0] = fma(g[0], zl, b[0]);
+            T En = b[S - 1];
+#pragma unroll
+            for (int tt = S - 2; tt >= 0; tt--) En = fma(g[tt], En, b[tt]);
+#pragma unroll
+            for (int st = 0; st < 5; st++) {
+                const int o = 1 << st;
+                if (o < L) {
+                    const T Eo = __shfl_down_sync(kFull, En, o, L);
+                    if (gl + o < L) En = fma(Cs[st], Eo, En);
+                }
+            }
+            T zz = __shfl_down_sync(kFull, En, 1, L);
+            if (gl == L - 1) zz = zero;
+#pragma unroll
+            for (int tt = S - W; tt >= 0; tt -= W) {
+                const Pack<T, W> rv = load<T, W>(seg + tt);
+                Pack<T, W> zv;
+#pragma unroll
+                for (int m = W - 1; m >= 0; m--) {
+                    zz = fma(g[tt + m], zz, b[tt + m]);
+                    zv.v[m] = zz;
+                    line_rz = fma(rv.v[m], zz, line_rz);
+                    line_rr = fma(rv.v[m], rv.v[m], line_rr);
+                }
+                store<T, W>(seg + tt, zv);
+            }
+            __syncwarp();
+            T* const zc = z + off;
+            auto hand_out = [&](auto width) {
+                constexpr int V = decltype(width)::value;
+                packs(width, l0, E, [&](int e, int w0) {
+                    const Pack<T, V> zv = load<T, V>(wb + w0);
+                    store<T, V>(zc + e, zv);
+                    if (MODE == kInit) store<T, V>(p + off + e, zv);
+                });
+            };
+            if (b16) hand_out(std::integral_constant<int, W>());
+            else hand_out(std::integral_constant<int, 2>());
+            __syncwarp();
+        }
+        if (valid) {
+            a_rz += (double)line_rz;
+            a_rr = fma(dgv[line0 + ln], (double)line_rr, a_rr);
+        }
     }
+    line_finish<T, MODE>(a_rz, a_rr, sc, partials, restart);
 }
 
 template <typename T>
@@ -281,50 +544,53 @@ size_t line_smem(const Dims& d, int warps) {
     return (size_t)warps * 3 * padded_len(d.np) * sizeof(T);
 }
 
-// compile-time segment length for np = 512 (16 elements per lane), else the generic kernel
-int seg_of(const Dims& d) { return (d.np == 512) ? 16 : 0; }
-
-template <typename T, int MODE, int SEG>
-cudaError_t set_smem(size_t bytes) {
-    cudaError_t e = cudaFuncSetAttribute(k_pc2_line<T, 1, MODE, SEG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)bytes);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_pc2_line<T, 2, MODE, SEG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)bytes);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_pc2_line<T, 3, MODE, SEG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)bytes);
-    return e;
+// the kernel of a mode for a segment length
+template <typename T, int MODE>
+auto seg_kernel(int seg) {
+    switch (seg) {
+        case 4: return k_pc2_seg<T, 4, MODE>;
+        case 8: return k_pc2_seg<T, 8, MODE>;
+        case 12: return k_pc2_seg<T, 12, MODE>;
+        case 16: return k_pc2_seg<T, 16, MODE>;
+        case 20: return k_pc2_seg<T, 20, MODE>;
+        default: return k_pc2_seg<T, kSegMax, MODE>;
+    }
 }
 
-template <typename T, int SEG>
-cudaError_t set_smem_all(size_t bytes) {
-    cudaError_t e = set_smem<T, kIter, SEG>(bytes);
-    if (e == cudaSuccess) e = set_smem<T, kInit, SEG>(bytes);
-    if (e == cudaSuccess) e = set_smem<T, kReliable, SEG>(bytes);
-    return e;
+template <typename T, int MODE>
+cudaError_t set_smem(const LineShape& s) {
+    return s.seg ? cudaFuncSetAttribute(seg_kernel<T, MODE>(s.seg), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem)
+                 : cudaFuncSetAttribute(k_pc2_line<T, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem);
 }
 
-// launch shape of the line kernel for element type T: up to 8 warps per CTA within 200 KB
+// Lines of up to 32 kSegMax elements take the register kernel, longer ones the generic kernel (up to 8 warps per
+// CTA within 200 KB).
 template <typename T>
-mhd_status_t line_shape(mhd_grid_s* g, Pc2Work* w, int slot) {
-    int warps = 8;
-    while (warps > 1 && line_smem<T>(g->d, warps) > 200 * 1024) warps >>= 1;
-    if (line_smem<T>(g->d, warps) > 200 * 1024) return set_error(g, MHD_ERR_ARG, "PC2: np too large for the line kernel");
-    const size_t bytes = line_smem<T>(g->d, warps);
-    const bool s16 = seg_of(g->d) == 16;
-    if ((s16 ? set_smem_all<T, 16>(bytes) : set_smem_all<T, 0>(bytes)) != cudaSuccess)
+mhd_status_t line_shape(mhd_grid_s* g, LineShape* s) {
+    const int np = g->d.np, nl = g->d.nr * g->d.nt;
+    int per_cta = 0;   // lines a CTA takes at once
+    if (np <= 32 * kSegMax) {
+        s->lanes = sizeof(T) == 4 ? 32 : (np <= 128 ? 8 : np <= 256 ? 16 : 32);
+        s->seg = ((np + s->lanes - 1) / s->lanes + 3) & ~3;
+        s->warps = 4;
+        s->smem = (size_t)s->warps * 32 * (4 * s->seg + 16 / sizeof(T)) * sizeof(T);   // at most (kSegDist)
+        per_cta = s->warps * (32 / s->lanes);
+    } else {
+        s->lanes = s->seg = 0;
+        s->warps = 8;
+        while (s->warps > 1 && line_smem<T>(g->d, s->warps) > 200 * 1024) s->warps >>= 1;
+        s->smem = line_smem<T>(g->d, s->warps);
+        if (s->smem > 200 * 1024) return set_error(g, MHD_ERR_ARG, "PC2: np too large for the line kernel");
+        per_cta = s->warps;
+    }
+    constexpr int kFirst = sizeof(T) == 8 ? kInit : kReliable;   // the mode that starts or renews a recurrence
+    if (set_smem<T, kIter>(*s) != cudaSuccess || set_smem<T, kFirst>(*s) != cudaSuccess)
         return check_cuda(g, "PC2: shared memory attribute");
     int per_sm = 0;
-    if (s16)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pc2_line<T, 3, kIter, 16>, 32 * warps, bytes);
-    else
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pc2_line<T, 3, kIter, 0>, 32 * warps, bytes);
+    if (s->seg) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, seg_kernel<T, kIter>(s->seg), 32 * s->warps, s->smem);
+    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pc2_line<T, kIter>, 32 * s->warps, s->smem);
     if (per_sm < 1) per_sm = 1;
-    const int nl = g->d.nr * g->d.nt;
-    w->warps[slot] = warps;
-    w->smem[slot] = bytes;
-    w->line_blocks[slot] = std::min(std::min(g->num_sms * per_sm, (nl + warps - 1) / warps), kMaxBlocks);
+    s->blocks = std::min(std::min(g->num_sms * per_sm, (nl + per_cta - 1) / per_cta), kMaxBlocks);
     return MHD_OK;
 }
 
@@ -344,8 +610,8 @@ mhd_status_t pc2_workspace(mhd_grid_s* g, Pc2Work** out) {
         cudaGetLastError();
         return set_error(g, MHD_ERR_OOM, "PC2: workspace allocation failed");
     }
-    mhd_status_t st = line_shape<double>(g, w, 0);
-    if (st == MHD_OK) st = line_shape<float>(g, w, 1);
+    mhd_status_t st = line_shape<double>(g, &w->shape[0]);
+    if (st == MHD_OK) st = line_shape<float>(g, &w->shape[1]);
     if (st == MHD_OK && cudaMemsetAsync(w->z32, 0, sizeof(float) * 3 * N, g->stream) != cudaSuccess)
         st = check_cuda(g, "PC2: workspace clear");
     if (st != MHD_OK) {
@@ -360,40 +626,29 @@ mhd_status_t pc2_workspace(mhd_grid_s* g, Pc2Work** out) {
     return MHD_OK;
 }
 
-template <typename T, int MODE, int SEG>
-void launch_seg(mhd_grid_s* g, cudaStream_t st, const Pc2Work* w, int nc, int restart) {
+template <typename T, int MODE>
+void launch_line(mhd_grid_s* g, cudaStream_t st, int nc, int restart = 0) {
+    const auto* w = reinterpret_cast<const Pc2Work*>(g->pc2_mem);
     const Dims d = g->d;
-    const int slot = sizeof(T) == 8 ? 0 : 1;
-    const dim3 grid(w->line_blocks[slot]), block(32 * w->warps[slot]);
-    const size_t sm = w->smem[slot];
-    T *x, *p, *r, *q;
+    const LineShape& s = w->shape[sizeof(T) == 8 ? 0 : 1];
+    T *p, *r, *q;
     const T* idt;
     OpTab<T> t;
     if constexpr (sizeof(T) == 8) {
-        x = g->x64; p = g->p64; r = g->r64; q = g->q64; idt = w->idt; t = g->t64;
+        p = g->p64; r = g->r64; q = g->q64; idt = w->idt; t = g->t64;
     } else {
-        x = g->x32; p = g->p32; r = g->r32; q = g->q32; idt = w->idt32; t = g->t32;
+        p = g->p32; r = g->r32; q = g->q32; idt = w->idt32; t = g->t32;
     }
     // z~: FP64 in the second half of the p double buffer, FP32 in the workspace
     T* z;
     if constexpr (sizeof(T) == 8) z = p + 3 * (size_t)d.N;
     else z = w->z32;
-    if (nc == 3)
-        k_pc2_line<T, 3, MODE, SEG><<<grid, block, sm, st>>>(d, t, g->tu.dg, idt, x, p, r, q, z, g->sc, g->partials,
-                                                              restart);
-    else if (nc == 2)
-        k_pc2_line<T, 2, MODE, SEG><<<grid, block, sm, st>>>(d, t, g->tu.dg, idt, x, p, r, q, z, g->sc, g->partials,
-                                                              restart);
+    if (s.seg)
+        seg_kernel<T, MODE>(s.seg)<<<s.blocks, 32 * s.warps, s.smem, st>>>(d, nc, s.lanes, t, g->tu.dg, idt, p, r, q, z,
+                                                                          g->sc, g->partials, restart);
     else
-        k_pc2_line<T, 1, MODE, SEG><<<grid, block, sm, st>>>(d, t, g->tu.dg, idt, x, p, r, q, z, g->sc, g->partials,
-                                                              restart);
-}
-
-template <typename T, int MODE>
-void launch_line(mhd_grid_s* g, cudaStream_t st, int nc, int restart = 0) {
-    const auto* w = reinterpret_cast<const Pc2Work*>(g->pc2_mem);
-    if (seg_of(g->d) == 16) launch_seg<T, MODE, 16>(g, st, w, nc, restart);
-    else launch_seg<T, MODE, 0>(g, st, w, nc, restart);
+        k_pc2_line<T, MODE><<<s.blocks, 32 * s.warps, s.smem, st>>>(d, nc, t, g->tu.dg, idt, p, r, q, z, g->sc, g->partials,
+                                                                    restart);
 }
 
 }  // namespace

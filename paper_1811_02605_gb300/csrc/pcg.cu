@@ -1404,7 +1404,7 @@ void enqueue_pc2(mhd_grid_s* g, cudaStream_t st, int blocks) {
     const Dims d = g->d;
     double* z = g->p64 + 3 * (size_t)d.N;
     int ps = prof_begin(g, st, MHD_KERNEL_PUPDATE64);
-    k_pupdate<double, 2, NC><<<blocks, kThreads, 0, st>>>(d, z, g->p64, nullptr, g->sc);
+    k_pupdate<double, 2, NC, true><<<blocks, kThreads, 0, st>>>(d, z, g->p64, g->x64, g->sc);
     prof_end(g, st, ps);
     ps = prof_begin(g, st, MHD_KERNEL_SPMV64);
     k_spmv_dot<double, 2, NC><<<blocks, kThreads, 0, st>>>(d, g->p64, g->q64, g->t64, g->sc, g->partials);
