@@ -181,26 +181,8 @@ mhd_status_t coeffs(mhd_grid_s* g, const mhd_params_t* p, const double* vr, cons
 }
 
 // ------------------------------------------------------------------------------------------
-// polar ring sums: out[i] (north, ring j = 0) and out[nr + i] (south, ring j = nt-1) of a
-// cell-centred array (one CTA per ring, fixed-order reduction)
+// polar rings
 // ------------------------------------------------------------------------------------------
-__global__ void k_ring(Dims d, const double* __restrict__ a, double* __restrict__ out) {
-    const int i = blockIdx.x % d.nr;
-    const int south = blockIdx.x / d.nr;
-    const int j = south ? d.nt - 1 : 0;
-    double s = 0.0;
-    for (int k = threadIdx.x; k < d.np; k += blockDim.x) s += a[ix(d, i, j, k)];
-    __shared__ double sm[kThreads / 32];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); w++) t += sm[w];
-        out[blockIdx.x] = t;
-    }
-}
-
 // first-harmonic sums of the rows next to the poles (one CTA per row, fixed-order reduction):
 // out[2 b] = sum_k a_k cos(phi_c_k), out[2 b + 1] = sum_k a_k sin(phi_c_k), b = i (north row at
 // off_n + i stride_i) or nr + i (south row at off_s + i stride_i)
@@ -251,14 +233,16 @@ void bt_harmonics(mhd_grid_s* g, const double* bt, cudaStream_t st) {
 // ------------------------------------------------------------------------------------------
 // J on all edges in one launch, a warp per row; a polar radial row takes its ring's sum of B_phi itself (the cap
 // circulation), and with bh the warps of the first 2 nr rows form the harmonics of the B_theta rings beside the
-// poles. walls_zero: the resistive operator's current, 0 on the tangential edges of r0 and r1.
+// poles. walls_zero: the resistive operator's current, 0 on the tangential edges of r0 and r1. done (may be null):
+// a solve's flag, nothing is formed once it is set.
 __global__ void __launch_bounds__(kThreads) k_current(Dims d, const double* __restrict__ cr,
                                                       const double* __restrict__ ct, const double* __restrict__ cp,
                                                       const double* __restrict__ br, const double* __restrict__ bt,
                                                       const double* __restrict__ bp, double* __restrict__ jr,
                                                       double* __restrict__ jt, double* __restrict__ jp,
                                                       const double* __restrict__ pcs, double* __restrict__ bh,
-                                                      int walls_zero) {
+                                                      int walls_zero, const int* __restrict__ done) {
+    if (done && *done) return;
     const unsigned int n_h = bh ? 2u * d.nr : 0u, n_r = (unsigned int)(d.nr * (d.nt + 1)),
                        n_t = (unsigned int)((d.nr + 1) * d.nt), n_p = (unsigned int)((d.nr + 1) * (d.nt + 1));
     const int np = d.np, lane = threadIdx.x & 31;
@@ -333,20 +317,28 @@ int row_blocks(const mhd_grid_s* g, long long rows) {
     return grid_blocks(g, 32 * rows, resident_per_sm<K>());
 }
 
-void current_and_harmonics(mhd_grid_s* g, const double* br, const double* bt, const double* bp, double* bh,
-                           bool walls_zero, cudaStream_t st) {
+void edge_current(mhd_grid_s* g, const double* cr, const double* ct, const double* cp, const double* br, const double* bt,
+                  const double* bp, double* bh, bool walls_zero, const int* done, cudaStream_t st) {
     const Dims d = g->d;
     const long long rows = (bh ? 2ll * d.nr : 0ll) + (long long)d.nr * (d.nt + 1) + (long long)(d.nr + 1) * d.nt +
                            (long long)(d.nr + 1) * (d.nt + 1);
-    k_current<<<row_blocks<k_current>(g, rows), kThreads, 0, st>>>(d, g->ex.jr, g->ex.jt, g->ex.jp, br, bt, bp, g->er, g->et,
-                                                                   g->ep, g->geo.pcs, bh, walls_zero ? 1 : 0);
+    k_current<<<row_blocks<k_current>(g, rows), kThreads, 0, st>>>(d, cr, ct, cp, br, bt, bp, g->er, g->et, g->ep,
+                                                                   g->geo.pcs, bh, walls_zero ? 1 : 0, done);
+}
+
+void current_and_harmonics(mhd_grid_s* g, const double* br, const double* bt, const double* bp, double* bh, cudaStream_t st) {
+    edge_current(g, g->ex.jr, g->ex.jt, g->ex.jp, br, bt, bp, bh, false, nullptr, st);
 }
 
 }  // namespace
 
-void current_edges(mhd_grid_s* g, const double* br, const double* bt, const double* bp, bool walls_zero,
-                   cudaStream_t st) {
-    current_and_harmonics(g, br, bt, bp, nullptr, walls_zero, st ? st : g->stream);
+void current_edges(mhd_grid_s* g, const double* br, const double* bt, const double* bp) {
+    current_and_harmonics(g, br, bt, bp, nullptr, g->stream);
+}
+
+void res_edge_current(mhd_grid_s* g, const double* cr, const double* ct, const double* cp, const double* br, const double* bt,
+                      const double* bp, const int* done, cudaStream_t st) {
+    edge_current(g, cr, ct, cp, br, bt, bp, nullptr, true, done, st);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -439,7 +431,7 @@ void force_launch(mhd_grid_s* g, const Vel<DLT>& v, const double* br, const doub
 void force(mhd_grid_s* g, const double* vr, const double* vt, const double* vp, const double* dlt, double dfac,
            const double* br, const double* bt, const double* bp, const double* dt_dev, double dt_host,
            const double* b_avg, double* b) {
-    current_and_harmonics(g, br, bt, bp, g->bharm, false, g->stream);
+    current_and_harmonics(g, br, bt, bp, g->bharm, g->stream);
     const Vel<false> v{vr, vt, vp, nullptr, 0.0, g->d.N};
     const Vel<true> w{vr, vt, vp, dlt, dfac, g->d.N};
     if (dlt && b_avg) force_launch<true, true>(g, w, br, bt, bp, dt_dev, dt_host, b_avg, b);
@@ -610,7 +602,7 @@ void induction(mhd_grid_s* g, const double* vr, const double* vt, const double* 
                double eta, const double* dt_dev, double dt_host, double* br, double* bt, double* bp, bool current_ready) {
     const Dims d = g->d;
     if (!current_ready) {
-        if (eta != 0.0) current_and_harmonics(g, br, bt, bp, g->bharm, false, g->stream);
+        if (eta != 0.0) current_and_harmonics(g, br, bt, bp, g->bharm, g->stream);
         else bt_harmonics(g, bt);
     }
     const Vel<false> v{vr, vt, vp, nullptr, 0.0, d.N};
@@ -622,10 +614,6 @@ void induction(mhd_grid_s* g, const double* vr, const double* vt, const double* 
     const long long rows = (long long)d.nr * (d.nt + 1) + (long long)(d.nr + 1) * d.nt + (long long)(d.nr + 1) * (d.nt + 1);
     k_eedges<<<row_blocks<k_eedges>(g, rows), kThreads, 0, g->stream>>>(d, g->ec, g->er, g->et, g->ep);
     ct_launch(g, dt_dev, dt_host, kEdgeScale, br, bt, bp);
-}
-
-void ring_sums(mhd_grid_s* g, const double* a, cudaStream_t st) {
-    k_ring<<<2 * g->d.nr, kThreads, 0, st ? st : g->stream>>>(g->d, a, g->ring);
 }
 
 void ct_apply(mhd_grid_s* g, const double* dt_dev, double* br, double* bt, double* bp) {
@@ -690,7 +678,7 @@ __global__ void __launch_bounds__(kThreads) k_diag(Dims d, Geo G, ExTab X, Vel<f
 void diagnostics(mhd_grid_s* g, const double* vr, const double* vt, const double* vp, const double* br,
                  const double* bt, const double* bp, double* out) {
     const Dims d = g->d;
-    current_and_harmonics(g, br, bt, bp, g->bharm, false, g->stream);
+    current_and_harmonics(g, br, bt, bp, g->bharm, g->stream);
     const Vel<false> v{vr, vt, vp, nullptr, 0.0, d.N};
     // two reductions: 5 partials a CTA in the array's 4 kMaxBlocks, and a ticket each (the solver's is idle here)
     const int blocks = std::min(row_blocks<k_diag>(g, (long long)d.nr * d.nt), kMaxBlocks * kPartialsPerBlock / 5);

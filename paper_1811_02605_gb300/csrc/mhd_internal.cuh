@@ -349,10 +349,11 @@ int resident_per_sm() {
 // explicit kernels (explicit.cu)
 mhd_status_t coeffs(mhd_grid_s* g, const mhd_params_t* p, const double* vr, const double* vt,
                     const double* vp, const double* br, const double* bt, const double* bp);
-void current_edges(mhd_grid_s* g, const double* br, const double* bt, const double* bp, bool walls_zero = false,
-                   cudaStream_t st = nullptr);
-// polar ring sums of a cell-centred array into the grid's ring buffer (north rows, then south)
-void ring_sums(mhd_grid_s* g, const double* a, cudaStream_t st);
+void current_edges(mhd_grid_s* g, const double* br, const double* bt, const double* bp);
+// the same with the resistive operator's edge tables, 0 on the tangential edges of r0 and r1; done (may be null): a
+// solve's flag, nothing is formed once it is set
+void res_edge_current(mhd_grid_s* g, const double* cr, const double* ct, const double* cp, const double* br,
+                      const double* bt, const double* bp, const int* done, cudaStream_t st);
 // first-harmonic sums (cos, sin of the phi centres) of the rows next to the poles of an array of
 // np-element rows: out[2 b], out[2 b + 1] for b = i (row off_n + i stride_i) and b = nr + i (row
 // off_s + i stride_i), i < nr

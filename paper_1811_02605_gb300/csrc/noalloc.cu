@@ -157,7 +157,6 @@ extern "C" mhd_status_t mhd_force_noalloc(const mhd_grid_desc_t* desc, const mhd
     double* jr = take(nr * (nt + 1) * np);
     double* jt = take((nr + 1) * nt * np);
     double* jp = take((nr + 1) * (nt + 1) * np);
-    double* ring = take(2 * nr);
     double* pcs = take(2 * np);
     double* bharm = take(4 * nr);   // north and south B_theta rings; the adjoint half is not used here
     if (off > kScratchDoubles) return MHD_ERR_ARG;
@@ -217,7 +216,6 @@ extern "C" mhd_status_t mhd_force_noalloc(const mhd_grid_desc_t* desc, const mhd
     v.er = jr;
     v.et = jt;
     v.ep = jp;
-    v.ring = ring;
     v.bharm = bharm;
 
     k_noalloc_radial<<<1, 1, 0, v.stream>>>(d.nr, d.r0, d.r1, d.stretch, r);

@@ -84,68 +84,9 @@ __device__ __forceinline__ int face_row(const Dims& d, long long f) {
 
 // ------------------------------------------------------------------------------------------
 // edge current of the resistive operator (interior edges; the tangential edges of r0 and r1
-// carry none), from per-row coefficient tables
-// ------------------------------------------------------------------------------------------
-// radial edges (i, j, k), rows i (nt + 1) + j: c = {w_phi(j), w_phi(j-1), w_theta, w_polar}
-__global__ void __launch_bounds__(kThreads) k_res_jr(Dims d, const double* __restrict__ cr,
-                                                     const double* __restrict__ ring, const double* __restrict__ bt,
-                                                     const double* __restrict__ bp, double* __restrict__ jr) {
-    const long long n = (long long)d.nr * (d.nt + 1) * d.np;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-        int k;
-        unsigned int row;
-        split_np(d, e, k, row);
-        const int i = (int)(row / (unsigned int)(d.nt + 1)), j = (int)(row - (unsigned int)i * (d.nt + 1));
-        const double* c = cr + 4 * (size_t)row;
-        double val;
-        if (j == 0) val = ring[i] * c[3];
-        else if (j == d.nt) val = -ring[d.nr + i] * c[3];
-        else val = c[0] * bp[ix(d, i, j, k)] - c[1] * bp[ix(d, i, j - 1, k)] -
-                   c[2] * (bt[ixt(d, i, j, k)] - bt[ixt(d, i, j, km1(d, k))]);
-        jr[e] = val;
-    }
-}
-
-// theta edges (i, j, k), rows i nt + j: c = {w_phi(i-1), w_r, w_phi(i)}
-__global__ void __launch_bounds__(kThreads) k_res_jt(Dims d, const double* __restrict__ ct,
-                                                     const double* __restrict__ br, const double* __restrict__ bp,
-                                                     double* __restrict__ jt) {
-    const long long n = (long long)(d.nr + 1) * d.nt * d.np;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-        int k;
-        unsigned int row;
-        split_np(d, e, k, row);
-        const int i = (int)(row / (unsigned int)d.nt), j = (int)(row - (unsigned int)i * d.nt);
-        double val = 0.0;
-        if (i > 0 && i < d.nr) {
-            const double* c = ct + 3 * (size_t)row;
-            val = c[0] * bp[ix(d, i - 1, j, k)] + c[1] * (br[ix(d, i, j, k)] - br[ix(d, i, j, km1(d, k))]) -
-                  c[2] * bp[ix(d, i, j, k)];
-        }
-        jt[e] = val;
-    }
-}
-
-// phi edges (i, j, k), rows i (nt + 1) + j: c = {w_r, w_theta(i), w_theta(i-1)}
-__global__ void __launch_bounds__(kThreads) k_res_jp(Dims d, const double* __restrict__ cp,
-                                                     const double* __restrict__ br, const double* __restrict__ bt,
-                                                     double* __restrict__ jp) {
-    const long long n = (long long)(d.nr + 1) * (d.nt + 1) * d.np;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-        int k;
-        unsigned int row;
-        split_np(d, e, k, row);
-        const int i = (int)(row / (unsigned int)(d.nt + 1)), j = (int)(row - (unsigned int)i * (d.nt + 1));
-        double val = 0.0;
-        if (i > 0 && i < d.nr && j > 0 && j < d.nt) {
-            const double* c = cp + 3 * (size_t)row;
-            val = c[0] * (br[ix(d, i, j - 1, k)] - br[ix(d, i, j, k)]) + c[1] * bt[ixt(d, i, j, k)] -
-                  c[2] * bt[ixt(d, i - 1, j, k)];
-        }
-        jp[e] = val;
-    }
-}
-
+// carry none), from per-row coefficient tables (k_current): radial edges, rows i (nt + 1) + j, {w_phi(j),
+// w_phi(j-1), w_theta, w_polar}; theta edges, rows i nt + j, {w_phi(i-1), w_r, w_phi(i)}; phi edges, rows
+// i (nt + 1) + j, {w_r, w_theta(i), w_theta(i-1)}
 // ------------------------------------------------------------------------------------------
 // face kernels; co[4 t + 0..2] = dte l* x the three edge-length factors of row t, co[4 t + 3] =
 // 1 / diag (both formed per solve), w[t] = W of row t
@@ -497,22 +438,18 @@ mhd_status_t res_workspace(mhd_grid_s* g, ResWork** out) {
     return check_cuda(g, "implicit resistivity workspace");
 }
 
-// edge current of the stacked face vector v into the grid's edge arrays
-void res_current(mhd_grid_s* g, cudaStream_t st, const ResWork* w, const double* v) {
-    const Dims d = g->d;
-    const ResSizes z = res_sizes(d);
-    const double *br = v, *bt = v + z.nbr, *bp = v + z.nbr + z.nbt;
-    ring_sums(g, bp, st);
-    const long long n = (long long)(d.nr + 1) * (d.nt + 1) * d.np;
-    k_res_jr<<<grid_blocks(g, n, resident_per_sm<k_res_jr>()), kThreads, 0, st>>>(d, w->cr, g->ring, bt, bp, g->er);
-    k_res_jt<<<grid_blocks(g, n, resident_per_sm<k_res_jt>()), kThreads, 0, st>>>(d, w->ct, br, bp, g->et);
-    k_res_jp<<<grid_blocks(g, n, resident_per_sm<k_res_jp>()), kThreads, 0, st>>>(d, w->cp, br, bt, g->ep);
+// edge current of the stacked face vector v into the grid's edge arrays, one launch. In an iteration it is skipped
+// once the solve is done: the graph's remaining iterations went on forming it (64x64x128, 65 iterations: with the
+// four launches it took before, 76 us an iteration, now 70).
+void res_current(mhd_grid_s* g, cudaStream_t st, const ResWork* w, const double* v, bool iterating) {
+    const ResSizes z = res_sizes(g->d);
+    res_edge_current(g, w->cr, w->ct, w->cp, v, v + z.nbr, v + z.nbr + z.nbt, iterating ? &g->sc->done : nullptr, st);
 }
 
 void res_enqueue_iteration(mhd_grid_s* g, cudaStream_t st, ResWork* w) {
     const Dims d = g->d;
     const ResSizes z = res_sizes(d);
-    res_current(g, st, w, w->p);
+    res_current(g, st, w, w->p, true);
     k_res_apply<<<grid_blocks(g, z.nf, resident_per_sm<k_res_apply>()), kThreads, 0, st>>>(
         d, w->w, w->co, w->p, g->er, g->et, g->ep, w->q, g->sc, g->partials, z.nf);
     k_res_update<<<grid_blocks(g, z.nf, resident_per_sm<k_res_update>()), kThreads, 0, st>>>(
@@ -619,14 +556,14 @@ mhd_status_t res_solve(mhd_grid_s* g, const double* dt_dev, double eta, double* 
     cudaMemcpyAsync(w->q + z.nbr, bt, sizeof(double) * z.nbt, cudaMemcpyDeviceToDevice, g->stream);
     cudaMemcpyAsync(w->q + z.nbr + z.nbt, bp, sizeof(double) * z.nbp, cudaMemcpyDeviceToDevice, g->stream);
     res_begin(g, w, dt_dev, eta, p);
-    res_current(g, g->stream, w, w->q);
+    res_current(g, g->stream, w, w->q, false);
     k_res_init<<<blocks, kThreads, 0, g->stream>>>(d, w->w, w->co, w->q, g->er, g->et, g->ep, w->x, w->r, w->p, g->sc,
                                                    g->partials, z.nf);
     if ((st = check_cuda(g, "res init")) != MHD_OK) return st;
     if ((st = res_iterate(g, w)) != MHD_OK) return st;
     const PcgScalars h = *g->h_sc;
     // B = B* - dte curl_h J(x)
-    res_current(g, g->stream, w, w->x);
+    res_current(g, g->stream, w, w->x, false);
     ct_apply(g, &g->sc->dte, br, bt, bp);
     if ((st = check_cuda(g, "res final update")) != MHD_OK) return st;
     if (iters) *iters = h.iter;
