@@ -1033,57 +1033,53 @@ __global__ void k_finish64(Dims d, int nc, const double* __restrict__ xs, const 
 // (beta = 0, so the next p update gives p~32 = r~32); otherwise the true residual replaces the
 // recursive one and the CG recurrence continues with the same p~32 (reliable update, residual
 // replacement): beta = <r~_true, r~_true> / rho of the previous iteration.
-template <int V>
+// Bound by its FP64 instructions (2 multiply-adds per clock and SM). The three sums of the residual are one:
+// dg s^2 = 1, so sum dg r~^2 = ||r||^2, and <r~, r~> is the sum of s^2 times the groups' ||r||^2. At 256x256x512,
+// 3 components, with the FP64 sum of each r~32 in its place and FIRST tested at run time 2.7 ms, now 2.0 (both with the PC2 pass that follows it).
+template <bool FIRST>
 __global__ void __launch_bounds__(kThreads) k_outer_res(Dims d, int nc, const double* __restrict__ b,
                                                         const double* __restrict__ x, float* __restrict__ r32a,
                                                         float* __restrict__ r32b,
                                                         float* __restrict__ p32, float* __restrict__ x32,
                                                         OpTab<double> t, OpTab64u tu, PcgScalars* sc,
-                                                        double* __restrict__ partials, int first, int restart,
-                                                        int pc2, OpTab<float> t32) {
+                                                        double* __restrict__ partials, int restart, int pc2,
+                                                        OpTab<float> t32) {
     const int nt = d.nt;
     const unsigned int G = (unsigned int)(d.N / 2);
     // single-reduction FP32 pair (r32b non-null): <r~, A~ p~_old> of the replaced residual, in FP32
     // as its update kernel would have formed it, for the denominator of the next iteration
-    const bool want_wp = (r32b != nullptr) && !first;
-    const float* __restrict__ pold = p32 + (long long)(first ? 0 : sc->par) * 3 * d.N;
+    const bool want_wp = !FIRST && r32b != nullptr;
+    const float* __restrict__ pold = p32 + (long long)(FIRST ? 0 : sc->par) * 3 * d.N;
     double a_wp = 0.0;
     const long long plane = (long long)nt * d.np;
     // r~ goes to the half of a double-buffered r~ (r32b non-null) on the parity of p~
-    float* __restrict__ r32 = (r32b && !first && sc->par) ? r32b : r32a;
-    double a_rout = 0.0, a_bb = 0.0, a_rho = 0.0, a_rin = 0.0;
+    float* __restrict__ r32 = (r32b && !FIRST && sc->par) ? r32b : r32a;
+    double a_rout = 0.0, a_bb = 0.0, a_rho = 0.0;
     for (unsigned int g = blockIdx.x * blockDim.x + threadIdx.x; g < G; g += gridDim.x * blockDim.x) {
         const Cell c = decompose<2>(d, g);
         const double s = t.s[c.ij];
-        const double dg = tu.dg[c.ij];
+        const double dg = tu.dg[c.ij], s2 = s * s;
         const double wl = tu.awr[c.i * nt + c.j], wh = tu.awr[(c.i + 1) * nt + c.j];
         const double tl = tu.awt[c.i * (nt + 1) + c.j], th = tu.awt[c.i * (nt + 1) + c.j + 1];
         const double wp = tu.awp[c.ij];
-        double cell_in = 0.0;
+        double cell = 0.0;
         for (int k = 0; k < nc; k++) {
             const double* u = x + k * d.N;
-            double bv[2], xv[2], n[2], mx[2];
-            ldv<double, 2>(b + k * d.N + c.base, bv);
+            double rv[2], xv[2], n[2];
+            ldv<double, 2>(b + k * d.N + c.base, rv);
             ldv<double, 2>(u + c.base, xv);
             const long long row = c.base - c.k0;
             const int km = (c.k0 == 0) ? d.np - 1 : c.k0 - 1;
             const int kp = (c.k0 + 2 == d.np) ? 0 : c.k0 + 2;
-            mx[0] = dg * xv[0] - wp * (u[row + km] + xv[1]);
-            mx[1] = dg * xv[1] - wp * (xv[0] + u[row + kp]);
-            if (c.i > 0) { ldv<double, 2>(u + c.base - plane, n); mx[0] -= wl * n[0]; mx[1] -= wl * n[1]; }
-            if (c.i < d.nr - 1) { ldv<double, 2>(u + c.base + plane, n); mx[0] -= wh * n[0]; mx[1] -= wh * n[1]; }
-            if (c.j > 0) { ldv<double, 2>(u + c.base - d.np, n); mx[0] -= tl * n[0]; mx[1] -= tl * n[1]; }
-            if (c.j < nt - 1) { ldv<double, 2>(u + c.base + d.np, n); mx[0] -= th * n[0]; mx[1] -= th * n[1]; }
-            float rs[2];
-            for (int e = 0; e < 2; e++) {
-                const double rv = bv[e] - mx[e];
-                rs[e] = (float)(s * rv);
-                a_rout = fma(rv, rv, a_rout);
-                if (first) a_bb = fma(bv[e], bv[e], a_bb);
-                const double rd = (double)rs[e];
-                a_rho = fma(rd, rd, a_rho);
-                cell_in = fma(rd, rd, cell_in);
-            }
+            if constexpr (FIRST) a_bb = fma(rv[0], rv[0], fma(rv[1], rv[1], a_bb));
+            rv[0] = fma(wp, u[row + km] + xv[1], fma(-dg, xv[0], rv[0]));
+            rv[1] = fma(wp, xv[0] + u[row + kp], fma(-dg, xv[1], rv[1]));
+            if (c.i > 0) { ldv<double, 2>(u + c.base - plane, n); rv[0] = fma(wl, n[0], rv[0]); rv[1] = fma(wl, n[1], rv[1]); }
+            if (c.i < d.nr - 1) { ldv<double, 2>(u + c.base + plane, n); rv[0] = fma(wh, n[0], rv[0]); rv[1] = fma(wh, n[1], rv[1]); }
+            if (c.j > 0) { ldv<double, 2>(u + c.base - d.np, n); rv[0] = fma(tl, n[0], rv[0]); rv[1] = fma(tl, n[1], rv[1]); }
+            if (c.j < nt - 1) { ldv<double, 2>(u + c.base + d.np, n); rv[0] = fma(th, n[0], rv[0]); rv[1] = fma(th, n[1], rv[1]); }
+            cell = fma(rv[0], rv[0], fma(rv[1], rv[1], cell));
+            const float rs[2] = {(float)(s * rv[0]), (float)(s * rv[1])};
             *reinterpret_cast<float2*>(r32 + k * d.N + c.base) = make_float2(rs[0], rs[1]);
             if (want_wp) {
                 const float* pk = pold + k * d.N;
@@ -1112,14 +1108,15 @@ __global__ void __launch_bounds__(kThreads) k_outer_res(Dims d, int nc, const do
             }
             *reinterpret_cast<float2*>(x32 + k * d.N + c.base) = make_float2(0.f, 0.f);
             // first pass: p~32 = r~32 so no value left from an earlier solve can reach 0 * p
-            if (first) *reinterpret_cast<float2*>(p32 + k * d.N + c.base) = make_float2(rs[0], rs[1]);
+            if constexpr (FIRST) *reinterpret_cast<float2*>(p32 + k * d.N + c.base) = make_float2(rs[0], rs[1]);
         }
-        a_rin = fma(dg, cell_in, a_rin);
+        a_rout += cell;
+        a_rho = fma(s2, cell, a_rho);
     }
-    double val[4] = {a_rout, first ? a_bb : a_wp, a_rho, a_rin}, out[4];
-    if (reduce_last<4>(val, partials, &sc->count, out) && threadIdx.x == 0) {
+    double val[3] = {a_rout, FIRST ? a_bb : a_wp, a_rho}, out[3];
+    if (reduce_last<3>(val, partials, &sc->count, out) && threadIdx.x == 0) {
         if (want_wp) sc->wp = out[1];
-        if (first) {
+        if (FIRST) {
             sc->bb = out[1];
             sc->par = 0;
         }
@@ -1133,7 +1130,7 @@ __global__ void __launch_bounds__(kThreads) k_outer_res(Dims d, int nc, const do
             sc->beta = keep ? out[2] / sc->rho_prev : 0.0;
             sc->rho = out[2];
         }
-        sc->rr = out[3];
+        sc->rr = out[0];
         sc->iter = 0;
         const double bn = sqrt(sc->bb);
         if (!finite(out[0]) || !finite(out[2])) { sc->done = 3; sc->outer_done = 3; }
@@ -1901,9 +1898,14 @@ mhd_status_t solve(mhd_grid_s* g, const double* alpha_dev, int nc, const double*
     for (int o = 0; o <= prm->max_outer; o++) {
         const int ps = prof_begin(g, g->stream, MHD_KERNEL_OUTER_RES);
         const int restart = (o == 0 || prm->mixed_restart) ? 1 : 0;
-        k_outer_res<2><<<grid_blocks(g, d.N / 2, resident_per_sm<k_outer_res<2>>()), kThreads, 0, g->stream>>>(
-            d, nc, b, x, g->r32, (!pc2 && ((g->slab32 <= -6 && g->slab32 >= -8) || g->slab32 == -10)) ? g->q32 : nullptr, g->p32, g->x32, g->t64, g->tu, g->sc,
-            g->partials, o == 0 ? 1 : 0, restart, pc2 ? 1 : 0, g->t32);
+        float* const r_alt = (!pc2 && ((g->slab32 <= -6 && g->slab32 >= -8) || g->slab32 == -10)) ? g->q32 : nullptr;
+        auto outer_res = [&](auto kernel, int per_sm) {
+            kernel<<<grid_blocks(g, d.N / 2, per_sm), kThreads, 0, g->stream>>>(d, nc, b, x, g->r32, r_alt, g->p32, g->x32, g->t64,
+                                                                               g->tu, g->sc, g->partials, restart, pc2 ? 1 : 0,
+                                                                               g->t32);
+        };
+        if (o == 0) outer_res(k_outer_res<true>, resident_per_sm<k_outer_res<true>>());
+        else outer_res(k_outer_res<false>, resident_per_sm<k_outer_res<false>>());
         if (pc2) pc2_reliable32(g, nc, restart);
         prof_end(g, g->stream, ps);
         mhd_status_t st = check_cuda(g, "outer residual");
