@@ -240,21 +240,19 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 6 : 4) k_spmv_dot(D
     const int nt = d.nt;
     const unsigned int G = (unsigned int)(d.N / V);
     Acc<T> acc;
-    for (unsigned int g = blockIdx.x * blockDim.x + threadIdx.x; g < G; g += gridDim.x * blockDim.x) {
-        const Cell c = decompose<V>(d, g);
+    // one component at a time: holding all three components' neighbours at once raises the
+    // register count past two CTAs per SM and was measured slower
+    for (unsigned int it = blockIdx.x * blockDim.x + threadIdx.x; it < NC * G; it += gridDim.x * blockDim.x) {
+        const unsigned int k = it / G;
+        const Cell c = decompose<V>(d, it - k * G);
         const T cr_lo = t.ar[c.i * nt + c.j], cr_hi = t.ar[(c.i + 1) * nt + c.j];
         const T ct_lo = t.at[c.i * (nt + 1) + c.j], ct_hi = t.at[c.i * (nt + 1) + c.j + 1];
         const T cp = t.ap[c.ij];
-        // one component at a time: holding all three components' neighbours at once raises the
-        // register count past two CTAs per SM and was measured slower
-#pragma unroll 1
-        for (int k = 0; k < NC; k++) {
-            T v[V], o[V];
-            scaled_stencil<T, V>(d, c, p + k * d.N, cr_lo, cr_hi, ct_lo, ct_hi, cp, v, o);
-            stv<T, V>(q + k * d.N + c.base, o);
+        T v[V], o[V];
+        scaled_stencil<T, V>(d, c, p + k * d.N, cr_lo, cr_hi, ct_lo, ct_hi, cp, v, o);
+        stv<T, V>(q + k * d.N + c.base, o);
 #pragma unroll
-            for (int e = 0; e < V; e++) acc.fma_add(v[e], o[e]);
-        }
+        for (int e = 0; e < V; e++) acc.fma_add(v[e], o[e]);
     }
     double val[1] = {acc.get()}, out[1];
     if (reduce_last<1>(val, partials, &sc->count, out) && threadIdx.x == 0) {
@@ -1232,6 +1230,15 @@ constexpr int kPerSmIter = 4;
 
 bool use_v4(const mhd_grid_s* g) { return (g->d.np % 4) == 0; }
 
+// CTAs of the FP64 stencil over nc components: it is bound by FP64 instructions, so what counts is how evenly its
+// items (one component of a cell pair) fall on the SMs. 4 CTAs per SM, or 3 where the items then make fewer rounds
+// times CTAs (64x64x128: 7 x 3 against 6 x 4: 31 -> 29 us).
+int spmv64_blocks(const mhd_grid_s* g, int nc) {
+    const long long items = nc * (g->d.N / 2), wave = (long long)g->num_sms * kThreads;
+    const long long c4 = 4 * ((items + 4 * wave - 1) / (4 * wave)), c3 = 3 * ((items + 3 * wave - 1) / (3 * wave));
+    return grid_blocks(g, items, c3 < c4 ? 3 : 4);
+}
+
 // enqueue one CG iteration (p update, stencil + <p,q>, update) of the given precision
 template <typename T, int V, int NC>
 void enqueue_split(mhd_grid_s* g, cudaStream_t st, T* x, T* r, T* p, T* q, const OpTab<T>& t, int blocks,
@@ -1242,7 +1249,7 @@ void enqueue_split(mhd_grid_s* g, cudaStream_t st, T* x, T* r, T* p, T* q, const
     prof_end(g, st, s);
     s = prof_begin(g, st, prof0 + 1);
     // the FP32 stencil is latency-bound: 6 CTAs per SM instead of 4 for more loads in flight
-    const int bs = (sizeof(T) == 4) ? grid_blocks(g, d.N / V, 6) : blocks;
+    const int bs = (sizeof(T) == 4) ? grid_blocks(g, NC * (d.N / V), 6) : spmv64_blocks(g, NC);
     k_spmv_dot<T, V, NC><<<bs, kThreads, 0, st>>>(d, p, q, t, g->sc, g->partials);
     prof_end(g, st, s);
     s = prof_begin(g, st, prof0 + 2);
@@ -1404,7 +1411,7 @@ void enqueue_pc2(mhd_grid_s* g, cudaStream_t st, int blocks) {
     k_pupdate<double, 2, NC, true><<<blocks, kThreads, 0, st>>>(d, z, g->p64, g->x64, g->sc);
     prof_end(g, st, ps);
     ps = prof_begin(g, st, MHD_KERNEL_SPMV64);
-    k_spmv_dot<double, 2, NC><<<blocks, kThreads, 0, st>>>(d, g->p64, g->q64, g->t64, g->sc, g->partials);
+    k_spmv_dot<double, 2, NC><<<spmv64_blocks(g, NC), kThreads, 0, st>>>(d, g->p64, g->q64, g->t64, g->sc, g->partials);
     prof_end(g, st, ps);
     ps = prof_begin(g, st, MHD_KERNEL_PC2);
     pc2_enqueue_line(g, st, NC, false);
@@ -1428,7 +1435,7 @@ void enqueue_pc2_32(mhd_grid_s* g, cudaStream_t st) {
                                                                                                 g->sc);
         prof_end(g, st, ps);
         ps = prof_begin(g, st, MHD_KERNEL_SPMV32);
-        k_spmv_dot<float, V, NC><<<grid_blocks(g, d.N / V, 6), kThreads, 0, st>>>(d, g->p32, g->q32, g->t32, g->sc,
+        k_spmv_dot<float, V, NC><<<grid_blocks(g, NC * (d.N / V), 6), kThreads, 0, st>>>(d, g->p32, g->q32, g->t32, g->sc,
                                                                                   g->partials);
         prof_end(g, st, ps);
     }
