@@ -12,7 +12,8 @@
 // Hestenes-Stiefel one of pcg.cu, same expressions and rounding:
 //   p = r + beta p                               | exchange 1: p visible to the neighbours
 //   q = A~ p, <p, q>                             | exchange 2: sum of <p, q>, alpha
-//   x += alpha p, r -= alpha q, <r, r>, sum dg r^2 | exchange 3: sums, beta, stop test
+//   r -= alpha q, <r, r>, sum dg r^2             | exchange 3: sums, beta, stop test; x += alpha p
+//                                                | before it (FP32) or meanwhile (FP64)
 //
 // Exchange 1 waits for the CTAs whose groups a chunk's stencil reads, one flag each. Exchanges 2 and 3
 // go through CTA 0: each CTA posts its partial sums in its own slot, a warp of CTA 0 reads the slots,
@@ -248,6 +249,7 @@ __global__ void __launch_bounds__(kPT, 1) k_persist(Dims d, unsigned int groups,
                                                     const double* __restrict__ dg, PcgScalars* sc, PersistBuf* buf,
                                                     int expect, unsigned long long budget_ns) {
     using VT = typename Vec<T, V>::type;
+    constexpr bool kLateX = sizeof(T) == 8;
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ PersistShared sh;
     if (sc->done) return;
@@ -407,23 +409,28 @@ __global__ void __launch_bounds__(kPT, 1) k_persist(Dims d, unsigned int groups,
         __syncthreads();
         if (sh.state) break;
         const T al = (T)sh.alpha;
+        auto add_x = [&](unsigned int l) {
+            T xv[V], pv[V];
+            get<T, V>(xs + l, xv);
+            get<T, V>(ps + l, pv);
+#pragma unroll
+            for (int e = 0; e < V; e++) xv[e] = fma(al, pv[e], xv[e]);
+            put<T, V>(xs + l, xv);
+        };
         Sum<T> a_rho;
         Sum<double> a_rr;
 #pragma unroll 2
         for (unsigned int l = threadIdx.x; l < n; l += blockDim.x) {
-            T xv[V], pv[V], rv[V], qv[V];
-            get<T, V>(xs + l, xv);
-            get<T, V>(ps + l, pv);
+            T rv[V], qv[V];
             get<T, V>(rs + l, rv);
             get<T, V>(qs + l, qv);
+            if constexpr (!kLateX) add_x(l);
             T cell = T(0);
 #pragma unroll
             for (int e = 0; e < V; e++) {
-                xv[e] = fma(al, pv[e], xv[e]);
                 rv[e] = fma(-al, qv[e], rv[e]);
                 cell = fma(rv[e], rv[e], cell);
             }
-            put<T, V>(xs + l, xv);
             put<T, V>(rs + l, rv);
             a_rho.add(cell);
             a_rr.s = fma(dgs[(g0 + l) / npv - row0], (double)cell, a_rr.s);
@@ -467,6 +474,13 @@ __global__ void __launch_bounds__(kPT, 1) k_persist(Dims d, unsigned int groups,
                 sh.state = state;
                 sh.beta = be64;
             }
+        } else if (kLateX && (threadIdx.x & 96)) {
+            // meanwhile x += alpha p, by the warps that share no scheduler with the first one, whose FP64 sums
+            // would queue behind theirs (warps are dealt to the four schedulers in turn). us per iteration:
+            // 32x32x64 13.5 -> 13.1, 48x48x96 23.5 -> 22.7, 61x47x118 30.7 -> 29.8; in FP32 it gave nothing.
+            const unsigned int w = threadIdx.x >> 5, helpers = nw - (nw + 3) / 4, at = w - 1 - w / 4;
+#pragma unroll 4
+            for (unsigned int l = 32 * at + lane; l < n; l += 32 * helpers) add_x(l);
         }
         __syncthreads();
         if (sh.state) break;
