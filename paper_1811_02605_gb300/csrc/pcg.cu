@@ -617,13 +617,16 @@ __global__ void __launch_bounds__(kThreads) k_update(Dims d, T* __restrict__ x,
 #pragma unroll
             for (int e = 0; e < V; e++) {
                 rv[e] = fma(-al, qv[e], rv[e]);
-                rs[e] = fma(rv[e], rv[e], rs[e]);
+                // FP64: one chain, without additions at its end (an instruction costs a scheduler's pipe 64 cycles)
+                if constexpr (sizeof(T) == 8) rs[0] = fma(rv[e], rv[e], rs[0]);
+                else rs[e] = fma(rv[e], rv[e], rs[e]);
             }
             stv<T, V>(r + k * d.N + off, rv);
         }
         T cell = rs[0];
 #pragma unroll
-        for (int e = 1; e < V; e++) cell += rs[e];
+        for (int e = 1; e < V; e++)
+            if constexpr (sizeof(T) == 4) cell += rs[e];
         a_rho.add(cell);
         a_rr = fma(dg[g / npv], (double)cell, a_rr);
     }
