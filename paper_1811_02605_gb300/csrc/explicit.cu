@@ -16,6 +16,7 @@
 //   - Tangential E is 0 on r0 (line-tied); on r1 it is the mean of the two interior cells.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "mhd_internal.cuh"
 #include "reduce.cuh"
@@ -31,7 +32,8 @@ namespace {
 // formed once a row; the means are kept as plain sums (B_c doubled, J_c and the edge E by powers of two, which
 // scale exactly) and the factor goes into a row constant; signs and maxima are integer tests; the upwind
 // difference is |u_d| / h (u - u_upwind), one form for both signs. Coefficients, force, induction with
-// resistivity and diagnostics of a 256x256x512 grid: 21.3 -> 13.9 ms, at about 200 FP64 instructions a cell and 82 to 89% of the pipe.
+// resistivity and diagnostics of a 256x256x512 grid: 21.3 -> 13.0 ms, at about 190 FP64 instructions a cell and 82 to
+// 89% of the pipe.
 __device__ __forceinline__ unsigned int first_row() {
     return blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
 }
@@ -64,12 +66,21 @@ struct FaceRow {
         if (j == 0) t0 = t1;        // the non-polar face on either side
         else if (j == d.nt - 1) t1 = t0;
     }
-    // twice the cell-centred B: sums of opposite faces; in the polar rings B_theta is the non-polar face and the
-    // pole value (first phi harmonic of the ring, see polar_btc)
+    // twice the cell-centred B: sums of opposite faces; in the polar rings (POLAR) B_theta is the non-polar face and
+    // the pole value (first phi harmonic of the ring, see polar_btc)
+    template <bool POLAR>
     __device__ __forceinline__ void twice(int k, int kp, double (&o)[3]) const {
         o[0] = r0[k] + r1[k];
-        o[1] = h ? t0[k] + (h[0] * pcs[k] + h[1] * pcs[np + k]) * pole_f : t0[k] + t1[k];
+        if constexpr (POLAR) o[1] = t0[k] + (h[0] * pcs[k] + h[1] * pcs[np + k]) * pole_f;
+        else o[1] = t0[k] + t1[k];
         o[2] = p0[k] + p0[kp];
+    }
+    // f(polar) with polar a compile-time truth value: a loop over the row of its own for the polar rings (the pole
+    // value as a choice within one loop takes its turns of the FP64 pipe in every row)
+    template <typename F>
+    __device__ __forceinline__ void over(F f) const {
+        if (h) f(std::true_type());
+        else f(std::false_type());
     }
 };
 
@@ -129,14 +140,16 @@ __global__ void __launch_bounds__(kThreads) k_coeffs(Dims d, Geo G, Vel<false> v
         const int i = (int)(ij / d.nt), j = (int)(ij - (unsigned int)i * d.nt);
         const FaceRow F(d, G, bh, br, bt, bp, i, j);
         long long mv = 0, mb = 0;
+        F.over([&](auto polar) {
 #pragma unroll 4
-        for (int k = threadIdx.x & 31; k < d.np; k += 32) {
-            double u[3], B[3];
-            v.at((long long)ij * d.np + k, u);
-            F.twice(k, kp1(d, k), B);
-            max_abs(mv, u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
-            max_abs(mb, B[0] * B[0] + B[1] * B[1] + B[2] * B[2]);
-        }
+            for (int k = threadIdx.x & 31; k < d.np; k += 32) {
+                double u[3], B[3];
+                v.at((long long)ij * d.np + k, u);
+                F.twice<decltype(polar)::value>(k, kp1(d, k), B);
+                max_abs(mv, u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+                max_abs(mb, B[0] * B[0] + B[1] * B[1] + B[2] * B[2]);
+            }
+        });
         const double kt2 = G.kt2[ij];
         mkv = fmax(mkv, kt2 * __longlong_as_double(mv));
         mka = fmax(mka, kt2 * (0.25 * __longlong_as_double(mb)) / G.rho[i]);
@@ -370,52 +383,56 @@ __global__ void __launch_bounds__(kThreads) k_force(Dims d, Geo G, ExTab X, Vel<
         const long long c_row = (long long)ij * d.np;
         const long long r_lo = i > 0 ? -plane : 0, r_hi = i < d.nr - 1 ? plane : 0;
         const long long t_lo = j > 0 ? -d.np : 0, t_hi = j < d.nt - 1 ? d.np : 0;
+        F.over([&](auto polar) {
 #pragma unroll 1
-        for (int k = threadIdx.x & 31; k < d.np; k += 32) {
-            const long long c = c_row + k;
-            const int kp = kp1(d, k), km = km1(d, k);
-            double u[3], n[3], adv[3], B[3], J[3];
-            v.at(c, u);
-            const bool ur = positive(u[0]), ut = positive(u[1]), up = positive(u[2]);
-            F.twice(k, kp, B);
-            E.four(k, kp, J);
-            {
-                v.at(c + (ur ? r_lo : r_hi), n);
-                if (i == 0 && ur)
-                    for (int m = 0; m < 3; m++) n[m] = -n[m];
-                const double a = fabs(u[0]) * (ur ? ir_lo : ir_hi);
+            for (int k = threadIdx.x & 31; k < d.np; k += 32) {
+                const long long c = c_row + k;
+                const int kp = kp1(d, k), km = km1(d, k);
+                double u[3], n[3], adv[3], B[3], J[3];
+                v.at(c, u);
+                const bool ur = positive(u[0]), ut = positive(u[1]), up = positive(u[2]);
+                F.twice<decltype(polar)::value>(k, kp, B);
+                E.four(k, kp, J);
+                {
+                    v.at(c + (ur ? r_lo : r_hi), n);
+                    // (the ghost's sign by its bit: three negations would be FP64 instructions of every row)
+                    const long long ghost = i == 0 && ur ? (long long)0x8000000000000000ull : 0ll;
 #pragma unroll
-                for (int m = 0; m < 3; m++) adv[m] = a * (u[m] - n[m]);
-            }
-            {
-                v.at(c + (ut ? t_lo : t_hi), n);
-                const double a = fabs(u[1]) * iht;
+                    for (int m = 0; m < 3; m++) n[m] = __longlong_as_double(__double_as_longlong(n[m]) ^ ghost);
+                    const double a = fabs(u[0]) * (ur ? ir_lo : ir_hi);
 #pragma unroll
-                for (int m = 0; m < 3; m++) adv[m] = fma(a, u[m] - n[m], adv[m]);
-            }
-            {
-                v.at(c_row + (up ? km : kp), n);
-                const double a = fabs(u[2]) * ihp;
+                    for (int m = 0; m < 3; m++) adv[m] = a * (u[m] - n[m]);
+                }
+                {
+                    v.at(c + (ut ? t_lo : t_hi), n);
+                    const double a = fabs(u[1]) * iht;
 #pragma unroll
-                for (int m = 0; m < 3; m++) adv[m] = fma(a, u[m] - n[m], adv[m]);
+                    for (int m = 0; m < 3; m++) adv[m] = fma(a, u[m] - n[m], adv[m]);
+                }
+                {
+                    v.at(c_row + (up ? km : kp), n);
+                    const double a = fabs(u[2]) * ihp;
+#pragma unroll
+                    for (int m = 0; m < 3; m++) adv[m] = fma(a, u[m] - n[m], adv[m]);
+                }
+                // spherical curvature terms
+                const double a1 = u[1] * irc, a2 = u[2] * irc, c2 = u[2] * cot;
+                adv[0] = fma(-u[1], a1, fma(-u[2], a2, adv[0]));
+                adv[1] = fma(u[0], a1, fma(-c2, a2, adv[1]));
+                adv[2] = fma(u[0], a2, fma(c2, a1, adv[2]));
+                double f0 = s * fma(J[1] * B[2] - J[2] * B[1], irho8, -adv[0]);
+                double f1 = s * fma(J[2] * B[0] - J[0] * B[2], irho8, -adv[1]);
+                double f2 = s * fma(J[0] * B[1] - J[1] * B[0], irho8, -adv[2]);
+                if constexpr (AVG) {
+                    f0 = fma(0.5, b_avg[c], f0);
+                    f1 = fma(0.5, b_avg[d.N + c], f1);
+                    f2 = fma(0.5, b_avg[2 * d.N + c], f2);
+                }
+                b[c] = f0;
+                b[d.N + c] = f1;
+                b[2 * d.N + c] = f2;
             }
-            // spherical curvature terms
-            const double a1 = u[1] * irc, a2 = u[2] * irc, c2 = u[2] * cot;
-            adv[0] = fma(-u[1], a1, fma(-u[2], a2, adv[0]));
-            adv[1] = fma(u[0], a1, fma(-c2, a2, adv[1]));
-            adv[2] = fma(u[0], a2, fma(c2, a1, adv[2]));
-            double f0 = s * fma(J[1] * B[2] - J[2] * B[1], irho8, -adv[0]);
-            double f1 = s * fma(J[2] * B[0] - J[0] * B[2], irho8, -adv[1]);
-            double f2 = s * fma(J[0] * B[1] - J[1] * B[0], irho8, -adv[2]);
-            if constexpr (AVG) {
-                f0 = fma(0.5, b_avg[c], f0);
-                f1 = fma(0.5, b_avg[d.N + c], f1);
-                f2 = fma(0.5, b_avg[2 * d.N + c], f2);
-            }
-            b[c] = f0;
-            b[d.N + c] = f1;
-            b[2 * d.N + c] = f2;
-        }
+        });
     }
 }
 
@@ -457,27 +474,29 @@ __global__ void __launch_bounds__(kThreads) k_ecentre(Dims d, Geo G, Vel<DLT> v,
         const int i = (int)(ij / d.nt), j = (int)(ij - (unsigned int)i * d.nt);
         const FaceRow F(d, G, bh, br, bt, bp, i, j);
         const EdgeRow E(d, jr, jt, jp, i, j);
+        F.over([&](auto polar) {
 #pragma unroll 2
-        for (int k = threadIdx.x & 31; k < d.np; k += 32) {
-            const long long c = (long long)ij * d.np + k;
-            const int kp = kp1(d, k);
-            double u[3], B[3];
-            v.at(c, u);
-            F.twice(k, kp, B);
-            double e0 = u[2] * B[1] - u[1] * B[2];
-            double e1 = u[0] * B[2] - u[2] * B[0];
-            double e2 = u[1] * B[0] - u[0] * B[1];
-            if constexpr (ETA) {
-                double J[3];
-                E.four(k, kp, J);
-                e0 = fma(eta_h, J[0], e0);
-                e1 = fma(eta_h, J[1], e1);
-                e2 = fma(eta_h, J[2], e2);
+            for (int k = threadIdx.x & 31; k < d.np; k += 32) {
+                const long long c = (long long)ij * d.np + k;
+                const int kp = kp1(d, k);
+                double u[3], B[3];
+                v.at(c, u);
+                F.twice<decltype(polar)::value>(k, kp, B);
+                double e0 = u[2] * B[1] - u[1] * B[2];
+                double e1 = u[0] * B[2] - u[2] * B[0];
+                double e2 = u[1] * B[0] - u[0] * B[1];
+                if constexpr (ETA) {
+                    double J[3];
+                    E.four(k, kp, J);
+                    e0 = fma(eta_h, J[0], e0);
+                    e1 = fma(eta_h, J[1], e1);
+                    e2 = fma(eta_h, J[2], e2);
+                }
+                ec[c] = e0;
+                ec[d.N + c] = e1;
+                ec[2 * d.N + c] = e2;
             }
-            ec[c] = e0;
-            ec[d.N + c] = e1;
-            ec[2 * d.N + c] = e2;
-        }
+        });
     }
 }
 
@@ -646,20 +665,22 @@ __global__ void __launch_bounds__(kThreads) k_diag(Dims d, Geo G, ExTab X, Vel<f
         const double ap = ring * G.dth, V = G.rhoV[ij] * X.sh[5 * (size_t)i + 3];
         double sb = 0.0, su = 0.0, sx = 0.0, sd = 0.0;
         long long mf = 0;
+        F.over([&](auto polar) {
 #pragma unroll 1
-        for (int k = threadIdx.x & 31; k < d.np; k += 32) {
-            const int kp = kp1(d, k);
-            double u[3], B[3], J[3];
-            v.at((long long)ij * d.np + k, u);
-            F.twice(k, kp, B);
-            E.four(k, kp, J);
-            const double x0 = J[1] * B[2] - J[2] * B[1], x1 = J[2] * B[0] - J[0] * B[2], x2 = J[0] * B[1] - J[1] * B[0];
-            sb = fma(B[0], B[0], fma(B[1], B[1], fma(B[2], B[2], sb)));
-            su = fma(u[0], u[0], fma(u[1], u[1], fma(u[2], u[2], su)));
-            sx += sqrt(x0 * x0 + x1 * x1 + x2 * x2);
-            sd += fabs(J[0] * B[0] + J[1] * B[1] + J[2] * B[2]);
-            max_abs(mf, F.r1[k] * aro - F.r0[k] * ari + t1[k] * atj1 - t0[k] * atj + (F.p0[kp] - F.p0[k]) * ap);
-        }
+            for (int k = threadIdx.x & 31; k < d.np; k += 32) {
+                const int kp = kp1(d, k);
+                double u[3], B[3], J[3];
+                v.at((long long)ij * d.np + k, u);
+                F.twice<decltype(polar)::value>(k, kp, B);
+                E.four(k, kp, J);
+                const double x0 = J[1] * B[2] - J[2] * B[1], x1 = J[2] * B[0] - J[0] * B[2], x2 = J[0] * B[1] - J[1] * B[0];
+                sb = fma(B[0], B[0], fma(B[1], B[1], fma(B[2], B[2], sb)));
+                su = fma(u[0], u[0], fma(u[1], u[1], fma(u[2], u[2], su)));
+                sx += sqrt(x0 * x0 + x1 * x1 + x2 * x2);
+                sd += fabs(J[0] * B[0] + J[1] * B[1] + J[2] * B[2]);
+                max_abs(mf, F.r1[k] * aro - F.r0[k] * ari + t1[k] * atj1 - t0[k] * atj + (F.p0[kp] - F.p0[k]) * ap);
+            }
+        });
         // the sums hold 4 B^2 and 8 times the products of J and B
         em = fma(0.125 * V, sb, em);
         ek = fma(0.5 * G.rho[i] * V, su, ek);
