@@ -59,9 +59,9 @@ FP64_INSTR_PEAK = 2 * 152 * 2.070e9
 # D_{j-2} and ly0 read, D_j written = 4 x 3 x 8 B
 STS_FLOPS_PER_CELL = 3 * 16 + 3
 STS_BYTES_PER_CELL = 4 * 3 * 8
-# FP64 PC2 line kernel per cell: r, q read, r, z written (4 x 3 x 8 B) plus 1/dt (8 B,
+# FP64 PC2 line kernel per cell: x, p, r, q read, x, r, z written (7 x 3 x 8 B) plus 1/dt (8 B,
 # shared by the three components)
-PC2_LINE_BYTES_PER_CELL = 4 * 3 * 8 + 8
+PC2_LINE_BYTES_PER_CELL = 7 * 3 * 8 + 8
 # resistivity of the explicit-against-implicit comparison (the workload itself has eta = 0)
 RES_ETA = 1e-3
 
