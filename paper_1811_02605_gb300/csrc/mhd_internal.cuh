@@ -71,6 +71,7 @@ struct StepScalars {
     double dt, cf, cw, alpha_si, alpha_nu;
     double max_kv2, max_kva2, max_kt2;
     double alpha_user;   // alpha of a direct operator/solver call
+    double alpha_trial;  // alpha of the timed trial iterations that choose the kernel forms
     int status;      // MHD_OK or MHD_ERR_ARG (C_f >= 1 / no dt)
     unsigned int count;
 };

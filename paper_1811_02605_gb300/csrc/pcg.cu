@@ -1562,13 +1562,15 @@ void enqueue_first_residual(mhd_grid_s* g) {
     prof_end(g, g->stream, s);
 }
 
+void enqueue_first_residual_nc(mhd_grid_s* g, int nc) {
+    if (nc == 3) enqueue_first_residual<3>(g);
+    else if (nc == 2) enqueue_first_residual<2>(g);
+    else enqueue_first_residual<1>(g);
+}
+
 // run batches of iterations until the device flags completion
 mhd_status_t run_iterations(mhd_grid_s* g, int prec, int nc) {
-    if (prec == 1 && g->slab32 == -10) {
-        if (nc == 3) enqueue_first_residual<3>(g);
-        else if (nc == 2) enqueue_first_residual<2>(g);
-        else enqueue_first_residual<1>(g);
-    }
+    if (prec == 1 && g->slab32 == -10) enqueue_first_residual_nc(g, nc);
     cudaGraphExec_t ge = nullptr;
     if (!g->prof) {
         mhd_status_t st = iteration_graph(g, prec, nc, &ge);
@@ -1634,12 +1636,49 @@ __global__ void k_tune_reset(PcgScalars* sc, int max_iter = 1 << 30) {
     sc->total_iter = 0;
     sc->par = 0;
     sc->ax = 0.0;
+    sc->pq = 0.0;
+    sc->wp = 0.0;
     sc->count = 0u;
 }
 
-// choose the r-slab length of the tiled FP32 kernels by timing a few iterations of each
-// candidate (alpha = beta = 0, so the vectors are left as they are); run before a solve sets up
-// its scalars
+__global__ void k_set_value(double* a, double v) { *a = v; }
+
+// a residual with every frequency in it, between 1/2 and 1
+template <typename T>
+__global__ void k_trial_fill(T* __restrict__ a, unsigned int n) {
+    for (unsigned int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+        a[i] = T(0.5) + T((i * 2654435761u) >> 9) * T(1.0 / (1 << 24));
+}
+
+// The system of the timed trial iterations: the operator of alpha = 100 over the bound on the spectrum of D^-1 K,
+// whatever the alpha of the solve that comes first. Its eigenvalues spread over two decades at most, so that neither
+// a trial converges (at alpha = 0 the scaled operator is the identity, and CG on it ends after one iteration) nor
+// FP32 runs out of digits. Run before a solve builds its own tables.
+mhd_status_t trial_tables(mhd_grid_s* g, bool fp32) {
+    k_set_value<<<1, 1, 0, g->stream>>>(&g->ss->alpha_trial, 100.0 / g->visc_lambda_unit);
+    build_tables(g, &g->ss->alpha_trial, fp32);
+    return check_cuda(g, "tune: tables");
+}
+void trial_vectors32(mhd_grid_s* g) {
+    const size_t n3 = 3 * (size_t)g->d.N;
+    k_trial_fill<<<grid_blocks(g, 3 * g->d.N, 8), kThreads, 0, g->stream>>>(g->r32, (unsigned int)n3);
+    cudaMemsetAsync(g->p32, 0, sizeof(float) * 2 * n3, g->stream);
+    cudaMemsetAsync(g->x32, 0, sizeof(float) * n3, g->stream);
+}
+void trial_vectors64(mhd_grid_s* g) {
+    const size_t n3 = 3 * (size_t)g->d.N;
+    k_trial_fill<<<grid_blocks(g, 3 * g->d.N, 8), kThreads, 0, g->stream>>>(g->r64, (unsigned int)n3);
+    cudaMemsetAsync(g->p64, 0, sizeof(double) * 2 * n3, g->stream);
+    cudaMemsetAsync(g->x64, 0, sizeof(double) * n3, g->stream);
+}
+// Kernels return at once after a solve has ended, so a trial is a measurement only if it ran all its iterations
+// (done: how it ends then).
+bool trial_ran(mhd_grid_s* g, int iters, int done = 0) {
+    return read_scalars(g) == MHD_OK && g->h_sc->iter == iters && g->h_sc->done == done;
+}
+
+// choose the FP32 kernel form by timing a few iterations of each candidate; run before a solve sets up its
+// tables and scalars
 // Diagnostics: MHD_FORCE_SLAB=<n> skips the timing and uses slab n (-1: split kernels, -2 (FP32
 // only): the p update folded into the stencil).
 int forced_slab() {
@@ -1653,9 +1692,11 @@ int forced_slab() {
 constexpr long long kPersistTrial = 2500000;
 
 // milliseconds per iteration of the persistent kernel over 8 iterations, one untimed launch before
-// (huge when it cannot run); the vectors hold the trial values
+// (huge when it cannot run)
 float time_persist(mhd_grid_s* g, bool fp32, int nc, cudaEvent_t e0, cudaEvent_t e1) {
     if (!persist_mode(g, fp32, nc)) return 1e30f;
+    if (fp32) trial_vectors32(g);
+    else trial_vectors64(g);
     for (int warm = 1; warm >= 0; warm--) {
         k_tune_reset<<<1, 1, 0, g->stream>>>(g->sc, 8);
         if (!warm) cudaEventRecord(e0, g->stream);
@@ -1664,7 +1705,7 @@ float time_persist(mhd_grid_s* g, bool fp32, int nc, cudaEvent_t e0, cudaEvent_t
     }
     float ms = 0.f;
     if (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) return 1e30f;
-    return ms / 8.f;
+    return trial_ran(g, 8, 2) ? ms / 8.f : 1e30f;   // ended by max_iter
 }
 
 mhd_status_t tune_slab32(mhd_grid_s* g, int nc) {
@@ -1684,15 +1725,14 @@ mhd_status_t tune_slab32(mhd_grid_s* g, int nc) {
         g->slab32 = -9;
         return MHD_OK;
     }
+    if (const mhd_status_t st = trial_tables(g, true)) return st;
     cudaEvent_t e0, e1;
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) return check_cuda(g, "tune events");
     int best = 0;
     float best_ms = 1e30f;
     const int prof = g->prof;
     g->prof = 0;
-    // positive finite vectors (bytes 0x3F: 0.747f) so the timed iterations do real work and no
-    // reduction trips a breakdown flag (the solve's set-up overwrites every vector afterwards)
-    const size_t n3 = 3 * (size_t)g->d.N;
+    // (the solve's set-up overwrites every vector afterwards)
     // candidates -1: the split kernels (p update, stencil, update); -2: the p update folded into
     // the stencil, then the update; -3, -4, -5: the recompute pair (no q~ stored), forwards, with
     // the r update walking backwards, or at 6 CTAs per SM; -6, -7, -8: the single-reduction pair
@@ -1709,9 +1749,10 @@ mhd_status_t tune_slab32(mhd_grid_s* g, int nc) {
         if (cand <= -100 && !bulk32_ok(g)) continue;
         k_tune_reset<<<1, 1, 0, g->stream>>>(g->sc);
         g->slab32 = cand;
-        cudaMemsetAsync(g->r32, 0x3F, sizeof(float) * n3, g->stream);
-        cudaMemsetAsync(g->p32, 0x3F, sizeof(float) * 2 * n3, g->stream);
-        cudaMemsetAsync(g->x32, 0, sizeof(float) * n3, g->stream);
+        trial_vectors32(g);
+        // the marching iterations go on from the residual kernel's scalars, as in a solve: without them the next
+        // <p, A p> that they predict can come out negative, which ends the trial
+        if (cand == -10) enqueue_first_residual_nc(g, nc);
         enqueue_iteration(g, g->stream, 1, nc);
         cudaEventRecord(e0, g->stream);
         for (int it = 0; it < 4; it++) enqueue_iteration(g, g->stream, 1, nc);
@@ -1720,13 +1761,12 @@ mhd_status_t tune_slab32(mhd_grid_s* g, int nc) {
         float ms = 0.f;
         cudaEventElapsedTime(&ms, e0, e1);
         ms *= 0.75f;   // per 3 iterations, as the tiled candidates below
-        if (ms < best_ms) {
+        if (ms < best_ms && trial_ran(g, 5)) {
             best_ms = ms;
             best = cand;
         }
     }
-    cudaMemsetAsync(g->r32, 0x3F, sizeof(float) * n3, g->stream);
-    cudaMemsetAsync(g->p32, 0x3F, sizeof(float) * 2 * n3, g->stream);
+    trial_vectors32(g);
     for (int slab : {8, 16, 32, 64}) {
         if (march || !tiled32_ok(g)) break;
         if (slab > 2 * g->d.nr && best > 0) break;
@@ -1739,29 +1779,24 @@ mhd_status_t tune_slab32(mhd_grid_s* g, int nc) {
         if (cudaEventSynchronize(e1) != cudaSuccess) break;
         float ms = 0.f;
         cudaEventElapsedTime(&ms, e0, e1);
-        if (ms < best_ms) {
+        if (ms < best_ms && trial_ran(g, 4)) {
             best_ms = ms;
             best = slab;
         }
     }
-    if (g->d.N <= kPersistTrial) {
-        cudaMemsetAsync(g->r32, 0x3F, sizeof(float) * n3, g->stream);
-        cudaMemsetAsync(g->p32, 0x3F, sizeof(float) * 2 * n3, g->stream);
-        if (3.f * time_persist(g, true, nc, e0, e1) < best_ms) best = -9;
-    }
+    if (g->d.N <= kPersistTrial && 3.f * time_persist(g, true, nc, e0, e1) < best_ms) best = -9;
     g->prof = prof;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    if (best == 0) return set_error(g, MHD_ERR_CUDA, "FP32 CG kernels: no launchable variant");
-    g->slab32 = best;  // -1 split, -2 folded, -3/-4 recompute pair, -9 persistent, -10 marching,
+    g->slab32 = (best == 0) ? -1 : best;  // -1 split, -2 folded, -3/-4 recompute pair, -9 persistent, -10 marching,
                        // <= -100 bulk-staged pair, > 0 tiled slab
     return check_cuda(g, "tune slab");
 }
 }  // namespace
 
 namespace {
-// FP64: time the split iteration against the fused tiled kernel A at each slab length (alpha =
-// beta = 0 on positive finite vectors) and keep the fastest
+// FP64: time the split iteration, the overlapped one, the fused tiled kernel A at each slab length and the
+// persistent kernel, and keep the fastest
 mhd_status_t tune_slab64(mhd_grid_s* g) {
     if (g->slab64 != 0) return MHD_OK;
     if (const int f = forced_slab()) {
@@ -1776,13 +1811,11 @@ mhd_status_t tune_slab64(mhd_grid_s* g) {
         g->slab64 = -3;
         return MHD_OK;
     }
+    if (const mhd_status_t st = trial_tables(g, false)) return st;
     cudaEvent_t e0, e1;
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) return check_cuda(g, "tune events");
     const int prof = g->prof;
     g->prof = 0;
-    const size_t n3 = 3 * (size_t)g->d.N;
-    cudaMemsetAsync(g->r64, 0x3F, sizeof(double) * n3, g->stream);
-    cudaMemsetAsync(g->p64, 0x3F, sizeof(double) * 2 * n3, g->stream);
     int best = 0;
     float best_ms = 1e30f;
     for (int slab : {-1, -2, 8, 16, 32, 64}) {
@@ -1790,6 +1823,7 @@ mhd_status_t tune_slab64(mhd_grid_s* g) {
         if (slab > 0 && (!tiled32_ok(g) || tiled32_blocks(g, slab) > kMaxBlocks || (slab > 2 * g->d.nr && best != 0)))
             continue;
         g->slab64 = slab;
+        trial_vectors64(g);
         k_tune_reset<<<1, 1, 0, g->stream>>>(g->sc);
         enqueue_iteration(g, g->stream, 0, 3);
         cudaEventRecord(e0, g->stream);
@@ -1798,36 +1832,24 @@ mhd_status_t tune_slab64(mhd_grid_s* g) {
         if (cudaEventSynchronize(e1) != cudaSuccess) break;
         float ms = 0.f;
         cudaEventElapsedTime(&ms, e0, e1);
-        if (ms < best_ms) {
+        if (ms < best_ms && trial_ran(g, 3)) {
             best_ms = ms;
             best = slab;
         }
     }
-    if (g->d.N <= kPersistTrial) {
-        cudaMemsetAsync(g->r64, 0x3F, sizeof(double) * n3, g->stream);
-        cudaMemsetAsync(g->p64, 0x3F, sizeof(double) * 2 * n3, g->stream);
-        if (2.f * time_persist(g, false, 3, e0, e1) < best_ms) best = -3;
-    }
+    if (g->d.N <= kPersistTrial && 2.f * time_persist(g, false, 3, e0, e1) < best_ms) best = -3;
     g->prof = prof;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     g->slab64 = (best == 0) ? -1 : best;
-    cudaMemsetAsync(g->p64, 0, sizeof(double) * 2 * n3, g->stream);
+    cudaMemsetAsync(g->p64, 0, sizeof(double) * 6 * (size_t)g->d.N, g->stream);
     return check_cuda(g, "tune slab64");
 }
 }  // namespace
 
-namespace {
-__global__ void k_set_unit(double* a) { *a = 1.0; }
-}  // namespace
-
-// kernel choices and CUDA graphs of 3-component solves, ahead of the first solve (mhd_grid_reserve);
-// the tables are built for alpha = 1 so the timed trial iterations run on finite coefficients
+// kernel choices and CUDA graphs of 3-component solves, ahead of the first solve (mhd_grid_reserve)
 mhd_status_t solver_reserve(mhd_grid_s* g, int features) {
-    k_set_unit<<<1, 1, 0, g->stream>>>(&g->ss->alpha_user);
-    build_tables(g, &g->ss->alpha_user, true);
-    mhd_status_t st = check_cuda(g, "reserve: tables");
-    if (st != MHD_OK) return st;
+    mhd_status_t st = MHD_OK;
     cudaGraphExec_t ge = nullptr;
     if (features & MHD_RESERVE_PC1) {
         if (g->slab64 == 0 && (st = tune_slab64(g)) != MHD_OK) return st;
@@ -1856,7 +1878,6 @@ mhd_status_t solve(mhd_grid_s* g, const double* alpha_dev, int nc, const double*
                    const double* x0, const mhd_params_t* prm, int* iters, int* outer, double* relres) {
     const Dims d = g->d;
     const bool mixed = (prm->precision == MHD_PREC_MIXED);
-    build_tables(g, alpha_dev, mixed);
     const bool pc2 = (prm->preconditioner == 1);
     if (mixed && g->slab32 == 0 && !pc2) {
         mhd_status_t st = tune_slab32(g, 3);
@@ -1866,6 +1887,7 @@ mhd_status_t solve(mhd_grid_s* g, const double* alpha_dev, int nc, const double*
         mhd_status_t st = tune_slab64(g);
         if (st != MHD_OK) return st;
     }
+    build_tables(g, alpha_dev, mixed);
     k_setup<<<1, 1, 0, g->stream>>>(g->sc, prm->tol, prm->inner_tol, prm->max_iter);
     const int blocks2 = grid_blocks(g, d.N / 2, kPerSmIter);
     if (!mixed) {
