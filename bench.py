@@ -59,9 +59,14 @@ FP64_INSTR_PEAK = 2 * 152 * 2.070e9
 # D_{j-2} and ly0 read, D_j written = 4 x 3 x 8 B
 STS_FLOPS_PER_CELL = 3 * 16 + 3
 STS_BYTES_PER_CELL = 4 * 3 * 8
-# FP64 PC2 line kernel per cell: x, p, r, q read, x, r, z written (7 x 3 x 8 B) plus 1/dt (8 B,
-# shared by the three components)
+# flops per cell of a whole FP64 iteration: p and x updates, stencil, r update with r~^2 (2 flops each of the p, x, r and
+# r~^2 multiply-adds of a component), sum dg r~^2 per cell
+PCG64_FLOPS_PER_CELL_ITER = SPMV_FLOPS_PER_CELL + 3 * 4 * 2 + 2
+# FP64 PC2 preconditioner step per cell, x update included: x, p, r, q read, x, r, z written (7 x 3 x 8 B) plus 1/dt
+# (8 B, shared by the three components)
 PC2_LINE_BYTES_PER_CELL = 7 * 3 * 8 + 8
+# what the line kernel itself moves, the x update left to the next p update: r, q read, r, z written, and 1/dt
+PC2_LINE_MOVED_BYTES_PER_CELL = 4 * 3 * 8 + 8
 # resistivity of the explicit-against-implicit comparison (the workload itself has eta = 0)
 RES_ETA = 1e-3
 
@@ -271,6 +276,102 @@ def run_reference(args):
 
 
 # ----------------------------------------------------------------------------------------------
+# bandwidth and roofline of a profiled run: `prof` maps a kernel's name to (milliseconds, launches)
+# ----------------------------------------------------------------------------------------------
+def pcg64_account(prof, iters, N, hbm, form, iter_ms, iter_n):
+    """FP64 point-Jacobi PCG of `iters` iterations in the kernel form `form`, iter_ms an unprofiled
+    iteration: milliseconds, algorithmic GB/s, per-kernel table, roofline entry."""
+    overlap, persist = form == -2, form == -3
+    peak = FP64_PEAK_TFLOPS / 1e3
+    pcg_ms = sum(prof[k][0] for k in ("pupdate64", "spmv64", "update64", "persist64"))
+    gbs = PCG_BYTES_PER_CELL["fp64"] * N * iters / (pcg_ms * 1e-3) / 1e9
+    if overlap:   # concurrent kernels: the unprofiled iteration time, not the sum of launch times
+        gbs = PCG_BYTES_PER_CELL["fp64"] * N / (iter_ms * 1e-3) / 1e9
+    # per-kernel DRAM passes of a 3-component FP64 vector (8 B x 3 per cell per pass): the p update
+    # also adds the previous alpha p to x (r, p, x in; p, x out), the update reads r, q and writes r;
+    # the persistent form is one launch a solve, listed by iteration with the algorithmic 6 passes (its
+    # vectors stay in shared memory where they fit)
+    kernels = {}
+    for k, passes in (("pupdate64", 5), ("spmv64", 2), ("update64", 3), ("persist64", 6)):
+        ms_k, n_k = prof[k]
+        if n_k:
+            avg = ms_k / iters
+            kg = passes * 24 * N / (avg * 1e-3) / 1e9
+            kernels[k] = dict(avg_launch_ms=round(ms_k / n_k if k == "persist64" else avg, 4), bytes_per_cell=passes * 24,
+                              gbs=round(kg, 1), frac_of_hbm=round(kg / hbm, 4))
+            if k == "persist64":
+                kernels[k]["ms_per_iteration"] = round(avg, 4)
+    if persist:
+        # all iterations of a solve in one launch: the whole iteration's flops
+        avg, kernel = prof["persist64"][0] / iters, "k_persist<double,2> (all iterations of a solve; times are per iteration)"
+        tflops = PCG64_FLOPS_PER_CELL_ITER * N / (avg * 1e-3) / 1e12
+    elif overlap:
+        # one stencil launch per component, each overlapping the next component's p update
+        avg, kernel = prof["spmv64"][0] / max(prof["spmv64"][1], 1), \
+            "k_spmv_dotc<2> (one component per launch, beside the next component's p update)"
+        tflops = SPMV_FLOPS_PER_CELL / 3 * N / (avg * 1e-3) / 1e12
+    else:
+        avg, kernel = prof["spmv64"][0] / max(min(prof["spmv64"][1], iters), 1), "k_spmv_dot<double,2,3>"
+        tflops = SPMV_FLOPS_PER_CELL * N / (avg * 1e-3) / 1e12
+    roof = dict(bound="alu", achieved=round(tflops, 4), peak=round(peak, 4), unit="TFLOP/s", frac=round(tflops / peak, 4),
+                traffic=(int(SPMV64_DRAM_BYTES_PER_CELL * N) if prof["pupdate64"][1] and not overlap else None),
+                traffic_algorithmic=(None if persist else int(SPMV_BYTES_PER_CELL["fp64"] * N / (3 if overlap else 1))),
+                kernel=kernel, avg_launch_ms=round(avg, 4),
+                iteration=dict(fp64_instr_per_cell=FP64_INSTR_PER_CELL_ITER, ms=round(iter_ms, 4),
+                               fp64_pipe_frac=round(FP64_INSTR_PER_CELL_ITER * N / (iter_ms * 1e-3)
+                                                    / FP64_INSTR_PEAK, 4),
+                               form=form,
+                               note=f"the whole FP64 CG iteration (p update, stencil, update), timed unprofiled "
+                                    f"over a {iter_n}-iteration solve of the first step's SI system, against the "
+                                    f"part's FP64 instruction rate"),
+                peak_source="2 DFMA/clk/SM x 152 SMs x 2.07 GHz (nominal FP64 rate of the part)")
+    return pcg_ms, gbs, kernels, roof
+
+
+def pcg32_account(prof, iters, N, hbm):
+    """FP32 inner PCG of a mixed run, `iters` inner iterations: algorithmic GB/s, per-kernel table, the
+    kernel form's name."""
+    names = ("pupdate32", "spmv32", "pspmv32", "update32", "pfold32", "rupd32", "cgr32", "cgu32", "march32", "persist32")
+    ran = {k: prof[k][1] > 0 for k in names}
+    gbs = PCG_BYTES_PER_CELL["fp32"] * N * iters / (sum(prof[k][0] for k in names) * 1e-3) / 1e9
+    tiled = ran["update32"] and not ran["pupdate32"] and not ran["pspmv32"]
+    form = ("one plane-marching kernel (single-reduction iteration; the residual kernel ahead of each inner solve)"
+            if ran["march32"] else
+            "one persistent launch per inner solve" if ran["persist32"] else
+            "plane-marching pair (A: p update + stencil, B: stencil + update)" if tiled else
+            "single-reduction pair (residual kernel: gamma, delta, stop norm; update kernel: p, A p, r, x every second "
+            "iteration)" if ran["cgr32"] else
+            "recompute pair (p update folded into <p, Ap>; r update with Ap recomputed, x every second iteration)"
+            if ran["pfold32"] else
+            "p update folded into the stencil, then the update" if ran["pspmv32"] else
+            "split (p update, stencil, update)")
+    # per-kernel DRAM passes of a 3-component FP32 vector (4 B x 3 per cell per pass)
+    # split form: the p update also adds the previous alpha p to x (r, p, x in; p, x out) and the
+    # update kernel reads r, q and writes r; fused form: r, p, x in, p, x, q out, then the update;
+    # recompute pair: r, p_old in, p out; then p, r in, r out, and every second iteration x,
+    # p_prev in, x out (4.5 on average); single-reduction pair: r in; then r, p_old in, p, r out,
+    # and every second iteration x in and out (5 on average), which is also what the marching kernel
+    # moves; persistent form: the algorithmic 6 (its vectors stay in shared memory where they fit)
+    kb = {"spmv32": 3 if tiled else 2, "update32": 5 if tiled else 3, "pupdate32": 5, "pspmv32": 6,
+          "pfold32": 3, "rupd32": 4.5, "cgr32": 1, "cgu32": 5, "march32": 5, "persist32": 6}
+    kernels = {}
+    for k in names:
+        ms_k, n_k = prof[k]
+        if not n_k:
+            continue
+        # one launch per inner iteration that ran, except: the persistent kernel and, beside the marching
+        # kernel, the residual kernel are launched once per inner solve
+        once = k == "persist32" or (k == "cgr32" and ran["march32"])
+        avg = ms_k / iters
+        kg = kb[k] * 12 * N / ((ms_k / n_k if once and k == "cgr32" else avg) * 1e-3) / 1e9
+        kernels[k] = dict(avg_launch_ms=round(ms_k / n_k if once else avg, 4), bytes_per_cell=kb[k] * 12, gbs=round(kg, 1),
+                          frac_of_hbm=round(kg / hbm, 4))
+        if k == "persist32":
+            kernels[k]["ms_per_iteration"] = round(avg, 4)
+    return gbs, kernels, form
+
+
+# ----------------------------------------------------------------------------------------------
 # our arm
 # ----------------------------------------------------------------------------------------------
 def run_ours(args):
@@ -360,13 +461,9 @@ def run_ours(args):
     psteps = max(1, min(args.steps, args.profile_steps))
     ms64p, infos64, prof64, clk64p, ds64p = run(P.PREC_FP64, psteps, 1, True)
     ms64p = maxr(ms64p)
-    spmv_ms, spmv_n = prof64["spmv64"]
-    pcg64_ms = sum(prof64[k][0] for k in ("pupdate64", "spmv64", "update64"))
-    pcg64_n = prof64["spmv64"][1]
     it64_total = max(sum(sum(i["iters"]) for i in infos64), 1)   # CG iterations actually run
     # share of the FP64 PCG time spent in the viscous solves (by iteration count)
     visc_it = sum(i["iters"][2] for i in infos64)
-    visc64_ms = pcg64_ms * visc_it / it64_total / len(infos64)
     form64, _ = P.mhd_grid_kernel_forms(g)
     overlap64 = form64 == -2
     # ms per FP64 CG iteration, unprofiled: a fixed-count solve of the first step's SI system (the
@@ -388,68 +485,14 @@ def run_ours(args):
     barrier()
     iter64_ms = maxr(ea.elapsed_time(eb)) / iter_n
     del ds_i, f_i, b_i, x_i
-    if overlap64:
-        # one stencil launch per component, each overlapping the next component's p update
-        spmv_avg = spmv_ms / max(spmv_n, 1)
-        spmv_tflops = SPMV_FLOPS_PER_CELL / 3 * N / (spmv_avg * 1e-3) / 1e12
-    else:
-        spmv_avg = spmv_ms / max(min(spmv_n, sum(sum(i["iters"]) for i in infos64)), 1)
-        spmv_tflops = SPMV_FLOPS_PER_CELL * N / (spmv_avg * 1e-3) / 1e12
-    pcg64_gbs = PCG_BYTES_PER_CELL["fp64"] * N * it64_total / (pcg64_ms * 1e-3) / 1e9
-    if overlap64:   # concurrent kernels: the unprofiled iteration time, not the sum of launch times
-        pcg64_gbs = PCG_BYTES_PER_CELL["fp64"] * N / (iter64_ms * 1e-3) / 1e9
-    # per-kernel DRAM passes of a 3-component FP64 vector (8 B x 3 per cell per pass): the p update
-    # also adds the previous alpha p to x (r, p, x in; p, x out), the update reads r, q and writes r
-    kernels64 = {}
-    for k, passes in (("pupdate64", 5), ("spmv64", 2), ("update64", 3)):
-        ms_k, n_k = prof64[k]
-        if n_k:
-            avg = ms_k / it64_total
-            gbs = passes * 24 * N / (avg * 1e-3) / 1e9
-            kernels64[k] = dict(avg_launch_ms=round(avg, 4), bytes_per_cell=passes * 24, gbs=round(gbs, 1),
-                                frac_of_hbm=round(gbs / hbm, 4))
-    roof = dict(bound="alu", achieved=round(spmv_tflops, 4), peak=round(FP64_PEAK_TFLOPS / 1e3, 4),
-                unit="TFLOP/s", frac=round(spmv_tflops / (FP64_PEAK_TFLOPS / 1e3), 4),
-                traffic=(int(SPMV64_DRAM_BYTES_PER_CELL * N) if prof64["pupdate64"][1] and not overlap64 else None),
-                traffic_algorithmic=int(SPMV_BYTES_PER_CELL["fp64"] * N / (3 if overlap64 else 1)),
-                kernel=("k_spmv_dotc<2> (one component per launch, beside the next component's p update)"
-                        if overlap64 else "k_spmv_dot<double,2,3>"),
-                avg_launch_ms=round(spmv_avg, 4),
-                iteration=dict(fp64_instr_per_cell=FP64_INSTR_PER_CELL_ITER, ms=round(iter64_ms, 4),
-                               fp64_pipe_frac=round(FP64_INSTR_PER_CELL_ITER * N / (iter64_ms * 1e-3)
-                                                    / FP64_INSTR_PEAK, 4),
-                               form=form64,
-                               note=f"the whole FP64 CG iteration (p update, stencil, update), timed unprofiled "
-                                    f"over a {iter_n}-iteration solve of the first step's SI system, against the "
-                                    f"part's FP64 instruction rate"),
-                peak_source="2 DFMA/clk/SM x 152 SMs x 2.07 GHz (nominal FP64 rate of the part)")
+    pcg64_ms, pcg64_gbs, kernels64, roof = pcg64_account(prof64, it64_total, N, hbm, form64, iter64_ms, iter_n)
+    visc64_ms = pcg64_ms * visc_it / it64_total / len(infos64)
     # ---- mixed (FP32 inner PCG, FP64 refinement)
     def mixed_entry(inner_tol, restart):
         msm, infosm, profm, clkm, dsm = run(P.PREC_MIXED, args.steps, args.warmup, True, inner_tol, restart)
         msm = maxr(msm)
-        pcg32_ms = sum(profm[k][0] for k in ("pupdate32", "spmv32", "update32", "pspmv32", "pfold32", "rupd32",
-                                              "cgr32", "cgu32"))
         pcg32_n = max(sum(sum(i["iters"]) for i in infosm), 1)   # inner CG iterations actually run
-        pcg32_gbs = PCG_BYTES_PER_CELL["fp32"] * N * pcg32_n / (pcg32_ms * 1e-3) / 1e9
-        fused = profm["pspmv32"][1] > 0
-        recompute = profm["pfold32"][1] > 0 or profm["cgr32"][1] > 0
-        tiled = not fused and not recompute and profm["pupdate32"][1] == 0
-        # per-kernel DRAM passes of a 3-component FP32 vector (4 B x 3 per cell per pass)
-        # split form: the p update also adds the previous alpha p to x (r, p, x in; p, x out) and the
-        # update kernel reads r, q and writes r; fused form: r, p, x in, p, x, q out, then the update;
-        # recompute pair: r, p_old in, p out; then p, r in, r out, and every second iteration x,
-        # p_prev in, x out (4.5 on average); single-reduction pair: r in; then r, p_old in, p, r out,
-        # and every second iteration x in and out (5 on average)
-        kb = {"spmv32": 3 if tiled else 2, "update32": 5 if tiled else 3, "pupdate32": 5, "pspmv32": 6,
-              "pfold32": 3, "rupd32": 4.5, "cgr32": 1, "cgu32": 5}
-        kernels = {}
-        for k in ("pupdate32", "spmv32", "pspmv32", "update32", "pfold32", "rupd32", "cgr32", "cgu32"):
-            ms_k, n_k = profm[k]
-            if n_k:
-                avg = ms_k / pcg32_n   # one launch per inner iteration that ran
-                gbs = kb[k] * 12 * N / (avg * 1e-3) / 1e9
-                kernels[k] = dict(avg_launch_ms=round(avg, 4), bytes_per_cell=kb[k] * 12, gbs=round(gbs, 1),
-                                  frac_of_hbm=round(gbs / hbm, 4))
+        pcg32_gbs, kernels, form_name = pcg32_account(profm, pcg32_n, N, hbm)
         err = {k: float(torch.linalg.norm(dsm[k] - ds64[k]) / torch.linalg.norm(ds64[k])) for k in ds64}
         return dict(inner_tol=inner_tol, refinement=("restarted" if restart else "reliable updates"),
                     ms_per_step=round(msm, 3), speedup_vs_fp64=round(ms64 / msm, 3),
@@ -457,16 +500,7 @@ def run_ours(args):
                     outer_per_step=sum(sum(i["outer"]) for i in infosm) / len(infosm),
                     max_relres=max(max(i["relres"]) for i in infosm),
                     pcg_gbs=round(pcg32_gbs, 1), pcg_frac_of_hbm=round(pcg32_gbs / hbm, 4),
-                    kernels=kernels, fp32_kernels=("plane-marching pair (A: p update + stencil, B: stencil + "
-                                                   "update)" if tiled else
-                                                   "single-reduction pair (residual kernel: gamma, delta, "
-                                                   "stop norm; update kernel: p, A p, r, x every second "
-                                                   "iteration)" if profm["cgr32"][1] > 0 else
-                                                   "recompute pair (p update folded into <p, Ap>; r update "
-                                                   "with Ap recomputed, x every second iteration)" if recompute
-                                                   else
-                                                   "p update folded into the stencil, then the update" if fused
-                                                   else "split (p update, stencil, update)"),
+                    kernels=kernels, fp32_kernels=form_name,
                     rel_l2_vs_fp64_gpu_after_steps=err, clocks=clkm,
                     kernel_ms={k: round(v[0], 3) for k, v in profm.items() if v[1]})
 
@@ -544,7 +578,7 @@ def run_ours(args):
                     pcg_iters_per_step_pc1=[sum(i["iters"][q] for i in infos64) / len(infos64) for q in range(3)],
                     ms_per_iteration=round(sum(per_it.values()), 4), ms_per_iteration_pc1=round(iter64_ms, 4),
                     kernel_ms_per_iteration=per_it,
-                    line_kernel_gbs=round(PC2_LINE_BYTES_PER_CELL * N / (line_ms * 1e-3) / 1e9, 1),
+                    line_kernel_gbs=round(PC2_LINE_MOVED_BYTES_PER_CELL * N / (line_ms * 1e-3) / 1e9, 1),
                     rel_l2_vs_fp64_after_steps={k: float(torch.linalg.norm(dsp[k] - ds64p[k]) /
                                                          torch.linalg.norm(ds64p[k])) for k in ds64p},
                     clocks=clkp, kernel_ms={k: round(v[0], 3) for k, v in profp.items() if v[1]})
@@ -1060,8 +1094,8 @@ def main():
                     help="--profile-case pieces: fp64, mixed, pc2, pc2mixed (capped solves), sts, res (capped steps)")
     ap.add_argument("--iteration-forms", action="store_true",
                     help="time every kernel form of the FP64 and FP32 CG iterations on the first SI system and exit")
-    ap.add_argument("--forms64", default="-1,-64")
-    ap.add_argument("--forms32", default="-1,-2,-3,-4,-6,-7,-8")
+    ap.add_argument("--forms64", default="-1,-64,-65")
+    ap.add_argument("--forms32", default="-1,-2,-3,-4,-6,-7,-8,-9,-10")
     ap.add_argument("--form-iters", type=int, default=300)
     ap.add_argument("--batched", action="store_true", help="time the 64-system batched solve and exit")
     ap.add_argument("--batch", type=int, default=64)
