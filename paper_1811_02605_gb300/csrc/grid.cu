@@ -405,11 +405,14 @@ mhd_status_t create_grid(const mhd_grid_desc_t* desc, int i0, int i1, bool as_sl
     X.fr = x_fr; X.ft = x_ft; X.fp = x_fp;
     // row sums of |D^-1 K| (the Dirichlet weight sits on the diagonal only)
     double lam = 0.0;
+    G.d_max = G.k_max = 0.0;
     for (int i = 0; i < nr; i++)
         for (int j = 0; j < nt; j++) {
             const double s = h.wr[(size_t)i * nt + j] + h.wr[(size_t)(i + 1) * nt + j] + h.wt[(size_t)i * (nt + 1) + j] +
                              h.wt[(size_t)i * (nt + 1) + j + 1] + 2.0 * h.wp[(size_t)i * nt + j];
             const double off = s - (i == 0 ? h.wr[j] : 0.0);
+            G.d_max = std::max(G.d_max, h.rhoV[(size_t)i * nt + j]);
+            G.k_max = std::max(G.k_max, s);
             lam = std::max(lam, (s + off) / h.rhoV[(size_t)i * nt + j]);
         }
     g->visc_lambda_unit = lam;

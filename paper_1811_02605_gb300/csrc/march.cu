@@ -17,10 +17,14 @@
 // its own, so no barrier orders it. The halo (24 x 16) / (20 x 14) is read from L2; neighbouring columns
 // march in step, so HBM sees it once.
 //
-// us per iteration, the pair / this: 128x128x256 85.7 / 62.8, 192x192x384 247 / 163, 256x256x512 537 / 374 (5
+// us per iteration, the pair / this: 128x128x256 86.6 / 62.7, 192x192x384 247 / 162, 256x256x512 542 / 376 (5
 // passes at 6.8 TB/s are 296). What bounds it now is the latency of the steps (3 CTAs of 128 threads per SM
-// at 156 registers; issue slots half used, 3.9 TB/s of HBM). Other shapes at 192x192x384: one row a thread 242
+// at 152 registers; issue slots half used, 5.3 TB/s of HBM by the 60 B a cell). Other shapes at 192x192x384: one row a thread 242
 // (bound by instructions and shared-memory wavefronts), 2 rows 164 to 175, 4 rows 167 to 187, 5 rows 217.
+//
+// The sums are FP32 over the thread's 12 cells of a plane and compensated beyond; the weights dg of the stop norm
+// have 48 bits and each product's rounding is kept, as FP64 at this rate would take longer than all the rest (with
+// dg and the products rounded to FP32 an iteration at 256x256x512 took 0.9% less).
 //
 // One block barrier a plane: in step n a thread writes p of plane n and r' of plane n-1 to shared memory and
 // reads the neighbours' p of plane n-1 and r' of plane n-2, written in the step before.
@@ -78,12 +82,12 @@ __device__ __forceinline__ float4 stencil4(float4 u, float left, float right, fl
     return fma4(-c0.w, jp, o);
 }
 
-// compensated FP32 sum (two-sum)
+// compensated FP32 sum (two-sum) of x, or of x and a part of it below its rounding
 struct Sum2 {
     float s = 0.f, c = 0.f;
-    __device__ __forceinline__ void add(float x) {
+    __device__ __forceinline__ void add(float x, float low = 0.f) {
         const float t = s + x, b = t - s;
-        c += (s - (t - b)) + (x - b);
+        c += ((s - (t - b)) + (x - b)) + low;
         s = t;
     }
     __device__ __forceinline__ double get() const { return (double)s + (double)c; }
@@ -174,9 +178,9 @@ __global__ void __launch_bounds__(kMT, kCtas) k_march32(Dims d, Tiling T, float*
         const int tu = tr > 0 ? tr - 1 : 0, td = tr < kTR - 1 ? tr + 1 : tr;   // thread rows above and below
         fetch(0, 0);
         for (int n0 = 0; n0 < steps; n0 += 2) {
-            float pg = 0.f, pw = 0.f, pd = 0.f, pr = 0.f;   // plain over 32 cells, then compensated
 #pragma unroll
             for (int t = 0; t < 2; t++) {
+                float pg = 0.f, pw = 0.f, pd = 0.f;   // plain over the thread's 12 cells of a plane, then compensated
                 const int n = n0 + t;
                 fetch(n + 1, t ^ 1);
                 copy_wait<1>();
@@ -204,7 +208,7 @@ __global__ void __launch_bounds__(kMT, kCtas) k_march32(Dims d, Tiling T, float*
 #pragma unroll
                     for (int a = 0; a < kRT; a++) {
                         const float4 c0 = S.co[(n + 3) & 3][tr * kRT + a][0];
-                        const float2 c1 = *reinterpret_cast<const float2*>(&S.co[(n + 3) & 3][tr * kRT + a][1]);
+                        const float4 c1 = S.co[(n + 3) & 3][tr * kRT + a][1];
                         const float left = __shfl_up_sync(0xffffffffu, p1[a].w, 1, kLanes);
                         const float right = __shfl_down_sync(0xffffffffu, p1[a].x, 1, kLanes);
                         const float4 q = stencil4(p1[a], left, right, p2[a], p0[a], a > 0 ? p1[a > 0 ? a - 1 : 0] : above,
@@ -215,7 +219,9 @@ __global__ void __launch_bounds__(kMT, kCtas) k_march32(Dims d, Tiling T, float*
                             *reinterpret_cast<float4*>(rout + (o - plane) + a * d.np) = r1[a];
                             const float gg = fmaf(r1[a].x, r1[a].x, fmaf(r1[a].y, r1[a].y, fmaf(r1[a].z, r1[a].z, r1[a].w * r1[a].w)));
                             pg += gg;
-                            pr = fmaf(gg, c1.y, pr);
+                            // the stop norm's weight has 48 bits: the product is exact but for the low part's rounding
+                            const float wg = gg * c1.y;
+                            s_rr.add(wg, fmaf(gg, c1.z, fmaf(gg, c1.y, -wg)));
                             pw = fmaf(r1[a].x, q.x, fmaf(r1[a].y, q.y, fmaf(r1[a].z, q.z, fmaf(r1[a].w, q.w, pw))));
                         }
                     }
@@ -245,12 +251,11 @@ __global__ void __launch_bounds__(kMT, kCtas) k_march32(Dims d, Tiling T, float*
                     r2[a] = r1[a];
                     rk[a] = in[((t * 3 + 0) * kRT + a) * kMT];
                 }
+                s_g.add(pg);
+                s_w.add(pw);
+                s_d.add(pd);
                 __syncthreads();
             }
-            s_g.add(pg);
-            s_w.add(pw);
-            s_d.add(pd);
-            s_rr.add(pr);
         }
     }
     copy_wait<0>();

@@ -116,6 +116,7 @@ struct Geo {
     const double* wp;    // [nr*nt] phi-face weight (each of the two faces)
     const double* pcs;   // [2*np] cos, then sin, of the phi centres (polar pole values)
     double r0, r1, dth, dph;
+    double d_max, k_max;   // largest rho V and largest diagonal of K: every diagonal of M_alpha is below d_max + alpha k_max
     double max_kt2;
     double pole_f;       // 2 / (np cos(dth)): first-harmonic pole value of the B_theta face ring
 };
@@ -277,7 +278,7 @@ struct mhd_grid_s {
     // FP32 PCG workspace
     float *x32, *r32, *p32, *q32;
     float* row32;           // [8*nr*nt] per (i, j): ar low, ar high, at low, at high, ap, the diagonal over a power of
-                            // two, unused, and that power's exponent (the marching kernel's rows)
+                            // two (two floats), and that power's exponent (the marching kernel's rows)
     // step workspace
     double *b0, *b1, *dlt;
     double *er, *et, *ep;   // edge arrays (E or J)

@@ -125,13 +125,14 @@ __global__ void k_tables(Dims d, Geo G, const double* __restrict__ alpha_p, OpTa
         t32.ap[idx] = (float)ap;
         if (i == nr - 1) t32.ar[nr * nt + j] = 0.f;
         if (j == nt - 1) t32.at[i * (nt + 1) + nt] = 0.f;
-        // the marching kernel's rows: the coefficients and the diagonal over a power of two that keeps its
-        // products with r~^2 within r~^2's own range
+        // the marching kernel's rows: the coefficients and, in two floats (48 bits), the diagonal over a power of
+        // two above its largest value on the grid, so that its products with r~^2 stay within r~^2's own range
         const double ah = (i < nr - 1) ? a * G.wr[(i + 1) * nt + j] * (1.0 / sqrt(diag_at(G, nt, a, i + 1, j))) * s : 0.0;
         const double th = (j < nt - 1) ? a * G.wt[i * (nt + 1) + j + 1] * (1.0 / sqrt(diag_at(G, nt, a, i, j + 1))) * s : 0.0;
-        const int e = ilogb(diag_at(G, nt, a, nr - 1, nt / 2));
+        const int e = ilogb(G.d_max + a * G.k_max) + 1;
+        const double w = ldexp(dc, -e);
         row32[2 * idx] = make_float4((float)ar, (float)ah, (float)at, (float)th);
-        row32[2 * idx + 1] = make_float4((float)ap, (float)ldexp(dc, -e), 0.f, __int_as_float(e));
+        row32[2 * idx + 1] = make_float4((float)ap, (float)w, (float)(w - (double)(float)w), __int_as_float(e));
     }
 }
 
