@@ -406,7 +406,7 @@ void enqueue_march32(mhd_grid_s* g, cudaStream_t st, int nc);
 // all iterations of a point-Jacobi solve in one cooperative launch (persist.cu)
 size_t persist_buf_bytes();
 int persist_mode(const mhd_grid_s* g, bool fp32, int nc);
-mhd_status_t persist_iterate(mhd_grid_s* g, bool fp32, int nc);
+mhd_status_t persist_iterate(mhd_grid_s* g, bool fp32, int nc, bool* refused);
 
 // PCG (pcg.cu). alpha is read from device memory (alpha_dev) so a step never syncs on it.
 void build_tables(mhd_grid_s* g, const double* alpha_dev, bool fp32);

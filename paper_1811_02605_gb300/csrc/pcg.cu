@@ -1625,8 +1625,8 @@ __global__ void k_inner_end(PcgScalars* sc, const double* saved) {
 }  // namespace
 
 namespace {
-__global__ void k_tune_reset(PcgScalars* sc, int max_iter = 1 << 30) {
-    sc->done = 0;
+__global__ void k_tune_reset(PcgScalars* sc, int max_iter = 1 << 30, int done = 0) {
+    sc->done = done;
     sc->alpha = 0.0;
     sc->beta = 0.0;
     sc->rho = 1.0;
@@ -1701,12 +1701,26 @@ float time_persist(mhd_grid_s* g, bool fp32, int nc, cudaEvent_t e0, cudaEvent_t
     for (int warm = 1; warm >= 0; warm--) {
         k_tune_reset<<<1, 1, 0, g->stream>>>(g->sc, 8);
         if (!warm) cudaEventRecord(e0, g->stream);
-        if (persist_iterate(g, fp32, nc) != MHD_OK) return 1e30f;
+        bool refused = false;
+        if (persist_iterate(g, fp32, nc, &refused) != MHD_OK || refused) return 1e30f;
         if (!warm) cudaEventRecord(e1, g->stream);
     }
     float ms = 0.f;
     if (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) return 1e30f;
     return trial_ran(g, 8, 2) ? ms / 8.f : 1e30f;   // ended by max_iter
+}
+
+// whether the vectors fit the CTAs' shared memory and a launch of the persistent kernel (of a solve that has
+// ended: it returns at once) is accepted
+bool persist_by_rule(mhd_grid_s* g, bool fp32, int nc) {
+    if (persist_mode(g, fp32, nc) != 1) return false;
+    k_tune_reset<<<1, 1, 0, g->stream>>>(g->sc, 0, 1);
+    const int prof = g->prof;
+    g->prof = 0;
+    bool refused = false;
+    const bool ok = persist_iterate(g, fp32, nc, &refused) == MHD_OK && !refused;
+    g->prof = prof;
+    return ok;
 }
 
 mhd_status_t tune_slab32(mhd_grid_s* g, int nc) {
@@ -1722,7 +1736,7 @@ mhd_status_t tune_slab32(mhd_grid_s* g, int nc) {
     // vectors that fit the CTAs' shared memory (736 thousand cells with np a multiple of 4): the persistent
     // kernel, by rule. us per iteration, it against the best of the others: 32x32x64 10.0 / 17.4,
     // 48x48x96 11.5 / 20.4, 64x64x128 14.5 / 26.3. Above that it is one of the timed candidates.
-    if (persist_mode(g, true, nc) == 1) {
+    if (persist_by_rule(g, true, nc)) {
         g->slab32 = -9;
         return MHD_OK;
     }
@@ -1808,7 +1822,7 @@ mhd_status_t tune_slab64(mhd_grid_s* g) {
     // vectors that fit the CTAs' shared memory (368 thousand cells): the persistent kernel, by rule. us per
     // iteration, it against the split kernels: 32x32x64 13.5 / 20.0, 48x48x96 23.5 / 32.7,
     // 61x47x118 30.7 / 43.1. Above that it is one of the timed candidates.
-    if (persist_mode(g, false, 3) == 1) {
+    if (persist_by_rule(g, false, 3)) {
         g->slab64 = -3;
         return MHD_OK;
     }
@@ -1900,9 +1914,12 @@ mhd_status_t solve(mhd_grid_s* g, const double* alpha_dev, int nc, const double*
             if ((st = pc2_factor(g)) != MHD_OK) return st;
             pc2_init64(g, nc);
         }
-        if (!pc2 && prm->pcg_variant == 0 && g->slab64 == -3) st = persist_iterate(g, false, nc);
-        else st = run_iterations(g, pc2 ? 3 : (prm->pcg_variant == 1 ? 2 : 0), nc);
-        if (st != MHD_OK) return st;
+        bool split = pc2 || prm->pcg_variant != 0 || g->slab64 != -3;
+        if (!split) {
+            if ((st = persist_iterate(g, false, nc, &split)) != MHD_OK) return st;
+            if (split) g->slab64 = -1;   // the launch is refused here (fewer SMs than when the form was chosen)
+        }
+        if (split && (st = run_iterations(g, pc2 ? 3 : (prm->pcg_variant == 1 ? 2 : 0), nc)) != MHD_OK) return st;
         k_finish64<<<blocks2, kThreads, 0, g->stream>>>(d, nc, g->x64, g->p64, x, g->t64.s, g->sc);
         if ((st = check_cuda(g, "pcg finish")) != MHD_OK) return st;
         if (read_scalars(g) != MHD_OK) return MHD_ERR_CUDA;
@@ -1947,12 +1964,13 @@ mhd_status_t solve(mhd_grid_s* g, const double* alpha_dev, int nc, const double*
         outer_done = g->h_sc->outer_done;
         if (outer_done || o == prm->max_outer) break;
         k_inner_begin<<<1, 1, 0, g->stream>>>(g->sc, saved);
-        if (!pc2 && g->slab32 == -9) {
-            st = persist_iterate(g, true, nc);
-            if (st == MHD_OK) st = read_scalars(g);
-        } else {
-            st = run_iterations(g, pc2 ? 4 : 1, nc);
+        bool split = pc2 || g->slab32 != -9;
+        if (!split) {
+            if ((st = persist_iterate(g, true, nc, &split)) != MHD_OK) return st;
+            if (split) g->slab32 = -1;
+            else st = read_scalars(g);
         }
+        if (split) st = run_iterations(g, pc2 ? 4 : 1, nc);
         if (st != MHD_OK) return st;
         k_inner_end<<<1, 1, 0, g->stream>>>(g->sc, saved);
         if (g->h_sc->done == 6)

@@ -523,8 +523,9 @@ Shape shape_of(const mhd_grid_s* g, int nc, int V, bool sm) {
     return s;
 }
 
+// refused: the launch needs more SMs than this context may use (a green context, a partition); nothing has run
 template <typename T, int V, bool SM>
-mhd_status_t launch(mhd_grid_s* g, const Shape& s, T* x, T* r, T* p, T* q, const OpTab<T>& t) {
+mhd_status_t launch(mhd_grid_s* g, const Shape& s, T* x, T* r, T* p, T* q, const OpTab<T>& t, bool* refused) {
     const size_t bytes = smem_bytes<T, V>(s.chunk, s.rows, SM);
     if (cudaFuncSetAttribute(k_persist<T, V, SM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPSmemMax) != cudaSuccess)
         return check_cuda(g, "persistent PCG: shared memory");
@@ -550,8 +551,16 @@ mhd_status_t launch(mhd_grid_s* g, const Shape& s, T* x, T* r, T* p, T* q, const
     a[0].val.cooperative = 1;
     cfg.attrs = a;
     cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, k_persist<T, V, SM>, g->d, s.groups, s.chunk, x, r, p, q, t, (const double*)g->tu.dg, g->sc,
-                       buf, expect, budget);
+    // (the environment variable stands in for the refusal in tests, on the host)
+    const cudaError_t e = std::getenv("MHD_FAULT_COOP_LAUNCH")
+                              ? cudaErrorCooperativeLaunchTooLarge
+                              : cudaLaunchKernelEx(&cfg, k_persist<T, V, SM>, g->d, s.groups, s.chunk, x, r, p, q, t,
+                                                   (const double*)g->tu.dg, g->sc, buf, expect, budget);
+    if (e == cudaErrorCooperativeLaunchTooLarge) {
+        cudaGetLastError();
+        *refused = true;
+        return MHD_OK;
+    }
     return check_cuda(g, "persistent PCG launch");
 }
 
@@ -570,24 +579,26 @@ int persist_mode(const mhd_grid_s* g, bool fp32, int nc) {
 }
 
 // the iterations of a solve (FP64) or of an inner solve (FP32), after its set-up kernel; done, the
-// counts and the final scalars are in g->sc, x~ complete
-mhd_status_t persist_iterate(mhd_grid_s* g, bool fp32, int nc) {
+// counts and the final scalars are in g->sc, x~ complete. refused: the kernel cannot run here and has not touched
+// anything; the caller takes another form
+mhd_status_t persist_iterate(mhd_grid_s* g, bool fp32, int nc, bool* refused) {
     const int mode = persist_mode(g, fp32, nc);
-    if (!mode) return set_error(g, MHD_ERR_CUDA, "persistent PCG: not available on this grid");
+    *refused = !mode;
+    if (!mode) return MHD_OK;
     const int slot = prof_begin(g, g->stream, fp32 ? MHD_KERNEL_PERSIST32 : MHD_KERNEL_PERSIST64);
     mhd_status_t st;
     if (!fp32) {
         const Shape s = shape_of(g, nc, 2, mode == 1);
-        st = mode == 1 ? launch<double, 2, true>(g, s, g->x64, g->r64, g->p64, g->q64, g->t64)
-                       : launch<double, 2, false>(g, s, g->x64, g->r64, g->p64, g->q64, g->t64);
+        st = mode == 1 ? launch<double, 2, true>(g, s, g->x64, g->r64, g->p64, g->q64, g->t64, refused)
+                       : launch<double, 2, false>(g, s, g->x64, g->r64, g->p64, g->q64, g->t64, refused);
     } else if (g->d.np % 4 == 0) {
         const Shape s = shape_of(g, nc, 4, mode == 1);
-        st = mode == 1 ? launch<float, 4, true>(g, s, g->x32, g->r32, g->p32, g->q32, g->t32)
-                       : launch<float, 4, false>(g, s, g->x32, g->r32, g->p32, g->q32, g->t32);
+        st = mode == 1 ? launch<float, 4, true>(g, s, g->x32, g->r32, g->p32, g->q32, g->t32, refused)
+                       : launch<float, 4, false>(g, s, g->x32, g->r32, g->p32, g->q32, g->t32, refused);
     } else {
         const Shape s = shape_of(g, nc, 2, mode == 1);
-        st = mode == 1 ? launch<float, 2, true>(g, s, g->x32, g->r32, g->p32, g->q32, g->t32)
-                       : launch<float, 2, false>(g, s, g->x32, g->r32, g->p32, g->q32, g->t32);
+        st = mode == 1 ? launch<float, 2, true>(g, s, g->x32, g->r32, g->p32, g->q32, g->t32, refused)
+                       : launch<float, 2, false>(g, s, g->x32, g->r32, g->p32, g->q32, g->t32, refused);
     }
     prof_end(g, g->stream, slot);
     return st;
