@@ -118,17 +118,21 @@ enum { MHD_PREC_FP64 = 0, MHD_PREC_MIXED = 1 };
  *            mhd_adjoint_step; the first PC2 solve allocates N doubles + N floats for the
  *            factorisation and 3N floats for z of the FP32 iteration. pcg_solve_batched ignores it.
  *
- * Kernel variants of the FP32 inner iteration (split p update and stencil, the two folded into
- * one kernel, the recompute pair that stores no A p, the single-reduction pair, or plane-marching
- * tiles) and of the FP64 iteration (split, components overlapped on two streams, tiles) are chosen
- * per grid by timing on its first solve of each precision (or in mhd_grid_reserve); results agree
- * to the order of the dot products' reductions. Diagnostics only: the environment variable
+ * Kernel variants of the FP32 inner iteration (one persistent launch, the single-reduction
+ * iteration as one marching kernel or as a pair, split p update and stencil, the two folded into
+ * one kernel, or the recompute pair that stores no A p) and of the FP64 iteration (one persistent
+ * launch, split, components overlapped on two streams, tiles) are chosen per grid on its first
+ * solve of each precision (or in mhd_grid_reserve): the persistent launch by rule where the vectors
+ * fit the SMs' shared memory and the launch is accepted, else by timing; results agree to the order
+ * of the dot products' reductions. Diagnostics only: the environment variable
  * MHD_FORCE_SLAB skips the timing (-1 split, -2 folded, -3 recompute pair, -4 recompute pair with
  * the second kernel walking the grid backwards, -5 recompute pair at 6 CTAs per SM, -6 / -7 / -8
  * single-reduction pair (-7: its residual kernel unrolled over the components, both kernels at 3
  * CTAs per SM; -8: unrolled residual kernel, update kernel at 4), -9 whole inner solve in one
- * persistent launch, -10 the single-reduction iteration as one marching kernel, -64 the FP64 iteration with its components overlapped, -65 the whole FP64 solve
- * in one persistent launch, n > 0 tiles of n planes). */
+ * persistent launch, -10 the single-reduction iteration as one marching kernel, -64 the FP64
+ * iteration with its components overlapped, -65 the whole FP64 solve in one persistent launch, n > 0
+ * tiles of n planes, n < -100 the recompute pair staged by bulk copies in units of -100 - n planes;
+ * the FP32 tiles and the bulk-staged pair are reached in this way only). */
 typedef struct {
     double nu, eta, cfl, dt_fixed, dt_max, alpha_si_fixed;
     double tol, inner_tol;
@@ -350,7 +354,8 @@ mhd_status_t mhd_profile_read(mhd_grid_t grid, int kernel, double* total_ms, lon
  * FP64 iteration (-1 split, -2 components overlapped, -3 whole solve in one persistent launch, n > 0
  * tiles of n planes) and *fp32_form for the FP32 inner iteration (-1 split, -2 folded, -3/-4/-5
  * recompute pair, -6/-7/-8 single-reduction pair, -9 whole inner solve in one persistent launch, -10
- * single-reduction iteration as one marching kernel, <= -100 bulk-staged pair, n > 0 tiles); 0 where that precision has not been tuned yet.
+ * single-reduction iteration as one marching kernel, < -100 bulk-staged pair, n > 0 tiles); 0 where
+ * that precision has not been tuned yet.
  * Either pointer may be NULL. */
 mhd_status_t mhd_grid_kernel_forms(mhd_grid_t grid, int* fp64_form, int* fp32_form);
 

@@ -2,6 +2,9 @@
 // input rows are staged in shared memory by bulk asynchronous copies (cp.async.bulk, completion
 // on an mbarrier), a ring of planes in flight per CTA (3 in kernel A, 4 in kernel B).
 //
+// Not a timed candidate: np a multiple of 128 is where the marching kernel (march.cu) runs too, and it is 2.2 times as
+// fast and more (192x192x384: 162 against 449 us an iteration). MHD_FORCE_SLAB <= -101 takes this form.
+//
 // The arithmetic is that of the recompute pair in pcg.cu (k_pfold32 / k_rupd32):
 //   A: p~ = r~ + beta p~_old on the tile and its neighbours, <p~, A~ p~>, p~ stored (3 passes);
 //   B: q~ = A~ p~ from the stored p~, r~ -= alpha q~, <r~, r~>, sum dg r~^2, and on every second

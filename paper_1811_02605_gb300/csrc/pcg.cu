@@ -1490,7 +1490,7 @@ void enqueue_iteration(mhd_grid_s* g, cudaStream_t st, int prec, int nc) {
         enqueue_split_nc<double, 2>(g, st, nc, g->x64, g->r64, g->p64, g->q64, g->t64,
                                     grid_blocks(g, d.N / 2, kPerSmIter), MHD_KERNEL_PUPDATE64);
     } else if (g->slab32 <= -100) {
-        // plane-marching pair with bulk-copy staging, when the autotuner measured it fastest
+        // plane-marching pair with bulk-copy staging (MHD_FORCE_SLAB only)
         enqueue_bulk32(g, st, nc, -100 - g->slab32);
     } else if (g->slab32 == -10) {
         enqueue_march32(g, st, nc);
@@ -1508,7 +1508,7 @@ void enqueue_iteration(mhd_grid_s* g, cudaStream_t st, int prec, int nc) {
         if (use_v4(g)) enqueue_fused32_nc<4>(g, st, nc);
         else enqueue_fused32_nc<2>(g, st, nc);
     } else if (tiled32_ok(g) && g->slab32 > 0) {
-        // plane-marching pair, when the autotuner measured it faster than the split kernels
+        // plane-marching pair (MHD_FORCE_SLAB only)
         enqueue_tiled32(g, st, nc, g->slab32, MHD_KERNEL_SPMV32, MHD_KERNEL_UPDATE32);
     } else if (use_v4(g)) {
         enqueue_split_nc<float, 4>(g, st, nc, g->x32, g->r32, g->p32, g->q32, g->t32,
@@ -1733,7 +1733,7 @@ mhd_status_t tune_slab32(mhd_grid_s* g, int nc) {
         else g->slab32 = (f > 0 && tiled32_ok(g) && tiled32_blocks(g, f) <= kMaxBlocks) ? f : -1;
         return MHD_OK;
     }
-    // vectors that fit the CTAs' shared memory (736 thousand cells with np a multiple of 4): the persistent
+    // vectors that fit the CTAs' shared memory (220 KB each: at 152 SMs about 700 thousand cells): the persistent
     // kernel, by rule. us per iteration, it against the best of the others: 32x32x64 10.0 / 17.4,
     // 48x48x96 11.5 / 20.4, 64x64x128 14.5 / 26.3. Above that it is one of the timed candidates.
     if (persist_by_rule(g, true, nc)) {
@@ -1748,20 +1748,20 @@ mhd_status_t tune_slab32(mhd_grid_s* g, int nc) {
     const int prof = g->prof;
     g->prof = 0;
     // (the solve's set-up overwrites every vector afterwards)
-    // candidates -1: the split kernels (p update, stencil, update); -2: the p update folded into
-    // the stencil, then the update; -3, -4, -5: the recompute pair (no q~ stored), forwards, with
-    // the r update walking backwards, or at 6 CTAs per SM; -6, -7, -8: the single-reduction pair
-    // (-7: its residual kernel unrolled over the components and both kernels at 3 CTAs per SM; -8:
-    // the unrolled residual kernel with the update kernel at 4); -132,
-    // -164: the recompute pair as plane-marching kernels staged by bulk copies (units of 32 or 64
-    // planes). Four iterations each after one untimed: an even count, so each is timed with its
-    // x updates.
-    // Where the marching kernel (-10) can run, only the forms that come near it at some size are timed (us per
-    // iteration at 96x96x192 / 256x256x512: -10 36.9 / 374, -4 42.4 / 600, -7 45.6 / 537, -2 46.5 / 624).
+    // Candidates: -10: the marching kernel (np a multiple of 4); -2: the p update folded into the stencil, then the
+    // update; -1: the split kernels (p update, stencil, update); -3, -4, -5: the recompute pair (no q~ stored), forwards,
+    // with the r update walking backwards, or at 6 CTAs per SM; -6, -7, -8: the single-reduction pair (-7: its residual
+    // kernel unrolled over the components and both kernels at 3 CTAs per SM; -8: the unrolled residual kernel with
+    // the update kernel at 4). Four iterations each after one untimed: an even count, so each is timed with its x
+    // updates.
+    // Where the marching kernel can run, only the forms that come nearest it are timed: it or the persistent kernel
+    // was fastest at 13 grids from 100x100x104 to 256x256x512, flat, long and thin ones among them (us per iteration,
+    // -10 / the best of -7, -4, -2 / the best of -1, -3, -5, -6, -8 / the bulk-staged pair / tiles, these two needing np
+    // a multiple of 128 and left to MHD_FORCE_SLAB: 112x96x128 34.6 / 36.5 / 36.2 / 76 / 80, 16x256x512
+    // 40.2 / 49.9 / 49.9 / 101 / 107, 400x400x64 160 / 178 / 181, 256x256x512 376 / 542 / 546 / 900 / 1025).
     const bool march = march32_ok(g);
-    for (int cand : {-10, -7, -4, -2, -1, -3, -5, -6, -8, -132, -164}) {
+    for (int cand : {-10, -7, -4, -2, -1, -3, -5, -6, -8}) {
         if (cand == -10 ? !march : (march && cand != -7 && cand != -4 && cand != -2)) continue;
-        if (cand <= -100 && !bulk32_ok(g)) continue;
         k_tune_reset<<<1, 1, 0, g->stream>>>(g->sc);
         g->slab32 = cand;
         trial_vectors32(g);
@@ -1775,36 +1775,16 @@ mhd_status_t tune_slab32(mhd_grid_s* g, int nc) {
         if (cudaEventSynchronize(e1) != cudaSuccess) break;
         float ms = 0.f;
         cudaEventElapsedTime(&ms, e0, e1);
-        ms *= 0.75f;   // per 3 iterations, as the tiled candidates below
         if (ms < best_ms && trial_ran(g, 5)) {
             best_ms = ms;
             best = cand;
         }
     }
-    trial_vectors32(g);
-    for (int slab : {8, 16, 32, 64}) {
-        if (march || !tiled32_ok(g)) break;
-        if (slab > 2 * g->d.nr && best > 0) break;
-        if (tiled32_blocks(g, slab) > kMaxBlocks) continue;
-        k_tune_reset<<<1, 1, 0, g->stream>>>(g->sc);
-        enqueue_tiled32(g, g->stream, nc, slab, 0, 0);
-        cudaEventRecord(e0, g->stream);
-        for (int it = 0; it < 3; it++) enqueue_tiled32(g, g->stream, nc, slab, 0, 0);
-        cudaEventRecord(e1, g->stream);
-        if (cudaEventSynchronize(e1) != cudaSuccess) break;
-        float ms = 0.f;
-        cudaEventElapsedTime(&ms, e0, e1);
-        if (ms < best_ms && trial_ran(g, 4)) {
-            best_ms = ms;
-            best = slab;
-        }
-    }
-    if (g->d.N <= kPersistTrial && 3.f * time_persist(g, true, nc, e0, e1) < best_ms) best = -9;
+    if (g->d.N <= kPersistTrial && 4.f * time_persist(g, true, nc, e0, e1) < best_ms) best = -9;
     g->prof = prof;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    g->slab32 = (best == 0) ? -1 : best;  // -1 split, -2 folded, -3/-4 recompute pair, -9 persistent, -10 marching,
-                       // <= -100 bulk-staged pair, > 0 tiled slab
+    g->slab32 = (best == 0) ? -1 : best;
     return check_cuda(g, "tune slab");
 }
 }  // namespace
@@ -1819,7 +1799,8 @@ mhd_status_t tune_slab64(mhd_grid_s* g) {
         else g->slab64 = (f > 0 && tiled32_ok(g) && tiled32_blocks(g, f) <= kMaxBlocks) ? f : (f == -64 ? -2 : -1);
         return MHD_OK;
     }
-    // vectors that fit the CTAs' shared memory (368 thousand cells): the persistent kernel, by rule. us per
+    // vectors that fit the CTAs' shared memory (220 KB each: at 152 SMs about 350 thousand cells): the persistent
+    // kernel, by rule. us per
     // iteration, it against the split kernels: 32x32x64 13.5 / 20.0, 48x48x96 23.5 / 32.7,
     // 61x47x118 30.7 / 43.1. Above that it is one of the timed candidates.
     if (persist_by_rule(g, false, 3)) {

@@ -2,7 +2,7 @@
 // an inner solve (FP32) runs inside the kernel, with one CTA per SM.
 //
 // Why: below about a million cells an iteration's kernels are shorter than the launches and the
-// last-block reductions between them (32x32x64, FP64: 3.7 us of FP64 instructions in a 22 us
+// last-block reductions between them (32x32x64, FP64: 3.7 us of FP64 instructions in a 20.0 us
 // iteration of three kernels). Here the CTAs stay resident, each owns the same cells throughout, and
 // the vectors that only their owner touches (x~, r~, q~ and its share of p~) stay in shared memory;
 // only p~ is also written to global memory, where the neighbouring CTAs read it.

@@ -11,7 +11,7 @@
 // vector [br | bt | bp] (polar theta faces: identity rows), then B = B* - dte curl_h J(x): the
 // last update is a CT circulation, so div_h B keeps its value to rounding whatever the tolerance.
 //
-// Per iteration: edge current of p (ring sums + three edge kernels), q = M p with <p, q>, the
+// Per iteration: edge current of p (one launch), q = M p with <p, q>, the
 // x / r update with <r, z> and ||r||^2, and p = z + beta p; the scalar recurrence runs in the
 // last CTA of each reducing kernel, and batches of iterations replay as one CUDA graph.
 //

@@ -1,5 +1,9 @@
 // FP32 CG iteration in two plane-marching kernels (the inner solve of the mixed-precision path).
 //
+// The FP32 pair is not a timed candidate: np a multiple of 128 is where the marching kernel (march.cu) runs too, at
+// half the time and less (192x192x384: 162 against 471 us an iteration). MHD_FORCE_SLAB = n > 0 takes it. The FP64
+// kernel A at the end of this file is timed.
+//
 // The split form (p update, stencil, update) moves 10 passes of a 3-component vector per
 // iteration. Here:
 //   A: p_new = r + beta p_old at every point the stencil needs, q = A~ p_new, <p_new, q>;

@@ -63,3 +63,15 @@ def test_chosen_form_is_near_the_fastest(monkeypatch, d, mixed, first):
         assert P.pcg_solve(g, float(first.split()[1]), b, torch.zeros_like(b), prm)[0] == P.MHD_OK
     form = P.mhd_grid_kernel_forms(g)[1 if mixed else 0]
     assert ms[form] <= 1.15 * min(ms.values()), (form, ms)
+
+
+@pytest.mark.parametrize("d,mixed", [(I.GridDesc(45, 61, 128, 1.0, 10.0, 1.02), 0), (I.GridDesc(78, 70, 128, 1.0, 10.0, 1.02), 1)],
+                         ids=["45x61x128 fp64", "78x70x128 mixed"])
+def test_persistent_form_by_rule_up_to_shared_memory(d, mixed):
+    # the largest grids with np = 128, but a row or two, whose vectors fit 152 CTAs with 220 KB of shared memory
+    # each (351,360 cells in FP64, 701,952 in FP32)
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("sizes for 152 SMs")
+    g = grid(d)
+    P.mhd_grid_reserve(g, P.RESERVE_MIXED if mixed else P.RESERVE_PC1)
+    assert P.mhd_grid_kernel_forms(g)[1 if mixed else 0] == (-9 if mixed else -3)
