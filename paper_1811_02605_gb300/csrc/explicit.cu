@@ -1,5 +1,5 @@
 // Explicit parts of the zero-beta step (Eq. 1; Sec. 2.2 explicit predictor-corrector
-// upwinding), all FP64, one warp per row of output elements:
+// upwinding), all FP64, a warp or a part of one per row of output elements:
 //   - step coefficients: dt from the flow CFL, C_w, the semi-implicit coefficient (Sec. 2.1)
 //   - J = curl_h B on edges (Stokes on the dual faces around each edge)
 //   - momentum force b = rho V dt (-(v.grad)v + J x B / rho)
@@ -17,6 +17,7 @@
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
+#include <utility>
 
 #include "mhd_internal.cuh"
 #include "reduce.cuh"
@@ -28,21 +29,53 @@ namespace {
 
 // FP64 runs at 2 multiply-adds per clock and SM on this part (64 cycles a warp instruction and scheduler), so
 // these kernels are bound by their count of FP64 instructions; integer work, loads and address arithmetic are
-// free beside it. Hence: one warp per row (i, j) of np elements, so that whatever depends on the row alone is
+// free beside it. Hence: a row (i, j) of np elements, or a part of it, to a group of lanes, so that whatever depends on the row alone is
 // formed once a row; the means are kept as plain sums (B_c doubled, J_c and the edge E by powers of two, which
 // scale exactly) and the factor goes into a row constant; signs and maxima are integer tests; the upwind
 // difference is |u_d| / h (u - u_upwind), one form for both signs. Coefficients, force, induction with
 // resistivity and diagnostics of a 256x256x512 grid: 21.3 -> 13.0 ms, at about 190 FP64 instructions a cell and 82 to
 // 89% of the pipe.
-__device__ __forceinline__ unsigned int first_row() {
-    return blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
-}
-__device__ __forceinline__ unsigned int row_stride() { return gridDim.x * (kThreads / 32); }
 
-__device__ __forceinline__ double warp_sum(double s) {
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    return s;
-}
+// How rows of np elements are dealt to lanes: `lanes` of a warp (a power of two) take a row, or one of its `parts` of
+// len elements each.
+struct RowMap {
+    int lanes, parts, len;
+    // WHOLE: a warp takes whole rows, known at compile time (k_current takes 8 registers less then, so a CTA per SM
+    // more: 740 us at 256x256x512, else 790)
+    template <bool WHOLE>
+    __host__ __device__ RowMap fixed(int np) const {
+        return WHOLE ? RowMap{32, 1, np} : *this;
+    }
+};
+
+// a thread's place: rows (or parts of rows) w, w + stride, ...; lane is its lane within the row
+struct Lanes {
+    unsigned int first, stride, mask;
+    int lane, n;
+    __device__ __forceinline__ explicit Lanes(const RowMap& M) : n(M.lanes) {
+        const unsigned int sh = 31 - __clz(M.lanes);
+        first = (blockIdx.x * kThreads + threadIdx.x) >> sh;
+        stride = (gridDim.x * kThreads) >> sh;
+        lane = threadIdx.x & (M.lanes - 1);
+        mask = (0xffffffffu >> (32 - M.lanes)) << (threadIdx.x & 31 & ~(M.lanes - 1));
+    }
+    // sum over the row's lanes, in all of them
+    __device__ __forceinline__ double sum(double s) const {
+        for (int o = n / 2; o > 0; o >>= 1) s += __shfl_xor_sync(mask, s, o);
+        return s;
+    }
+};
+// item -> row and the elements [lo, hi) of it, lo the lane's first
+struct Part {
+    unsigned int row;
+    int part, lo, hi;
+    __device__ __forceinline__ Part(const RowMap& M, const Lanes& L, unsigned int item, int np) {
+        row = item / (unsigned int)M.parts;
+        part = (int)(item - row * (unsigned int)M.parts);
+        lo = part * M.len + L.lane;
+        hi = min(part * M.len + M.len, np);
+    }
+};
 // x > 0 (true also for a NaN with a clear sign, which makes every use of the result a NaN)
 __device__ __forceinline__ bool positive(double x) { return __double_as_longlong(x) > 0; }
 // m = max(m, |x|) on the bits of non-negative doubles; a NaN is ignored, as by fmax
@@ -121,6 +154,60 @@ struct Vel {
     }
 };
 
+// Lanes and parts of rows of np elements, and the CTAs of a kernel over them: as many as are resident at once.
+// Parts: where rows are so few that they would not fill the resident warps, a row is cut, down to 4 passes of its
+// lanes. Lanes: 32 while a row is many passes long (smaller groups at np = 512 took 15 to 50% longer: their accesses are spread
+// over more rows); below that the number with the least estimated time, which is the items that the busiest
+// SM gets, a CTA's worth at a time, times the passes of an item, with a factor for the spread. Times in us, coefficients + force +
+// induction without and with resistivity + diagnostics, with 32 lanes and one part for every row / by this rule:
+// 256x256x8 1364 / 460, 300x200x34 2196 / 1310, 100x100x48 529 / 426, 61x47x118 401 / 357, 16x16x4096 2010 / 829,
+// 4x4x8192 3430 / 435.
+struct RowLaunch {
+    RowMap m;
+    int blocks;
+};
+RowLaunch row_launch(const mhd_grid_s* g, long long rows, int resident) {
+    const int np = g->d.np;
+    const long long room = (long long)g->num_sms * resident * kThreads;
+    auto map = [&](int lanes) {
+        RowMap m{lanes, 1, 0};
+        m.parts = (int)std::max<long long>(1, std::min<long long>(np / (4 * lanes), (room + rows * lanes - 1) / (rows * lanes)));
+        const int len = (np + m.parts - 1) / m.parts;
+        m.len = (len + lanes - 1) / lanes * lanes;
+        m.parts = (np + m.len - 1) / m.len;
+        return m;
+    };
+    auto cost = [&](const RowMap& m, double spread) {
+        const long long ctas = (rows * m.parts * m.lanes + kThreads - 1) / kThreads;
+        return (double)((ctas + g->num_sms - 1) / g->num_sms) * (m.len / m.lanes + 0.2) * spread;
+    };
+    RowLaunch r{map(32), 0};
+    if (np < 256) {
+        double least = cost(r.m, 1.0);
+        for (const auto& [lanes, spread] : {std::pair(16, 1.15), std::pair(8, 1.15), std::pair(4, 1.2), std::pair(2, 1.4)}) {
+            const RowMap m = map(lanes);
+            const double c = cost(m, spread);
+            if (c < least) {
+                least = c;
+                r.m = m;
+            }
+        }
+    }
+    r.blocks = grid_blocks(g, rows * r.m.parts * r.m.lanes, resident);
+    return r;
+}
+// launch a row kernel: W where warps take whole rows, P otherwise
+template <auto W, auto P, typename... Args>
+void launch_rows(const mhd_grid_s* g, cudaStream_t st, long long rows, int max_blocks, Args... args) {
+    RowLaunch r = row_launch(g, rows, resident_per_sm<W>());
+    if (r.m.lanes == 32 && r.m.parts == 1) {
+        W<<<std::min(r.blocks, max_blocks), kThreads, 0, st>>>(g->d, r.m, args...);
+        return;
+    }
+    r = row_launch(g, rows, resident_per_sm<P>());
+    P<<<std::min(r.blocks, max_blocks), kThreads, 0, st>>>(g->d, r.m, args...);
+}
+
 }  // namespace
 
 // ------------------------------------------------------------------------------------------
@@ -128,7 +215,8 @@ struct Vel {
 // ------------------------------------------------------------------------------------------
 // Every term of a row has the same factors, and rounding is monotone, so the row's largest |v|^2 and |B|^2 give
 // the largest products bit for bit.
-__global__ void __launch_bounds__(kThreads) k_coeffs(Dims d, Geo G, Vel<false> v, const double* __restrict__ bh,
+template <bool WHOLE>
+__global__ void __launch_bounds__(kThreads) k_coeffs(Dims d, RowMap map, Geo G, Vel<false> v, const double* __restrict__ bh,
                                                      const double* __restrict__ br,
                                                      const double* __restrict__ bt,
                                                      const double* __restrict__ bp, double nu, double cfl,
@@ -136,13 +224,17 @@ __global__ void __launch_bounds__(kThreads) k_coeffs(Dims d, Geo G, Vel<false> v
                                                      StepScalars* ss, double* __restrict__ partials) {
     double mkv = 0.0, mka = 0.0;
     const unsigned int rows = (unsigned int)(d.nr * d.nt);
-    for (unsigned int ij = first_row(); ij < rows; ij += row_stride()) {
+    const RowMap M = map.fixed<WHOLE>(d.np);
+    const Lanes L(M);
+    for (unsigned int it = L.first; it < rows * M.parts; it += L.stride) {
+        const Part S(M, L, it, d.np);
+        const unsigned int ij = S.row;
         const int i = (int)(ij / d.nt), j = (int)(ij - (unsigned int)i * d.nt);
         const FaceRow F(d, G, bh, br, bt, bp, i, j);
         long long mv = 0, mb = 0;
         F.over([&](auto polar) {
 #pragma unroll 4
-            for (int k = threadIdx.x & 31; k < d.np; k += 32) {
+            for (int k = S.lo; k < S.hi; k += L.n) {
                 double u[3], B[3];
                 v.at((long long)ij * d.np + k, u);
                 F.twice<decltype(polar)::value>(k, kp1(d, k), B);
@@ -187,9 +279,9 @@ mhd_status_t coeffs(mhd_grid_s* g, const mhd_params_t* p, const double* vr, cons
                     const double* vp, const double* br, const double* bt, const double* bp) {
     const Vel<false> v{vr, vt, vp, nullptr, 0.0, g->d.N};
     bt_harmonics(g, bt);
-    const int blocks = grid_blocks(g, 32ll * g->d.nr * g->d.nt, resident_per_sm<k_coeffs>());
-    k_coeffs<<<blocks, kThreads, 0, g->stream>>>(g->d, g->geo, v, g->bharm, br, bt, bp, p->nu, p->cfl, p->dt_fixed,
-                                                 p->dt_max, p->alpha_si_fixed, g->ss, g->partials);
+    launch_rows<k_coeffs<true>, k_coeffs<false>>(g, g->stream, (long long)g->d.nr * g->d.nt, kMaxBlocks, g->geo, v, g->bharm, br,
+                                                 bt, bp, p->nu, p->cfl, p->dt_fixed, p->dt_max, p->alpha_si_fixed, g->ss,
+                                                 g->partials);
     return check_cuda(g, "coeffs");
 }
 
@@ -244,11 +336,12 @@ void bt_harmonics(mhd_grid_s* g, const double* bt, cudaStream_t st) {
 // ------------------------------------------------------------------------------------------
 // current density on edges
 // ------------------------------------------------------------------------------------------
-// J on all edges in one launch, a warp per row; a polar radial row takes its ring's sum of B_phi itself (the cap
+// J on all edges in one launch, a group of lanes per row; a polar radial row takes its ring's sum of B_phi itself (the cap
 // circulation), and with bh the warps of the first 2 nr rows form the harmonics of the B_theta rings beside the
 // poles. walls_zero: the resistive operator's current, 0 on the tangential edges of r0 and r1. done (may be null):
 // a solve's flag, nothing is formed once it is set.
-__global__ void __launch_bounds__(kThreads) k_current(Dims d, const double* __restrict__ cr,
+template <bool WHOLE>
+__global__ void __launch_bounds__(kThreads) k_current(Dims d, RowMap map, const double* __restrict__ cr,
                                                       const double* __restrict__ ct, const double* __restrict__ cp,
                                                       const double* __restrict__ br, const double* __restrict__ bt,
                                                       const double* __restrict__ bp, double* __restrict__ jr,
@@ -258,19 +351,24 @@ __global__ void __launch_bounds__(kThreads) k_current(Dims d, const double* __re
     if (done && *done) return;
     const unsigned int n_h = bh ? 2u * d.nr : 0u, n_r = (unsigned int)(d.nr * (d.nt + 1)),
                        n_t = (unsigned int)((d.nr + 1) * d.nt), n_p = (unsigned int)((d.nr + 1) * (d.nt + 1));
-    const int np = d.np, lane = threadIdx.x & 31;
-    for (unsigned int w = first_row(); w < n_h + n_r + n_t + n_p; w += row_stride()) {
+    const int np = d.np;
+    const RowMap M = map.fixed<WHOLE>(d.np);
+    const Lanes L(M);
+    for (unsigned int it = L.first; it < (n_h + n_r + n_t + n_p) * M.parts; it += L.stride) {
+        const Part S(M, L, it, np);
+        const unsigned int w = S.row;
         if (w < n_h) {
+            if (S.part) continue;
             const int i = (int)(w % d.nr), south = (int)(w / d.nr);
             const double* row = bt + ixt(d, i, south ? d.nt - 1 : 1, 0);
             double c = 0.0, s = 0.0;
-            for (int k = lane; k < np; k += 32) {
+            for (int k = L.lane; k < np; k += L.n) {
                 c = fma(row[k], pcs[k], c);
                 s = fma(row[k], pcs[np + k], s);
             }
-            c = warp_sum(c);
-            s = warp_sum(s);
-            if (lane == 0) {
+            c = L.sum(c);
+            s = L.sum(s);
+            if (L.lane == 0) {
                 bh[2 * w] = c;
                 bh[2 * w + 1] = s;
             }
@@ -282,14 +380,14 @@ __global__ void __launch_bounds__(kThreads) k_current(Dims d, const double* __re
             if (j == 0 || j == d.nt) {
                 const double* row = bp + ix(d, i, j == 0 ? 0 : d.nt - 1, 0);
                 double s = 0.0;
-                for (int k = lane; k < np; k += 32) s += row[k];
-                s = warp_sum(s) * (j == 0 ? c[3] : -c[3]);   // cap circulation / cap area
-                for (int k = lane; k < np; k += 32) out[k] = s;
+                for (int k = L.lane; k < np; k += L.n) s += row[k];
+                s = L.sum(s) * (j == 0 ? c[3] : -c[3]);   // cap circulation / cap area
+                for (int k = S.lo; k < S.hi; k += L.n) out[k] = s;
             } else {
                 const double c0 = c[0], c1 = c[1], c2 = c[2];
                 const double *b = bp + ix(d, i, j, 0), *a = b - np, *t = bt + ixt(d, i, j, 0);
 #pragma unroll 4
-                for (int k = lane; k < np; k += 32) out[k] = c0 * b[k] - c1 * a[k] - c2 * (t[k] - t[km1(d, k)]);
+                for (int k = S.lo; k < S.hi; k += L.n) out[k] = c0 * b[k] - c1 * a[k] - c2 * (t[k] - t[km1(d, k)]);
             }
         } else if (w < n_h + n_r + n_t) {
             const unsigned int q = w - n_h - n_r;
@@ -302,21 +400,21 @@ __global__ void __launch_bounds__(kThreads) k_current(Dims d, const double* __re
             const double c0 = c[0], c1 = c[1], c2 = c[2];
             double* out = jt + (long long)q * np;
 #pragma unroll 4
-            for (int k = lane; k < np; k += 32)
+            for (int k = S.lo; k < S.hi; k += L.n)
                 out[k] = wall ? 0.0 : c0 * lo[k] + c1 * (b[k] - b[km1(d, k)]) - c2 * hi[k];
         } else {
             const unsigned int q = w - n_h - n_r - n_t;
             const int i = (int)(q / (d.nt + 1)), j = (int)(q - (unsigned int)i * (d.nt + 1));
             double* out = jp + (long long)q * np;
             if (j == 0 || j == d.nt || (walls_zero && (i == 0 || i == d.nr))) {
-                for (int k = lane; k < np; k += 32) out[k] = 0.0;
+                for (int k = S.lo; k < S.hi; k += L.n) out[k] = 0.0;
             } else {
                 const double *lo = bt + ixt(d, i > 0 ? i - 1 : 0, j, 0), *hi = bt + ixt(d, i < d.nr ? i : d.nr - 1, j, 0);
                 const double *b = br + ix(d, i, j, 0), *a = b - np;
                 const double* c = cp + 3 * (size_t)q;
                 const double c0 = c[0], c1 = c[1], c2 = c[2];
 #pragma unroll 4
-                for (int k = lane; k < np; k += 32) out[k] = c0 * (a[k] - b[k]) + c1 * hi[k] - c2 * lo[k];
+                for (int k = S.lo; k < S.hi; k += L.n) out[k] = c0 * (a[k] - b[k]) + c1 * hi[k] - c2 * lo[k];
             }
         }
     }
@@ -324,19 +422,13 @@ __global__ void __launch_bounds__(kThreads) k_current(Dims d, const double* __re
 
 namespace {
 
-// CTAs of a kernel that hands rows to warps: as many as are resident at once
-template <auto K>
-int row_blocks(const mhd_grid_s* g, long long rows) {
-    return grid_blocks(g, 32 * rows, resident_per_sm<K>());
-}
-
 void edge_current(mhd_grid_s* g, const double* cr, const double* ct, const double* cp, const double* br, const double* bt,
                   const double* bp, double* bh, bool walls_zero, const int* done, cudaStream_t st) {
     const Dims d = g->d;
     const long long rows = (bh ? 2ll * d.nr : 0ll) + (long long)d.nr * (d.nt + 1) + (long long)(d.nr + 1) * d.nt +
                            (long long)(d.nr + 1) * (d.nt + 1);
-    k_current<<<row_blocks<k_current>(g, rows), kThreads, 0, st>>>(d, cr, ct, cp, br, bt, bp, g->er, g->et, g->ep,
-                                                                   g->geo.pcs, bh, walls_zero ? 1 : 0, done);
+    launch_rows<k_current<true>, k_current<false>>(g, st, rows, kMaxBlocks, cr, ct, cp, br, bt, bp, g->er, g->et, g->ep,
+                                                   g->geo.pcs, bh, walls_zero ? 1 : 0, done);
 }
 
 void current_and_harmonics(mhd_grid_s* g, const double* br, const double* bt, const double* bp, double* bh, cudaStream_t st) {
@@ -358,8 +450,8 @@ void res_edge_current(mhd_grid_s* g, const double* cr, const double* ct, const d
 // momentum force
 // ------------------------------------------------------------------------------------------
 // AVG: the mean with the force in b_avg
-template <bool DLT, bool AVG>
-__global__ void __launch_bounds__(kThreads) k_force(Dims d, Geo G, ExTab X, Vel<DLT> v, const double* __restrict__ bh,
+template <bool DLT, bool AVG, bool WHOLE>
+__global__ void __launch_bounds__(kThreads) k_force(Dims d, RowMap map, Geo G, ExTab X, Vel<DLT> v, const double* __restrict__ bh,
                                                     const double* __restrict__ br,
                                                     const double* __restrict__ bt, const double* __restrict__ bp,
                                                     const double* __restrict__ jr, const double* __restrict__ jt,
@@ -369,7 +461,11 @@ __global__ void __launch_bounds__(kThreads) k_force(Dims d, Geo G, ExTab X, Vel<
     const double dt = dt_dev ? *dt_dev : dt_host;
     const unsigned int rows = (unsigned int)(d.nr * d.nt);
     const long long plane = (long long)d.nt * d.np;
-    for (unsigned int ij = first_row(); ij < rows; ij += row_stride()) {
+    const RowMap M = map.fixed<WHOLE>(d.np);
+    const Lanes L(M);
+    for (unsigned int it = L.first; it < rows * M.parts; it += L.stride) {
+        const Part S(M, L, it, d.np);
+        const unsigned int ij = S.row;
         const int i = (int)(ij / d.nt), j = (int)(ij - (unsigned int)i * d.nt);
         const FaceRow F(d, G, bh, br, bt, bp, i, j);
         const EdgeRow E(d, jr, jt, jp, i, j);
@@ -385,7 +481,7 @@ __global__ void __launch_bounds__(kThreads) k_force(Dims d, Geo G, ExTab X, Vel<
         const long long t_lo = j > 0 ? -d.np : 0, t_hi = j < d.nt - 1 ? d.np : 0;
         F.over([&](auto polar) {
 #pragma unroll 1
-            for (int k = threadIdx.x & 31; k < d.np; k += 32) {
+            for (int k = S.lo; k < S.hi; k += L.n) {
                 const long long c = c_row + k;
                 const int kp = kp1(d, k), km = km1(d, k);
                 double u[3], n[3], adv[3], B[3], J[3];
@@ -440,8 +536,9 @@ namespace {
 template <bool DLT, bool AVG>
 void force_launch(mhd_grid_s* g, const Vel<DLT>& v, const double* br, const double* bt, const double* bp,
                   const double* dt_dev, double dt_host, const double* b_avg, double* b) {
-    k_force<DLT, AVG><<<row_blocks<k_force<DLT, AVG>>(g, (long long)g->d.nr * g->d.nt), kThreads, 0, g->stream>>>(
-        g->d, g->geo, g->ex, v, g->bharm, br, bt, bp, g->er, g->et, g->ep, dt_dev, dt_host, b_avg, b);
+    launch_rows<k_force<DLT, AVG, true>, k_force<DLT, AVG, false>>(g, g->stream, (long long)g->d.nr * g->d.nt, kMaxBlocks, g->geo,
+                                                                   g->ex, v, g->bharm, br, bt, bp, g->er, g->et, g->ep, dt_dev,
+                                                                   dt_host, b_avg, b);
 }
 }  // namespace
 
@@ -461,8 +558,8 @@ void force(mhd_grid_s* g, const double* vr, const double* vt, const double* vp, 
 // electric field and constrained transport
 // ------------------------------------------------------------------------------------------
 // twice E at the cell centres; ETA: with the resistive part
-template <bool DLT, bool ETA>
-__global__ void __launch_bounds__(kThreads) k_ecentre(Dims d, Geo G, Vel<DLT> v, const double* __restrict__ bh,
+template <bool DLT, bool ETA, bool WHOLE>
+__global__ void __launch_bounds__(kThreads) k_ecentre(Dims d, RowMap map, Geo G, Vel<DLT> v, const double* __restrict__ bh,
                                                       const double* __restrict__ br,
                                                       const double* __restrict__ bt, const double* __restrict__ bp,
                                                       const double* __restrict__ jr, const double* __restrict__ jt,
@@ -470,13 +567,17 @@ __global__ void __launch_bounds__(kThreads) k_ecentre(Dims d, Geo G, Vel<DLT> v,
                                                       double* __restrict__ ec) {
     const unsigned int rows = (unsigned int)(d.nr * d.nt);
     const double eta_h = 0.5 * eta;   // of four times J
-    for (unsigned int ij = first_row(); ij < rows; ij += row_stride()) {
+    const RowMap M = map.fixed<WHOLE>(d.np);
+    const Lanes L(M);
+    for (unsigned int it = L.first; it < rows * M.parts; it += L.stride) {
+        const Part S(M, L, it, d.np);
+        const unsigned int ij = S.row;
         const int i = (int)(ij / d.nt), j = (int)(ij - (unsigned int)i * d.nt);
         const FaceRow F(d, G, bh, br, bt, bp, i, j);
         const EdgeRow E(d, jr, jt, jp, i, j);
         F.over([&](auto polar) {
 #pragma unroll 2
-            for (int k = threadIdx.x & 31; k < d.np; k += 32) {
+            for (int k = S.lo; k < S.hi; k += L.n) {
                 const long long c = (long long)ij * d.np + k;
                 const int kp = kp1(d, k);
                 double u[3], B[3];
@@ -502,12 +603,17 @@ __global__ void __launch_bounds__(kThreads) k_ecentre(Dims d, Geo G, Vel<DLT> v,
 
 // eight times E on the edges, from twice E at the centres (kEdgeScale undoes it)
 constexpr double kEdgeScale = 0.125;
-__global__ void __launch_bounds__(kThreads) k_eedges(Dims d, const double* __restrict__ ec, double* __restrict__ er,
+template <bool WHOLE>
+__global__ void __launch_bounds__(kThreads) k_eedges(Dims d, RowMap map, const double* __restrict__ ec, double* __restrict__ er,
                                                      double* __restrict__ et, double* __restrict__ ep) {
     const unsigned int n_r = (unsigned int)(d.nr * (d.nt + 1)), n_t = (unsigned int)((d.nr + 1) * d.nt),
                        n_p = (unsigned int)((d.nr + 1) * (d.nt + 1));
-    const int np = d.np, lane = threadIdx.x & 31;
-    for (unsigned int w = first_row(); w < n_r + n_t + n_p; w += row_stride()) {
+    const int np = d.np;
+    const RowMap M = map.fixed<WHOLE>(d.np);
+    const Lanes L(M);
+    for (unsigned int it = L.first; it < (n_r + n_t + n_p) * M.parts; it += L.stride) {
+        const Part S(M, L, it, np);
+        const unsigned int w = S.row;
         if (w < n_r) {
             const int i = (int)(w / (d.nt + 1)), j = (int)(w - (unsigned int)i * (d.nt + 1));
             double* out = er + (long long)w * np;
@@ -515,13 +621,13 @@ __global__ void __launch_bounds__(kThreads) k_eedges(Dims d, const double* __res
                 // the polar radial edge: the mean of the polar ring
                 const double* row = ec + ix(d, i, j == 0 ? 0 : d.nt - 1, 0);
                 double s = 0.0;
-                for (int k = lane; k < np; k += 32) s += row[k];
-                s = 4.0 * (warp_sum(s) / np);
-                for (int k = lane; k < np; k += 32) out[k] = s;
+                for (int k = L.lane; k < np; k += L.n) s += row[k];
+                s = 4.0 * (L.sum(s) / np);
+                for (int k = S.lo; k < S.hi; k += L.n) out[k] = s;
             } else {
                 const double *b = ec + ix(d, i, j, 0), *a = b - np;
 #pragma unroll 4
-                for (int k = lane; k < np; k += 32) {
+                for (int k = S.lo; k < S.hi; k += L.n) {
                     const int km = km1(d, k);
                     out[k] = (a[km] + a[k]) + (b[km] + b[k]);
                 }
@@ -533,7 +639,7 @@ __global__ void __launch_bounds__(kThreads) k_eedges(Dims d, const double* __res
             // r0: 0 (line-tied); r1: the mean of the two interior cells
             const double *a = ec + d.N + ix(d, i > 0 ? i - 1 : 0, j, 0), *b = ec + d.N + ix(d, i < d.nr ? i : d.nr - 1, j, 0);
 #pragma unroll 4
-            for (int k = lane; k < np; k += 32) {
+            for (int k = S.lo; k < S.hi; k += L.n) {
                 const int km = km1(d, k);
                 out[k] = i == 0 ? 0.0 : (a[km] + a[k]) + (b[km] + b[k]);
             }
@@ -542,18 +648,19 @@ __global__ void __launch_bounds__(kThreads) k_eedges(Dims d, const double* __res
             const int i = (int)(q / (d.nt + 1)), j = (int)(q - (unsigned int)i * (d.nt + 1));
             double* out = ep + (long long)q * np;
             if (j == 0 || j == d.nt || i == 0) {
-                for (int k = lane; k < np; k += 32) out[k] = 0.0;
+                for (int k = S.lo; k < S.hi; k += L.n) out[k] = 0.0;
             } else {
                 const double *a = ec + 2 * d.N + ix(d, i - 1, j, 0), *b = ec + 2 * d.N + ix(d, i < d.nr ? i : d.nr - 1, j, 0);
 #pragma unroll 4
-                for (int k = lane; k < np; k += 32) out[k] = (a[k - np] + a[k]) + (b[k - np] + b[k]);
+                for (int k = S.lo; k < S.hi; k += L.n) out[k] = (a[k - np] + a[k]) + (b[k - np] + b[k]);
             }
         }
     }
 }
 
 // B -= scale dt curl_h of the edge arrays
-__global__ void __launch_bounds__(kThreads) k_ct(Dims d, ExTab X, const double* __restrict__ er,
+template <bool WHOLE>
+__global__ void __launch_bounds__(kThreads) k_ct(Dims d, RowMap map, ExTab X, const double* __restrict__ er,
                                                  const double* __restrict__ et, const double* __restrict__ ep,
                                                  const double* __restrict__ dt_dev, double dt_host, double scale,
                                                  double* __restrict__ br, double* __restrict__ bt,
@@ -561,8 +668,12 @@ __global__ void __launch_bounds__(kThreads) k_ct(Dims d, ExTab X, const double* 
     const double dt = scale * (dt_dev ? *dt_dev : dt_host);
     const unsigned int n_r = (unsigned int)((d.nr + 1) * d.nt), n_t = (unsigned int)(d.nr * (d.nt + 1)),
                        n_p = (unsigned int)(d.nr * d.nt);
-    const int np = d.np, lane = threadIdx.x & 31;
-    for (unsigned int w = first_row(); w < n_r + n_t + n_p; w += row_stride()) {
+    const int np = d.np;
+    const RowMap M = map.fixed<WHOLE>(d.np);
+    const Lanes L(M);
+    for (unsigned int it = L.first; it < (n_r + n_t + n_p) * M.parts; it += L.stride) {
+        const Part S(M, L, it, np);
+        const unsigned int w = S.row;
         if (w < n_r) {
             const int i = (int)(w / d.nt), j = (int)(w - (unsigned int)i * d.nt);
             const double* c = X.fr + 3 * (size_t)w;
@@ -570,7 +681,7 @@ __global__ void __launch_bounds__(kThreads) k_ct(Dims d, ExTab X, const double* 
             const double *t = et + ix(d, i, j, 0), *p0 = ep + ixt(d, i, j, 0), *p1 = p0 + np;
             double* out = br + (long long)w * np;
 #pragma unroll 4
-            for (int k = lane; k < np; k += 32) {
+            for (int k = S.lo; k < S.hi; k += L.n) {
                 const double circ = c0 * (t[k] - t[kp1(d, k)]) + c1 * p1[k] - c2 * p0[k];
                 out[k] -= dt * circ;
             }
@@ -583,7 +694,7 @@ __global__ void __launch_bounds__(kThreads) k_ct(Dims d, ExTab X, const double* 
             const double *r = er + ixt(d, i, j, 0), *p0 = ep + ixt(d, i, j, 0), *p1 = ep + ixt(d, i + 1, j, 0);
             double* out = bt + (long long)q * np;
 #pragma unroll 4
-            for (int k = lane; k < np; k += 32) {
+            for (int k = S.lo; k < S.hi; k += L.n) {
                 const double circ = c0 * p0[k] + c1 * (r[kp1(d, k)] - r[k]) - c2 * p1[k];
                 out[k] -= dt * circ;
             }
@@ -595,7 +706,7 @@ __global__ void __launch_bounds__(kThreads) k_ct(Dims d, ExTab X, const double* 
             const double *r0 = er + ixt(d, i, j, 0), *r1 = r0 + np, *t0 = et + ix(d, i, j, 0), *t1 = et + ix(d, i + 1, j, 0);
             double* out = bp + (long long)q * np;
 #pragma unroll 4
-            for (int k = lane; k < np; k += 32) {
+            for (int k = S.lo; k < S.hi; k += L.n) {
                 const double circ = c0 * (r0[k] - r1[k]) + c1 * t1[k] - c2 * t0[k];
                 out[k] -= dt * circ;
             }
@@ -606,14 +717,15 @@ __global__ void __launch_bounds__(kThreads) k_ct(Dims d, ExTab X, const double* 
 namespace {
 template <bool DLT, bool ETA>
 void ecentre_launch(mhd_grid_s* g, const Vel<DLT>& v, const double* br, const double* bt, const double* bp, double eta) {
-    k_ecentre<DLT, ETA><<<row_blocks<k_ecentre<DLT, ETA>>(g, (long long)g->d.nr * g->d.nt), kThreads, 0, g->stream>>>(
-        g->d, g->geo, v, g->bharm, br, bt, bp, g->er, g->et, g->ep, eta, g->ec);
+    launch_rows<k_ecentre<DLT, ETA, true>, k_ecentre<DLT, ETA, false>>(g, g->stream, (long long)g->d.nr * g->d.nt, kMaxBlocks,
+                                                                       g->geo, v, g->bharm, br, bt, bp, g->er, g->et, g->ep, eta,
+                                                                       g->ec);
 }
 void ct_launch(mhd_grid_s* g, const double* dt_dev, double dt_host, double scale, double* br, double* bt, double* bp) {
     const Dims d = g->d;
     const long long rows = (long long)(d.nr + 1) * d.nt + (long long)d.nr * (d.nt + 1) + (long long)d.nr * d.nt;
-    k_ct<<<row_blocks<k_ct>(g, rows), kThreads, 0, g->stream>>>(d, g->ex, g->er, g->et, g->ep, dt_dev, dt_host, scale, br, bt,
-                                                                bp);
+    launch_rows<k_ct<true>, k_ct<false>>(g, g->stream, rows, kMaxBlocks, g->ex, g->er, g->et, g->ep, dt_dev, dt_host, scale, br,
+                                         bt, bp);
 }
 }  // namespace
 
@@ -631,7 +743,7 @@ void induction(mhd_grid_s* g, const double* vr, const double* vt, const double* 
     else if (eta != 0.0) ecentre_launch<false, true>(g, v, br, bt, bp, eta);
     else ecentre_launch<false, false>(g, v, br, bt, bp, eta);
     const long long rows = (long long)d.nr * (d.nt + 1) + (long long)(d.nr + 1) * d.nt + (long long)(d.nr + 1) * (d.nt + 1);
-    k_eedges<<<row_blocks<k_eedges>(g, rows), kThreads, 0, g->stream>>>(d, g->ec, g->er, g->et, g->ep);
+    launch_rows<k_eedges<true>, k_eedges<false>>(g, g->stream, rows, kMaxBlocks, g->ec, g->er, g->et, g->ep);
     ct_launch(g, dt_dev, dt_host, kEdgeScale, br, bt, bp);
 }
 
@@ -644,7 +756,8 @@ void ct_apply(mhd_grid_s* g, const double* dt_dev, double* br, double* bt, doubl
 // out[0..3] = magnetic energy, kinetic energy, sum |J_c x B_c| V_c, sum |J_c . B_c| V_c; out[4] =
 // max |div_h B| (net outward flux over the cell volume). B_c and J_c as in the momentum force.
 // ------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreads) k_diag(Dims d, Geo G, ExTab X, Vel<false> v, const double* __restrict__ bh,
+template <bool WHOLE>
+__global__ void __launch_bounds__(kThreads) k_diag(Dims d, RowMap map, Geo G, ExTab X, Vel<false> v, const double* __restrict__ bh,
                                                    const double* __restrict__ br, const double* __restrict__ bt,
                                                    const double* __restrict__ bp, const double* __restrict__ jr,
                                                    const double* __restrict__ jt, const double* __restrict__ jp,
@@ -652,7 +765,11 @@ __global__ void __launch_bounds__(kThreads) k_diag(Dims d, Geo G, ExTab X, Vel<f
                                                    double* __restrict__ partials, double* __restrict__ out) {
     double em = 0.0, ek = 0.0, jxb = 0.0, jdb = 0.0, dmax = 0.0;
     const unsigned int rows = (unsigned int)(d.nr * d.nt);
-    for (unsigned int ij = first_row(); ij < rows; ij += row_stride()) {
+    const RowMap M = map.fixed<WHOLE>(d.np);
+    const Lanes L(M);
+    for (unsigned int it = L.first; it < rows * M.parts; it += L.stride) {
+        const Part S(M, L, it, d.np);
+        const unsigned int ij = S.row;
         const int i = (int)(ij / d.nt), j = (int)(ij - (unsigned int)i * d.nt);
         const FaceRow F(d, G, bh, br, bt, bp, i, j);
         const EdgeRow E(d, jr, jt, jp, i, j);
@@ -667,7 +784,7 @@ __global__ void __launch_bounds__(kThreads) k_diag(Dims d, Geo G, ExTab X, Vel<f
         long long mf = 0;
         F.over([&](auto polar) {
 #pragma unroll 1
-            for (int k = threadIdx.x & 31; k < d.np; k += 32) {
+            for (int k = S.lo; k < S.hi; k += L.n) {
                 const int kp = kp1(d, k);
                 double u[3], B[3], J[3];
                 v.at((long long)ij * d.np + k, u);
@@ -702,9 +819,9 @@ void diagnostics(mhd_grid_s* g, const double* vr, const double* vt, const double
     current_and_harmonics(g, br, bt, bp, g->bharm, g->stream);
     const Vel<false> v{vr, vt, vp, nullptr, 0.0, d.N};
     // two reductions: 5 partials a CTA in the array's 4 kMaxBlocks, and a ticket each (the solver's is idle here)
-    const int blocks = std::min(row_blocks<k_diag>(g, (long long)d.nr * d.nt), kMaxBlocks * kPartialsPerBlock / 5);
-    k_diag<<<blocks, kThreads, 0, g->stream>>>(d, g->geo, g->ex, v, g->bharm, br, bt, bp, g->er, g->et, g->ep,
-                                               &g->ss->count, &g->sc->count, g->partials, out);
+    launch_rows<k_diag<true>, k_diag<false>>(g, g->stream, (long long)d.nr * d.nt, kMaxBlocks * kPartialsPerBlock / 5, g->geo, g->ex, v,
+                                             g->bharm, br, bt, bp, g->er, g->et, g->ep, &g->ss->count, &g->sc->count, g->partials,
+                                             out);
 }
 
 // ------------------------------------------------------------------------------------------

@@ -19,6 +19,7 @@
 // thread, then FP64), CTAs reduce with warp shuffles, write one partial each, and the last CTA
 // to arrive sums the partials in CTA order and finishes the scalar recurrence (alpha, beta,
 // stop test). Results are deterministic for a fixed launch shape.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -1171,20 +1172,22 @@ __global__ void k_correct(Dims d, int nc, double* __restrict__ x, const float* _
     if (blockIdx.x == 0 && threadIdx.x == 0) sc->outer += 1;
 }
 
-// q = M_alpha p (unscaled FP64), for the C-ABI operator call, in one launch: a CTA takes kApplyRows rows (i, j), its
-// first threads form their coefficients (as k_tables does), and its warps take (row, component) items. Forming all
-// tables first, and alpha on the device before that, made three dependent launches of what is 2.4 us of FP64
-// instructions at 32x32x64, 3 components: 16.4 -> 8.2 us a call.
-constexpr int kApplyRows = 8;
-__global__ void __launch_bounds__(kThreads) k_apply64(Dims d, Geo G, double a, int nc, const double* __restrict__ p,
-                                                      double* __restrict__ q) {
+// q = M_alpha p (unscaled FP64), for the C-ABI operator call, in one launch: a CTA takes a range of phi pairs, its
+// threads first form the coefficients of the rows (i, j) in it (as k_tables does), then each takes pairs, whatever
+// the length of a row, and does them for every component. Forming all tables first, and alpha on the device before
+// that, made three dependent launches of what is 2.4 us of FP64 instructions at 32x32x64, 3 components: 16.4 -> 8.2 us
+// a call.
+constexpr int kApplyRows = kThreads + 2;   // most rows that a range touches (apply_operator)
+__global__ void __launch_bounds__(kThreads) k_apply64(Dims d, Geo G, double a, int nc, unsigned int range,
+                                                      const double* __restrict__ p, double* __restrict__ q) {
     __shared__ double co[kApplyRows][6];
     const int nt = d.nt;
-    const int row0 = blockIdx.x * kApplyRows, n = min(kApplyRows, d.nr * nt - row0);
+    const unsigned int npv = d.np / 2, g0 = blockIdx.x * range, g1 = min(g0 + range, (unsigned int)(d.N / 2));
+    const int row0 = (int)(g0 / npv), n = (int)((g1 - 1) / npv) - row0 + 1;
     const long long plane = (long long)nt * d.np;
-    if ((int)threadIdx.x < n) {
-        const int ij = row0 + threadIdx.x, i = ij / nt, j = ij - i * nt;
-        double* c = co[threadIdx.x];
+    for (int t = threadIdx.x; t < n; t += kThreads) {
+        const int ij = row0 + t, i = ij / nt, j = ij - i * nt;
+        double* c = co[t];
         c[0] = diag_at(G, nt, a, i, j);
         c[1] = a * G.wr[i * nt + j];
         c[2] = a * G.wr[(i + 1) * nt + j];
@@ -1193,23 +1196,22 @@ __global__ void __launch_bounds__(kThreads) k_apply64(Dims d, Geo G, double a, i
         c[5] = a * G.wp[ij];
     }
     __syncthreads();
-    for (int item = threadIdx.x >> 5; item < n * nc; item += kThreads / 32) {
-        const int k = item / n, rl = item - k * n, ij = row0 + rl, i = ij / nt, j = ij - i * nt;
-        const double dg = co[rl][0], wl = co[rl][1], wh = co[rl][2], tl = co[rl][3], th = co[rl][4], wp = co[rl][5];
-        const long long row = k * d.N + (long long)ij * d.np;
-        const double* u = p + row;
-        for (int k0 = 2 * (threadIdx.x & 31); k0 < d.np; k0 += 64) {
+    for (unsigned int g = g0 + threadIdx.x; g < g1; g += kThreads) {
+        const Cell c = decompose<2>(d, g);
+        const double* w = co[(int)c.ij - row0];
+        const double dg = w[0], wl = w[1], wh = w[2], tl = w[3], th = w[4], wp = w[5];
+        const int km = ((c.k0 == 0) ? d.np : c.k0) - 1 - c.k0, kp = (c.k0 + 2 == d.np) ? -c.k0 : 2;
+        for (int k = 0; k < nc; k++) {
+            const double* u = p + k * d.N + c.base;
             double xv[2], n2[2], mx[2];
-            ldv<double, 2>(u + k0, xv);
-            const int km = (k0 == 0) ? d.np - 1 : k0 - 1;
-            const int kp = (k0 + 2 == d.np) ? 0 : k0 + 2;
+            ldv<double, 2>(u, xv);
             mx[0] = dg * xv[0] - wp * (u[km] + xv[1]);
             mx[1] = dg * xv[1] - wp * (xv[0] + u[kp]);
-            if (i > 0) { ldv<double, 2>(u + k0 - plane, n2); mx[0] -= wl * n2[0]; mx[1] -= wl * n2[1]; }
-            if (i < d.nr - 1) { ldv<double, 2>(u + k0 + plane, n2); mx[0] -= wh * n2[0]; mx[1] -= wh * n2[1]; }
-            if (j > 0) { ldv<double, 2>(u + k0 - d.np, n2); mx[0] -= tl * n2[0]; mx[1] -= tl * n2[1]; }
-            if (j < nt - 1) { ldv<double, 2>(u + k0 + d.np, n2); mx[0] -= th * n2[0]; mx[1] -= th * n2[1]; }
-            stv<double, 2>(q + row + k0, mx);
+            if (c.i > 0) { ldv<double, 2>(u - plane, n2); mx[0] -= wl * n2[0]; mx[1] -= wl * n2[1]; }
+            if (c.i < d.nr - 1) { ldv<double, 2>(u + plane, n2); mx[0] -= wh * n2[0]; mx[1] -= wh * n2[1]; }
+            if (c.j > 0) { ldv<double, 2>(u - d.np, n2); mx[0] -= tl * n2[0]; mx[1] -= tl * n2[1]; }
+            if (c.j < nt - 1) { ldv<double, 2>(u + d.np, n2); mx[0] -= th * n2[0]; mx[1] -= th * n2[1]; }
+            stv<double, 2>(q + k * d.N + c.base, mx);
         }
     }
 }
@@ -1224,8 +1226,12 @@ void build_tables(mhd_grid_s* g, const double* alpha_dev, bool fp32) {
 }
 
 void apply_operator(mhd_grid_s* g, double alpha, int nc, const double* p, double* q) {
-    const int rows = g->d.nr * g->d.nt;
-    k_apply64<<<(rows + kApplyRows - 1) / kApplyRows, kThreads, 0, g->stream>>>(g->d, g->geo, alpha, nc, p, q);
+    // ranges of up to 6 pairs a thread, fewer where that leaves less than 8 CTAs per SM (us at 61x47x118, 160x160x320 and
+    // 256x256x512, 3 components: 1 pair 25.5, 317, 1259; 2 27.2, 310, 1229; 6 29.0, 314, 1216; 8 35.5, 324, 1214; with 8 rows a
+    // CTA 35.6, 318, 1211); no more pairs a thread than a row has, so that a range touches at most kApplyRows rows
+    const unsigned int pairs = (unsigned int)(g->d.N / 2), room = 8u * g->num_sms * kThreads;
+    const unsigned int m = std::max(1u, std::min({6u, (unsigned int)g->d.np / 2, pairs / room}));
+    k_apply64<<<(pairs + m * kThreads - 1) / (m * kThreads), kThreads, 0, g->stream>>>(g->d, g->geo, alpha, nc, m * kThreads, p, q);
 }
 
 namespace {
