@@ -22,7 +22,7 @@
 // at 152 registers; issue slots half used, 5.3 TB/s of HBM by the 60 B a cell). Other shapes at 192x192x384: one row a thread 242
 // (bound by instructions and shared-memory wavefronts), 2 rows 164 to 175, 4 rows 167 to 187, 5 rows 217.
 //
-// The sums are FP32 over the thread's 12 cells of a plane and compensated beyond; the weights dg of the stop norm
+// The sums are FP32 over the thread's 12 cells of a plane (<r', q>: 24 of two) and compensated beyond; the weights dg of the stop norm
 // have 48 bits and each product's rounding is kept, as FP64 at this rate would take longer than all the rest (with
 // dg and the products rounded to FP32 an iteration at 256x256x512 took 0.9% less).
 //
@@ -82,12 +82,18 @@ __device__ __forceinline__ float4 stencil4(float4 u, float left, float right, fl
     return fma4(-c0.w, jp, o);
 }
 
-// compensated FP32 sum (two-sum) of x, or of x and a part of it below its rounding
+// compensated FP32 sum (two-sum)
 struct Sum2 {
     float s = 0.f, c = 0.f;
-    __device__ __forceinline__ void add(float x, float low = 0.f) {
+    __device__ __forceinline__ void add(float x) {
         const float t = s + x, b = t - s;
-        c += ((s - (t - b)) + (x - b)) + low;
+        c += (s - (t - b)) + (x - b);
+        s = t;
+    }
+    // of a product g (hi + lo): its rounding and the low part go to the correction
+    __device__ __forceinline__ void add_product(float g, float hi, float lo) {
+        const float x = g * hi, t = s + x, b = t - s;
+        c += fmaf(g, lo, fmaf(g, hi, -x)) + ((s - (t - b)) + (x - b));
         s = t;
     }
     __device__ __forceinline__ double get() const { return (double)s + (double)c; }
@@ -178,9 +184,10 @@ __global__ void __launch_bounds__(kMT, kCtas) k_march32(Dims d, Tiling T, float*
         const int tu = tr > 0 ? tr - 1 : 0, td = tr < kTR - 1 ? tr + 1 : tr;   // thread rows above and below
         fetch(0, 0);
         for (int n0 = 0; n0 < steps; n0 += 2) {
+            float pw = 0.f;   // plain over the thread's 24 cells of two planes, then compensated
 #pragma unroll
             for (int t = 0; t < 2; t++) {
-                float pg = 0.f, pw = 0.f, pd = 0.f;   // plain over the thread's 12 cells of a plane, then compensated
+                float pg = 0.f, pd = 0.f;   // over the 12 of one
                 const int n = n0 + t;
                 fetch(n + 1, t ^ 1);
                 copy_wait<1>();
@@ -220,8 +227,7 @@ __global__ void __launch_bounds__(kMT, kCtas) k_march32(Dims d, Tiling T, float*
                             const float gg = fmaf(r1[a].x, r1[a].x, fmaf(r1[a].y, r1[a].y, fmaf(r1[a].z, r1[a].z, r1[a].w * r1[a].w)));
                             pg += gg;
                             // the stop norm's weight has 48 bits: the product is exact but for the low part's rounding
-                            const float wg = gg * c1.y;
-                            s_rr.add(wg, fmaf(gg, c1.z, fmaf(gg, c1.y, -wg)));
+                            s_rr.add_product(gg, c1.y, c1.z);
                             pw = fmaf(r1[a].x, q.x, fmaf(r1[a].y, q.y, fmaf(r1[a].z, q.z, fmaf(r1[a].w, q.w, pw))));
                         }
                     }
@@ -252,10 +258,10 @@ __global__ void __launch_bounds__(kMT, kCtas) k_march32(Dims d, Tiling T, float*
                     rk[a] = in[((t * 3 + 0) * kRT + a) * kMT];
                 }
                 s_g.add(pg);
-                s_w.add(pw);
                 s_d.add(pd);
                 __syncthreads();
             }
+            s_w.add(pw);
         }
     }
     copy_wait<0>();
