@@ -33,7 +33,9 @@
  *    enqueueing.
  *  - Status codes only: nothing throws or aborts across the ABI. After an error,
  *    mhd_last_error(grid) describes it. On MHD_ERR_NOCONV the best iterate is left in x.
- *  - One grid per stream; a grid is not thread-safe.
+ *  - One grid per stream; a grid is not thread-safe. Point-Jacobi solves of small grids are one launch that
+ *    takes the whole GPU (see mhd_params_t): on several streams they run one after another. For many
+ *    systems at once there is pcg_solve_batched.
  *  - np must be even (double2 loads along phi); nt >= 2, nr >= 2.
  */
 #ifndef MHD_H

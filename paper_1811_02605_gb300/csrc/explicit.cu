@@ -160,8 +160,7 @@ struct Vel {
 // over more rows); below that the number with the least estimated time, which is the items that the busiest
 // SM gets, a CTA's worth at a time, times the passes of an item, with a factor for the spread. Times in us, coefficients + force +
 // induction without and with resistivity + diagnostics, with 32 lanes and one part for every row / by this rule:
-// 256x256x8 1364 / 460, 300x200x34 2196 / 1310, 100x100x48 529 / 426, 61x47x118 401 / 357, 16x16x4096 2010 / 829,
-// 4x4x8192 3430 / 435.
+// 256x256x8 1332 / 477, 300x200x34 2293 / 1306, 100x100x48 530 / 423, 16x16x4096 2010 / 828, 4x4x8192 3433 / 435.
 struct RowLaunch {
     RowMap m;
     int blocks;
