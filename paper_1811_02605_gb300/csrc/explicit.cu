@@ -160,7 +160,7 @@ struct Vel {
 // over more rows); below that the number with the least estimated time, which is the items that the busiest
 // SM gets, a CTA's worth at a time, times the passes of an item, with a factor for the spread. Times in us, coefficients + force +
 // induction without and with resistivity + diagnostics, with 32 lanes and one part for every row / by this rule:
-// 256x256x8 1332 / 477, 300x200x34 2293 / 1306, 100x100x48 530 / 423, 16x16x4096 2010 / 828, 4x4x8192 3433 / 435.
+// 256x256x8 1332 / 477, 300x200x34 2293 / 1306, 100x100x48 530 / 423, 16x16x4096 2010 / 806, 4x4x8192 3433 / 301.
 struct RowLaunch {
     RowMap m;
     int blocks;
@@ -321,6 +321,26 @@ __global__ void k_ring_harm(Dims d, const double* __restrict__ a, long long stri
     }
 }
 
+// polar ring sums of a cell-centred array, one CTA per ring: out[i] (north), out[nr + i] (south). done (may be null):
+// a solve's flag
+__global__ void __launch_bounds__(kThreads) k_ring_sum(Dims d, const double* __restrict__ a, double* __restrict__ out,
+                                                       const int* __restrict__ done) {
+    if (done && *done) return;
+    const int i = blockIdx.x % d.nr, south = blockIdx.x / d.nr;
+    const double* row = a + ix(d, i, south ? d.nt - 1 : 0, 0);
+    double s = 0.0;
+    for (int k = threadIdx.x; k < d.np; k += kThreads) s += row[k];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    __shared__ double sm[kThreads / 32];
+    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        s = sm[0];
+        for (int w = 1; w < kThreads / 32; w++) s += sm[w];
+        out[blockIdx.x] = s;
+    }
+}
+
 void ring_harmonics(mhd_grid_s* g, const double* a, long long stride_i, long long off_n, long long off_s,
                     double* out, cudaStream_t st) {
     k_ring_harm<<<2 * g->d.nr, kThreads, 0, st ? st : g->stream>>>(g->d, a, stride_i, off_n, off_s, g->geo.pcs,
@@ -336,7 +356,7 @@ void bt_harmonics(mhd_grid_s* g, const double* bt, cudaStream_t st) {
 // current density on edges
 // ------------------------------------------------------------------------------------------
 // J on all edges in one launch, a group of lanes per row; a polar radial row takes its ring's sum of B_phi itself (the cap
-// circulation), and with bh the warps of the first 2 nr rows form the harmonics of the B_theta rings beside the
+// circulation) unless it comes in ring, and with bh the warps of the first 2 nr rows form the harmonics of the B_theta rings beside the
 // poles. walls_zero: the resistive operator's current, 0 on the tangential edges of r0 and r1. done (may be null):
 // a solve's flag, nothing is formed once it is set.
 template <bool WHOLE>
@@ -346,7 +366,8 @@ __global__ void __launch_bounds__(kThreads) k_current(Dims d, RowMap map, const 
                                                       const double* __restrict__ bp, double* __restrict__ jr,
                                                       double* __restrict__ jt, double* __restrict__ jp,
                                                       const double* __restrict__ pcs, double* __restrict__ bh,
-                                                      int walls_zero, const int* __restrict__ done) {
+                                                      int walls_zero, const int* __restrict__ done,
+                                                      const double* __restrict__ ring) {
     if (done && *done) return;
     const unsigned int n_h = bh ? 2u * d.nr : 0u, n_r = (unsigned int)(d.nr * (d.nt + 1)),
                        n_t = (unsigned int)((d.nr + 1) * d.nt), n_p = (unsigned int)((d.nr + 1) * (d.nt + 1));
@@ -379,8 +400,13 @@ __global__ void __launch_bounds__(kThreads) k_current(Dims d, RowMap map, const 
             if (j == 0 || j == d.nt) {
                 const double* row = bp + ix(d, i, j == 0 ? 0 : d.nt - 1, 0);
                 double s = 0.0;
-                for (int k = L.lane; k < np; k += L.n) s += row[k];
-                s = L.sum(s) * (j == 0 ? c[3] : -c[3]);   // cap circulation / cap area
+                if (!WHOLE && ring) {
+                    s = ring[j == 0 ? i : d.nr + i];
+                } else {
+                    for (int k = L.lane; k < np; k += L.n) s += row[k];
+                    s = L.sum(s);
+                }
+                s *= j == 0 ? c[3] : -c[3];   // cap circulation / cap area
                 for (int k = S.lo; k < S.hi; k += L.n) out[k] = s;
             } else {
                 const double c0 = c[0], c1 = c[1], c2 = c[2];
@@ -421,13 +447,31 @@ __global__ void __launch_bounds__(kThreads) k_current(Dims d, RowMap map, const 
 
 namespace {
 
+// Rows cut into parts, and long: every part of a polar radial row would take its ring's sum itself, a chain of np / 32
+// additions, so the sums and the harmonics are launches of their own, a CTA per ring (us of an induction with
+// resistivity, without / with: 4x4x8192 122 / 70, 16x16x4096 194 / 187).
+bool rings_apart(const mhd_grid_s* g) {
+    return g->d.np >= 2048 && row_launch(g, (long long)g->d.nr * g->d.nt, 2).m.parts > 1;
+}
+// the ring sums of a cell-centred array where they are launched apart, else null
+const double* ring_sums(mhd_grid_s* g, const double* a, const int* done, cudaStream_t st) {
+    if (!rings_apart(g)) return nullptr;
+    k_ring_sum<<<2 * g->d.nr, kThreads, 0, st>>>(g->d, a, g->ring, done);
+    return g->ring;
+}
+
 void edge_current(mhd_grid_s* g, const double* cr, const double* ct, const double* cp, const double* br, const double* bt,
                   const double* bp, double* bh, bool walls_zero, const int* done, cudaStream_t st) {
     const Dims d = g->d;
+    const double* ring = ring_sums(g, bp, done, st);
+    if (ring && bh) {
+        bt_harmonics(g, bt, st);
+        bh = nullptr;
+    }
     const long long rows = (bh ? 2ll * d.nr : 0ll) + (long long)d.nr * (d.nt + 1) + (long long)(d.nr + 1) * d.nt +
                            (long long)(d.nr + 1) * (d.nt + 1);
     launch_rows<k_current<true>, k_current<false>>(g, st, rows, kMaxBlocks, cr, ct, cp, br, bt, bp, g->er, g->et, g->ep,
-                                                   g->geo.pcs, bh, walls_zero ? 1 : 0, done);
+                                                   g->geo.pcs, bh, walls_zero ? 1 : 0, done, ring);
 }
 
 void current_and_harmonics(mhd_grid_s* g, const double* br, const double* bt, const double* bp, double* bh, cudaStream_t st) {
@@ -604,7 +648,8 @@ __global__ void __launch_bounds__(kThreads) k_ecentre(Dims d, RowMap map, Geo G,
 constexpr double kEdgeScale = 0.125;
 template <bool WHOLE>
 __global__ void __launch_bounds__(kThreads) k_eedges(Dims d, RowMap map, const double* __restrict__ ec, double* __restrict__ er,
-                                                     double* __restrict__ et, double* __restrict__ ep) {
+                                                     double* __restrict__ et, double* __restrict__ ep,
+                                                     const double* __restrict__ ring) {
     const unsigned int n_r = (unsigned int)(d.nr * (d.nt + 1)), n_t = (unsigned int)((d.nr + 1) * d.nt),
                        n_p = (unsigned int)((d.nr + 1) * (d.nt + 1));
     const int np = d.np;
@@ -620,8 +665,13 @@ __global__ void __launch_bounds__(kThreads) k_eedges(Dims d, RowMap map, const d
                 // the polar radial edge: the mean of the polar ring
                 const double* row = ec + ix(d, i, j == 0 ? 0 : d.nt - 1, 0);
                 double s = 0.0;
-                for (int k = L.lane; k < np; k += L.n) s += row[k];
-                s = 4.0 * (L.sum(s) / np);
+                if (!WHOLE && ring) {
+                    s = ring[j == 0 ? i : d.nr + i];
+                } else {
+                    for (int k = L.lane; k < np; k += L.n) s += row[k];
+                    s = L.sum(s);
+                }
+                s = 4.0 * (s / np);
                 for (int k = S.lo; k < S.hi; k += L.n) out[k] = s;
             } else {
                 const double *b = ec + ix(d, i, j, 0), *a = b - np;
@@ -742,7 +792,8 @@ void induction(mhd_grid_s* g, const double* vr, const double* vt, const double* 
     else if (eta != 0.0) ecentre_launch<false, true>(g, v, br, bt, bp, eta);
     else ecentre_launch<false, false>(g, v, br, bt, bp, eta);
     const long long rows = (long long)d.nr * (d.nt + 1) + (long long)(d.nr + 1) * d.nt + (long long)(d.nr + 1) * (d.nt + 1);
-    launch_rows<k_eedges<true>, k_eedges<false>>(g, g->stream, rows, kMaxBlocks, g->ec, g->er, g->et, g->ep);
+    const double* ring = ring_sums(g, g->ec, nullptr, g->stream);
+    launch_rows<k_eedges<true>, k_eedges<false>>(g, g->stream, rows, kMaxBlocks, g->ec, g->er, g->et, g->ep, ring);
     ct_launch(g, dt_dev, dt_host, kEdgeScale, br, bt, bp);
 }
 

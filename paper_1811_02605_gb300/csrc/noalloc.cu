@@ -6,7 +6,7 @@
 // allowed, and plug-in code run under an allocator policy that forbids new device allocations.
 // mhd_grid_create allocates the grid's tables and workspace, so those callers cannot use
 // mhd_force; this entry point takes the grid description instead and keeps all its scratch
-// (metric tables, current density on edges, polar harmonics) in one file-scope
+// (metric tables, current density on edges, polar ring sums and harmonics) in one file-scope
 // device array.
 //
 // The scratch array is static device memory: every GPU that loads the library holds it until
@@ -22,7 +22,7 @@
 
 namespace {
 
-// 10 MiB of FP64 scratch: tables plus the three edge arrays of J.
+// 10 MiB of FP64 scratch: tables plus the three edge arrays of J plus the ring sums.
 constexpr long long kScratchDoubles = 1310720;
 constexpr long long kMaxCells = 262144;  // e.g. 64 x 64 x 64
 constexpr int kMaxDevices = 64;
@@ -124,8 +124,7 @@ extern "C" mhd_status_t mhd_force_noalloc(const mhd_grid_desc_t* desc, const mhd
     const long long N = (long long)d.nr * d.nt * d.np;
     const long long nr = d.nr, nt = d.nt, np = d.np;
     // scratch layout (doubles): r, rc, sn, cn, sc, cc, rho, rhoV, the explicit tables (shell, 1/(r sin
-    // dph), cot, edge rows), jr, jt, jp, cos / sin of the phi centres, polar B_theta harmonics; 2 nr more
-    // are counted than used, so that the largest grids accepted stay what they were
+    // dph), cot, edge rows), jr, jt, jp, ring sums, cos / sin of the phi centres, polar B_theta harmonics
     const long long n_ex = 5 * nr + nr * nt + nt + 4 * nr * (nt + 1) + 3 * (nr + 1) * nt + 3 * (nr + 1) * (nt + 1);
     const long long n_tab = (nr + 1) + nr + 2 * (nt + 1) + 2 * nt + nr + nr * nt + n_ex;
     const long long n_edge = nr * (nt + 1) * np + (nr + 1) * nt * np + (nr + 1) * (nt + 1) * np;
@@ -158,6 +157,7 @@ extern "C" mhd_status_t mhd_force_noalloc(const mhd_grid_desc_t* desc, const mhd
     double* jr = take(nr * (nt + 1) * np);
     double* jt = take((nr + 1) * nt * np);
     double* jp = take((nr + 1) * (nt + 1) * np);
+    double* ring = take(2 * nr);
     double* pcs = take(2 * np);
     double* bharm = take(4 * nr);   // north and south B_theta rings; the adjoint half is not used here
     if (off > kScratchDoubles) return MHD_ERR_ARG;
@@ -217,6 +217,7 @@ extern "C" mhd_status_t mhd_force_noalloc(const mhd_grid_desc_t* desc, const mhd
     v.er = jr;
     v.et = jt;
     v.ep = jp;
+    v.ring = ring;
     v.bharm = bharm;
 
     k_noalloc_radial<<<1, 1, 0, v.stream>>>(d.nr, d.r0, d.r1, d.stretch, r);
